@@ -733,6 +733,11 @@ int pool_run(gesmc_pool_t p, uint64_t rounds) {
       }
       std::vector<uint32_t> jobs;
       for (uint32_t k = 0; k < kResidentClasses; ++k) {
+        // longest first: a class with more chains than its CTAs have room for
+        // ends with its shortest ones
+        std::stable_sort(by_class[k].begin(), by_class[k].end(), [p](uint32_t x, uint32_t y) {
+          return p->chains[x].shape.m > p->chains[y].shape.m;
+        });
         jobs.insert(jobs.end(), by_class[k].begin(), by_class[k].end());
         p->res_count[k] = (uint32_t)by_class[k].size();
       }

@@ -80,6 +80,14 @@ __device__ __forceinline__ uint32_t tau_g(uint32_t g, unsigned long long e1, uns
   return 0;
 }
 
+// ---------------------------------------------------------------- dependent launches
+// Programmatic dependent launch: let the next kernel of the stream start
+// (once every CTA of this one has called this or exited), and wait for the
+// kernel before this one to end with its writes visible.  Both do nothing in
+// a kernel launched without the attribute.
+__device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ---------------------------------------------------------------- bulk copies
 // One-dimensional bulk copy (the TMA engine, cp.async.bulk) of `bytes` from
 // global memory into this CTA's shared memory, completing on an mbarrier.

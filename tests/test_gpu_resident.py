@@ -246,3 +246,44 @@ def test_many_chains_with_exact_laziness_sorted_in_their_own_ctas():
     for t in range(0, len(graphs), 5):
         want, _ = oracle.run(graphs[t][0], seed=90 + t, rounds=6, lazy_threshold=thr, exact_ell=True)
         assert np.array_equal(outs[t], want), t
+
+
+@pytest.mark.parametrize("m", [2, 3, 5, 64, 65, 512, 1024, 1025, 2048, 2049, 4096, 4097, 8192, 8193, 10240])
+@pytest.mark.parametrize("dense", [False, True])
+def test_edges_of_the_size_classes(m, dense):
+    # sizes where the CTA, the bitmaps, the bucket scan and the table change
+    # shape; few nodes make most targets edges of the graph, so that the table
+    # of candidates outgrows the lists' bytes, many leave it nearly empty
+    n = next(v for v in range(3, 70000) if v * (v - 1) // 2 >= m + m // 8 + 1) if dense else 4 * m + 8
+    edges = inputs.random_simple_graph(n, m, seed=m)
+    with gesmc.Chain(edges, n=n) as c:
+        c.set_round_launch(RESIDENT)
+        c.run(4, 5)
+        got, st = c.edges(), c.stats()
+    want, want_st = oracle.run(edges, seed=5, rounds=4)
+    assert np.array_equal(got, want)
+    for k in ("accepted", "rejected_loop", "rejected_exists", "lazy"):
+        assert st[k] == want_st[k], k
+
+
+def test_keys_that_agree_in_the_bits_the_sort_compares():
+    # seed 7, round 994747: the keys of two positions below 10240 agree in
+    # their top 46 bits, the bucket's 14 and the 32 compared in it, so that
+    # the round's ranks are taken again from the full keys
+    import numpy.random as npr
+    edges = inputs.random_simple_graph(30000, gesmc.RESIDENT_MAX_EDGES, seed=3)
+    gen = npr.Philox(key=[7, 0], counter=[0, 994747, 0, 0])
+    gen.advance(-1)  # numpy steps the counter before each block
+    top = np.sort(gen.random_raw(gesmc.RESIDENT_MAX_EDGES) >> np.uint64(18))
+    assert (top[1:] == top[:-1]).any()
+    want = oracle.run(edges, seed=7, rounds=2, start_round=994746)[0]
+    with gesmc.Chain(edges, n=30000, start_round=994746) as c:  # sorted ahead
+        c.set_round_launch(RESIDENT)
+        assert np.array_equal(c.run(2, 7).edges(), want)
+    few = inputs.random_simple_graph(20, 30, seed=1)
+    with gesmc.Pool(max_edges=len(edges) + 60 * 30, max_chains=61) as pool:  # sorted in its own CTA
+        big = pool.add(edges, n=30000, seed=7, start_round=994746)
+        for t in range(60):
+            pool.add(few, n=20, seed=t)
+        pool.set_round_launch(RESIDENT)
+        assert np.array_equal(pool.run(2).edges(big), want)
