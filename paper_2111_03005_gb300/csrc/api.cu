@@ -154,7 +154,7 @@ Layout pool_layout(const Capacity &c, uint64_t M, uint64_t C) {
   l.list0 = take(4 * c.switches);
   l.list1 = take(4 * c.switches);
   l.ptup = take(16 * c.tuples);
-  l.otup = take(16 * c.ovf);
+  l.otup = take(std::max<uint64_t>(16 * c.ovf, 4096));  // at least a few hundred samples of ParES
   l.tcount = take(4 * c.tcounts);
   l.ocount = take(4 * c.parts);
   l.ooff = take(4 * (c.parts + 1));
@@ -944,21 +944,20 @@ int pool_es_run(gesmc_pool_t p, uint64_t switches, uint32_t only) {
     jb.m = hc.d.m;
     jb.seed = hc.d.seed;
     jb.k0 = hc.es_next;
-    jb.count = switches;
     jb.chain = c;
     if (jb.m >= 2) {
-      // the list (position order) in the chain's tuple storage (at least 32
-      // bytes per edge), the edge set in its permutation records (at least
+      // the list (position order, 16 bytes per edge) in the chain's tuple
+      // storage (at least 32 bytes per edge), the edge set in its permutation records (at least
       // 32 bytes per edge: 2^h >= 2m slots)
       char *base = tup + 16ull * hc.d.tuple_base;
       const uint64_t bytes = 16ull * hc.d.capt << hc.d.P;
-      if (8ull * jb.m > bytes) return GESMC_E_INTERNAL;
+      if (16ull * jb.m > bytes) return GESMC_E_INTERNAL;
       char *hbase = reinterpret_cast<char *>(a.prec) + (16ull << p->cap.bucket_log2) * hc.d.bucket_base;
       const uint64_t hbytes = (16ull << p->cap.bucket_log2) * hc.shape.nb;
       uint32_t hlog2 = 0;
       while ((16ull << hlog2) <= hbytes && hlog2 < 31) ++hlog2;  // largest 2^h with 8 * 2^h <= room
       if ((1ull << hlog2) < 2ull * jb.m) return GESMC_E_INTERNAL;
-      jb.E = reinterpret_cast<unsigned long long *>(base);
+      jb.E = reinterpret_cast<uint4 *>(base);
       jb.H = reinterpret_cast<unsigned long long *>(hbase);
       jb.hlog2 = hlog2;
     }
@@ -970,9 +969,12 @@ int pool_es_run(gesmc_pool_t p, uint64_t switches, uint32_t only) {
   // counted)
   std::stable_sort(jobs.begin(), jobs.end(),
                    [](const EsJob &x, const EsJob &y) { return es_window(x.m) > es_window(y.m); });
-  uint32_t group[4] = {0, 0, 0, 0};
+  uint32_t group[4] = {0, 0, 0, 0}, rows = 0;
   for (uint32_t t = 0; t < jobs.size(); ++t) {
-    if (jobs[t].m >= 2) job_of[jobs[t].chain] = t;
+    if (jobs[t].m >= 2) {
+      job_of[jobs[t].chain] = t;
+      jobs[t].row = rows++;
+    }
     const uint32_t w = es_window(jobs[t].m);
     ++group[w == 1024u ? 0 : w == 256u ? 1 : w == 128u ? 2 : 3];
   }
@@ -987,26 +989,40 @@ int pool_es_run(gesmc_pool_t p, uint64_t switches, uint32_t only) {
   const uint64_t set_launches = 2ull * ((nj + 65534) / 65535);
   ok &= launch_es_set(djobs, nj, err, s, p->num_sms, false) == cudaSuccess;
   p->launches += set_launches + 2;
-  // chains of the largest window stop when their edge set needs a rebuild;
-  // rebuild those sets on the whole GPU and launch them again until every
-  // job is done (each launch advances every stopped job by a superstep at
-  // least)
+  // The switches run in batches, sampled beforehand into the overflow-tuple
+  // array (free between rounds): 8 bytes and a 16-bit distance per switch and
+  // chain.  It has 32 bytes for every edge, so a batch has at least 6 switches
+  // of each chain, and three for every edge of the largest.
+  uint2 *samples = reinterpret_cast<uint2 *>(a.otup);
+  const uint64_t room = p->lay.tcount - p->lay.otup;
+  const uint64_t batch = std::min<uint64_t>(1u << 30, rows ? room / (10ull * rows) : switches);
   uint32_t *nstop = &a.ctl->es_stopped;
-  for (uint64_t iter = 0; ok; ++iter) {
+  for (uint64_t off = 0; ok && off < switches; off += batch) {
+    const uint32_t n = (uint32_t)std::min<uint64_t>(batch, switches - off);
+    uint16_t *dists = reinterpret_cast<uint16_t *>(samples + (uint64_t)rows * n);
     uint32_t run_launches = 0;
-    const uint32_t groups[4] = {group[0], iter ? 0u : group[1], iter ? 0u : group[2], iter ? 0u : group[3]};
-    if (group[0]) ok &= cudaMemsetAsync(nstop, 0, sizeof(uint32_t), s) == cudaSuccess;
-    ok &= launch_es_run(djobs, groups, a.st, a.chain_accepted, err, nstop, s, p->gstream, p->ev_in, p->ev_out,
-                        &run_launches) == cudaSuccess;
+    ok &= launch_es_sample(djobs, group, off, n, samples, dists, s, &run_launches) == cudaSuccess;
     p->launches += run_launches;
-    if (!ok || group[0] == 0) break;  // only the largest windows stop
-    uint32_t stopped = 0, e = 0;
-    ok &= cudaMemcpyAsync(&stopped, nstop, sizeof(uint32_t), cudaMemcpyDeviceToHost, s) == cudaSuccess;
-    ok &= cudaMemcpyAsync(&e, err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s) == cudaSuccess;
-    ok &= cudaStreamSynchronize(s) == cudaSuccess;
-    if (!ok || stopped == 0 || e != 0) break;
-    ok &= launch_es_set(djobs, nj, err, s, p->num_sms, true) == cudaSuccess;
-    p->launches += set_launches;
+    // chains of the largest window stop when their edge set needs a rebuild;
+    // rebuild those sets on the whole GPU and launch them again until every
+    // job is done (each launch advances every stopped job by a superstep at
+    // least)
+    for (uint64_t iter = 0; ok; ++iter) {
+      const uint32_t groups[4] = {group[0], iter ? 0u : group[1], iter ? 0u : group[2], iter ? 0u : group[3]};
+      if (group[0]) ok &= cudaMemsetAsync(nstop, 0, sizeof(uint32_t), s) == cudaSuccess;
+      ok &= launch_es_run(djobs, groups, n, samples, dists, a.st, a.chain_accepted, err, nstop, s, p->gstream, p->ev_in,
+                          p->ev_out, &run_launches) == cudaSuccess;
+      p->launches += run_launches;
+      if (!ok || group[0] == 0) break;  // only the largest windows stop
+      uint32_t stopped = 0, e = 0;
+      ok &= cudaMemcpyAsync(&stopped, nstop, sizeof(uint32_t), cudaMemcpyDeviceToHost, s) == cudaSuccess;
+      ok &= cudaMemcpyAsync(&e, err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s) == cudaSuccess;
+      ok &= cudaStreamSynchronize(s) == cudaSuccess;
+      if (e != 0) off = switches;  // an error ends the call
+      if (!ok || stopped == 0 || e != 0) break;
+      ok &= launch_es_set(djobs, nj, err, s, p->num_sms, true) == cudaSuccess;
+      p->launches += set_launches;
+    }
   }
   ok &= launch_es_load(a, djobs, djob_of, s, p->num_sms) == cudaSuccess;
   uint32_t host_err = 0;

@@ -3,27 +3,34 @@
 // ES-MC runs independent edge switches sigma_k = (i, j, g) one after
 // another (Def. 1's chain).  Algorithm 2 cuts the sequence into supersteps:
 // maximal runs of consecutive switches of which no two share a source
-// position, found with a first-touch table (each switch of a window writes
-// its index into the entries of its two positions with a minimum, and the
-// first switch that finds a smaller index there starts the next superstep;
-// the table is a shared-memory hash table keyed by position).  A
-// superstep has no source dependencies, so ParallelSuperstep (Algorithm 1)
-// performs it with the sequential outcome: each target edge exists when its
-// switch runs iff it was in E at the superstep's start and its eraser (the
-// switch whose source it is) is not an earlier legal switch, or an earlier
-// legal switch inserts it.
+// position.  Where a cut falls depends on the sampled positions only, never
+// on the graph, so the switches of a whole batch are sampled beforehand on
+// the whole GPU (k_es_sample), each with the distance to the last switch
+// before it that has a source position in common with it: the superstep that
+// starts at switch s ends before the first switch s + x whose distance is at
+// most x.  A superstep has no source dependencies, so ParallelSuperstep
+// (Algorithm 1) performs it with the sequential outcome: each target edge
+// exists when its switch runs iff it was in E at the superstep's start and its
+// eraser (the switch whose source it is) is not an earlier legal switch, or an
+// earlier legal switch inserts it.
 //
 // Supersteps of ES-MC hold about sqrt(m) switches (the birthday bound), so
-// one CTA runs all supersteps of one chain: the switches of a superstep, the
-// table of its erasers and the lists of its inserters live in shared memory,
-// the waves of Algorithm 1 are separated by __syncthreads, and the list E
+// one CTA runs all supersteps of one chain, a switch per thread.  The list E
 // (position order) and the edge set H (open addressing over canonical ids,
-// tombstones on erase) live in HBM.  Many chains run as many CTAs of one
-// launch.  A superstep is also cut at the window size (32 to 1024 switches,
-// by the chain's size); any cut into consecutive runs without source
-// dependencies gives the sequential result.  When tombstones pile up, the
-// set is rebuilt from the list between supersteps: in place by the CTA for
-// the smaller windows, on the whole GPU between launches for the largest.
+// tombstones on erase) live in HBM; a list entry also holds its edge's slot in
+// H, so that erasing it takes no search, and the search for a target ends at
+// the slot where it would be inserted.  Most supersteps have no dependency at
+// all: the targets go into a shared-memory table of fingerprints, and if no
+// fingerprint is met twice, by two targets or by a source, a switch is legal
+// iff none of its targets is in H.  Else the superstep's erasers and
+// inserters go into shared-memory tables and Algorithm 1's waves run,
+// separated by __syncthreads.  Many chains run as many CTAs of one launch.  A
+// superstep is also cut at the window size (32 to 1024 switches, by the
+// chain's size) and at the end of a batch; any cut into consecutive runs
+// without source dependencies gives the sequential result.  When tombstones
+// pile up, the set is rebuilt from the list between supersteps: in place by
+// the CTA for the smaller windows, on the whole GPU between launches for the
+// largest.
 #include "device_util.cuh"
 #include "gesmc_internal.cuh"
 
@@ -31,7 +38,7 @@ namespace gesmc {
 namespace {
 
 constexpr uint32_t kNil = 0xFFFFFFFFu;
-constexpr uint32_t kNoTouch = 0xFFFFFFFFu;
+constexpr unsigned long long kNoKey = 0;  // {0, 0}: not an edge, empty or tombstone
 constexpr uint8_t kEsUndecided = 0, kEsLegal = 1, kEsIllegal = 2;
 // Window sizes by chain size (supersteps hold about 0.63 sqrt(m) switches:
 // 450 at 2^19, 160 at 2^16, 57 at 2^13): chains of at least 2^19 edges run
@@ -48,128 +55,125 @@ __device__ __forceinline__ uint32_t hash32(unsigned long long key) { return (uin
 // ---------------------------------------------------------------- the edge set H
 // Open addressing with linear probing from h & mask (h = hash32(key)).
 // Insert a key that is not in the set into the first empty or tombstone
-// slot of its probe sequence.  Returns 0 (empty slot taken), 1 (tombstone
-// reused) or -1 (table full).
-__device__ __forceinline__ int hset_insert(unsigned long long *H, uint32_t mask, unsigned long long key, uint32_t h) {
-  uint32_t s = h & mask;
+// slot of its probe sequence from slot s on.  Returns the slot (with
+// *tomb = 1 if it held a tombstone), or kNil if the table is full.
+__device__ __forceinline__ uint32_t hset_insert(unsigned long long *H, uint32_t mask, unsigned long long key,
+                                                uint32_t s, uint32_t *tomb) {
   for (uint32_t n = 0; n <= mask; ++n) {
     const unsigned long long cur = __ldcg(&H[s]);
     if (cur == kEmptyKey || cur == kTombKey) {
-      if (atomicCAS(&H[s], cur, key) == cur) return cur == kTombKey ? 1 : 0;
+      if (atomicCAS(&H[s], cur, key) == cur) {
+        *tomb = cur == kTombKey ? 1u : 0u;
+        return s;
+      }
       continue;  // taken meanwhile: look at the same slot again
     }
     s = (s + 1) & mask;
   }
-  return -1;
+  return kNil;
 }
 
-// Two keys at once: both probe chains advance together, so that their loads
-// are in flight together (one HBM latency per step for the pair).
-// Presence: the first slots' loads are passed in (issued by the caller
-// before other work), bit w of the result says key w is in the set.
-__device__ __forceinline__ uint32_t hset_contains2(const unsigned long long *H, uint32_t mask,
-                                                   const unsigned long long (&key)[2], const uint32_t (&h)[2],
-                                                   unsigned long long (&cur)[2]) {
-  uint32_t s[2] = {h[0] & mask, h[1] & mask}, found = 0, done = 0;
+// Loads of a chain's list and set by its CTA.  kL1: through the SM's L1, for
+// the small windows, whose chains' lists and sets fit there (one CTA writes
+// them while the kernel runs, and its barriers order its own accesses); else
+// from L2.
+template <bool kL1>
+__device__ __forceinline__ unsigned long long set_load(const unsigned long long *p) {
+  unsigned long long v;
+  if constexpr (kL1) asm volatile("ld.global.ca.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  else asm volatile("ld.global.cg.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+template <bool kL1>
+__device__ __forceinline__ uint4 list_load(const uint4 *p) {
+  uint4 v;
+  if constexpr (kL1)
+    asm volatile("ld.global.ca.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+  else
+    asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+  return v;
+}
+
+// One warp inserts its lanes' keys (those of `legal` lanes, none of them in
+// the set) at once: every lane stores each of its keys in a free slot and
+// looks whose store stayed there, and the others search on.  p3, p4: where
+// the searches ended, f3, f4: whether that slot is known to be free; p3, p4, t3,
+// t4 receive the slots taken and whether they held tombstones.  All in the
+// SM's L1, where a compare-and-swap goes to L2 and back (512 chains of 65 to
+// 118,000 edges, 2^14 switches each: 10.3 ms with it, 8.9 ms without).  All lanes call it.
+__device__ __forceinline__ unsigned long long warp_load(const unsigned long long *p) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.cta.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void warp_store(unsigned long long *p, unsigned long long v) {
+  asm volatile("st.relaxed.cta.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+// The first free slot from p on; false if the table is full.
+__device__ __forceinline__ bool warp_find_free(const unsigned long long *H, uint32_t mask, uint32_t &p, uint32_t &t) {
   for (uint32_t n = 0; n <= mask; ++n) {
-#pragma unroll
-    for (int w = 0; w < 2; ++w) {
-      if ((done >> w) & 1u) continue;
-      if (cur[w] == key[w]) {
-        found |= 1u << w;
-        done |= 1u << w;
-      } else if (cur[w] == kEmptyKey) {
-        done |= 1u << w;
-      } else {
-        s[w] = (s[w] + 1) & mask;
-      }
+    const unsigned long long v = warp_load(&H[p]);
+    if (v == kEmptyKey || v == kTombKey) {
+      t = v == kTombKey;
+      return true;
     }
-    if (done == 3u) break;
-#pragma unroll
-    for (int w = 0; w < 2; ++w)
-      if (!((done >> w) & 1u)) cur[w] = __ldcg(&H[s[w]]);
+    p = (p + 1) & mask;
   }
-  return found;
+  return false;
 }
-
-__device__ __forceinline__ void hset_erase2(unsigned long long *H, uint32_t mask, const unsigned long long (&key)[2],
-                                            const uint32_t (&h)[2]) {
-  uint32_t s[2] = {h[0] & mask, h[1] & mask}, done = 0;
-  for (uint32_t n = 0; n <= mask && done != 3u; ++n) {
-    unsigned long long cur[2];
-#pragma unroll
-    for (int w = 0; w < 2; ++w)
-      if (!((done >> w) & 1u)) cur[w] = __ldcg(&H[s[w]]);
-#pragma unroll
-    for (int w = 0; w < 2; ++w) {
-      if ((done >> w) & 1u) continue;
-      if (cur[w] == key[w]) {
-        H[s[w]] = kTombKey;
-        done |= 1u << w;
-      } else if (cur[w] == kEmptyKey) {
-        done |= 1u << w;
-      } else {
-        s[w] = (s[w] + 1) & mask;
-      }
+__device__ __forceinline__ void warp_insert(unsigned long long *H, uint32_t mask, bool legal, unsigned long long e3,
+                                            unsigned long long e4, uint32_t &p3, uint32_t &p4, bool f3, bool f4,
+                                            uint32_t &t3, uint32_t &t4, uint32_t *err) {
+  bool o3 = legal, o4 = legal;
+  __syncwarp();  // the erasures
+  for (int round = 0;; ++round) {
+    bool full = false;
+    if (o3 && !f3) full |= !(o3 = warp_find_free(H, mask, p3, t3));
+    if (o4 && !f4) full |= !(o4 = warp_find_free(H, mask, p4, t4));
+    if (full) atomicOr(err, kErrTableFull);
+    __syncwarp();
+    if (o3) warp_store(&H[p3], e3);
+    if (o4) warp_store(&H[p4], e4);
+    __syncwarp();
+    if (o3) o3 = warp_load(&H[p3]) != e3;
+    if (o4) o4 = warp_load(&H[p4]) != e4;
+    if (!__any_sync(0xffffffffu, o3 || o4)) break;
+    if (round > 64) {  // a slot in dispute goes to one of the 64 keys each time: only in a full table
+      if (o3 || o4) atomicOr(err, kErrTableFull);
+      break;
     }
+    f3 = f4 = false;
   }
 }
 
-// Insert two keys that are not in the set, each into the first empty or
-// tombstone slot of its probe sequence.  r[w] = 0 (empty slot taken), 1
-// (tombstone reused) or -1 (table full).
-__device__ __forceinline__ void hset_insert2(unsigned long long *H, uint32_t mask, const unsigned long long (&key)[2],
-                                             const uint32_t (&h)[2], int (&r)[2]) {
-  uint32_t s[2] = {h[0] & mask, h[1] & mask}, done = 0;
-  uint32_t left[2] = {mask + 1, mask + 1};  // probes each key may still take
-  r[0] = r[1] = -1;
-  while (done != 3u) {
-    unsigned long long cur[2];
-#pragma unroll
-    for (int w = 0; w < 2; ++w)
-      if (!((done >> w) & 1u)) cur[w] = __ldcg(&H[s[w]]);
-#pragma unroll
-    for (int w = 0; w < 2; ++w) {
-      if ((done >> w) & 1u) continue;
-      if (left[w] == 0) {  // every slot looked at: table full
-        done |= 1u << w;
-        continue;
-      }
-      --left[w];
-      if (cur[w] == kEmptyKey || cur[w] == kTombKey) {
-        if (atomicCAS(&H[s[w]], cur[w], key[w]) == cur[w]) {
-          r[w] = cur[w] == kTombKey ? 1 : 0;
-          done |= 1u << w;
-        }
-        // taken meanwhile: look at the same slot again
-      } else {
-        s[w] = (s[w] + 1) & mask;
-      }
-    }
-  }
+// The list by position: {edge lo, edge hi, its slot in H, 0}.
+__device__ __forceinline__ unsigned long long rec_edge(const uint4 &r) {
+  return ((unsigned long long)r.y << 32) | r.x;
+}
+__device__ __forceinline__ uint4 make_rec(unsigned long long e, uint32_t slot) {
+  return make_uint4((uint32_t)e, (uint32_t)(e >> 32), slot, 0u);
 }
 
 // ---------------------------------------------------------------- shared memory
-// Per CTA, for windows of B switches (one per thread) and tables of S = 4B
-// slots: a region that holds the first-touch table while the window is cut
-// (position keys and minima, u32) and the erasers' and inserters' key tables
-// afterwards (u64), then the erasers' switches, the inserters' list heads and
-// links, and every switch's state.  Everything else a switch needs (its
+// Per CTA, for windows of B switches (one per thread): the fingerprints of
+// the superstep's targets (always empty between supersteps), and, for the
+// supersteps that have a dependency, tables of S = 4B slots: the erasers'
+// and inserters' keys (u64), the erasers' switches, the inserters' list heads
+// and links, and every switch's state.  Everything else a switch needs (its
 // positions, edges, hashes, outcome) stays in its thread's registers.
 template <int B>
 struct EsShape {
   static constexpr int kSlots = 4 * B;
-  static constexpr int kSlotsLog2 = B == 1024 ? 12 : B == 256 ? 10 : B == 128 ? 9 : B == 32 ? 7 : -1;
-  static constexpr size_t kRegion = 16ull * kSlots;
-  static constexpr size_t kBytes = kRegion + 4ull * (2 * kSlots + 2 * B) + B;
-  static_assert(kSlotsLog2 > 0, "window of 32, 128, 256 or 1024 switches");
+  static constexpr int kPrintLog2 = B == 1024 ? 13 : B == 256 ? 11 : B == 128 ? 10 : B == 32 ? 8 : -1;
+  static constexpr int kPrints = 1 << (kPrintLog2 > 0 ? kPrintLog2 : 0);
+  static constexpr size_t kBytes = 16ull * kSlots + 4ull * (2 * kSlots + 2 * B) + 4ull * kPrints + B;
+  static_assert(kPrintLog2 > 0, "window of 32, 128, 256 or 1024 switches");
 };
 
 template <int B>
 struct EsSmem {
-  unsigned long long *skey, *ikey;  // key tables (after the cut)
-  uint32_t *pkey, *pmin;            // first-touch table (until the cut); the same bytes
-  uint32_t *sval, *ihead, *tnext;
+  unsigned long long *skey, *ikey;  // key tables
+  uint32_t *sval, *ihead, *tnext, *print;
   uint8_t *st;
 };
 
@@ -180,13 +184,12 @@ __device__ __forceinline__ EsSmem<B> es_smem() {
   EsSmem<B> m;
   m.skey = es_dyn;
   m.ikey = es_dyn + S;
-  m.pkey = reinterpret_cast<uint32_t *>(es_dyn);
-  m.pmin = m.pkey + S;
   uint32_t *q = reinterpret_cast<uint32_t *>(es_dyn + 2 * S);
   m.sval = q;
   m.ihead = q + S;
   m.tnext = q + 2 * S;
-  m.st = reinterpret_cast<uint8_t *>(q + 2 * S + 2 * B);
+  m.print = q + 2 * S + 2 * B;
+  m.st = reinterpret_cast<uint8_t *>(m.print + EsShape<B>::kPrints);
   return m;
 }
 
@@ -209,257 +212,434 @@ __device__ __forceinline__ uint32_t table_slot(unsigned long long *keys, unsigne
   return kNil;
 }
 
-// First touches of a window (Algorithm 2's insert_if_min): position ->
-// smallest switch of the window that has it as a source position.  At most
-// 2B positions in S = 4B slots; a position is below 2^31, so never kNil.
-template <int S, int LOG2>
-__device__ __forceinline__ void touch_first(uint32_t *pkey, uint32_t *pmin, uint32_t pos, uint32_t x) {
-  uint32_t s = (pos * 0x9E3779B1u) >> (32 - LOG2);
-  for (int n = 0; n < S; ++n) {
-    uint32_t cur = pkey[s];
-    if (cur == kNil) {
-      cur = atomicCAS(&pkey[s], kNil, pos);
-      if (cur == kNil) cur = pos;
-    }
-    if (cur == pos) {
-      atomicMin(&pmin[s], x);
-      return;
-    }
-    s = (s + 1) & (S - 1);
-  }
-}
-
-template <int S, int LOG2>
-__device__ __forceinline__ uint32_t first_touch(const uint32_t *pkey, const uint32_t *pmin, uint32_t pos) {
-  uint32_t s = (pos * 0x9E3779B1u) >> (32 - LOG2);
-  for (int n = 0; n < S; ++n) {
-    const uint32_t cur = pkey[s];
-    if (cur == pos) return pmin[s];
-    if (cur == kNil) break;
-    s = (s + 1) & (S - 1);
-  }
-  return kNoTouch;
-}
-
-// The region as the first-touch table / as the key tables (with the list heads).
+// The CTA's barrier and vote (one warp: the warp's).
 template <int B>
-__device__ __forceinline__ void clear_touch(const EsSmem<B> &sm) {
-  for (uint32_t t = threadIdx.x; t < (uint32_t)EsShape<B>::kSlots; t += B) {
-    sm.pkey[t] = kNil;
-    sm.pmin[t] = kNoTouch;
-  }
+__device__ __forceinline__ void window_sync() {
+  if constexpr (B == 32) __syncwarp();
+  else __syncthreads();
 }
-
 template <int B>
-__device__ __forceinline__ void clear_tables(const EsSmem<B> &sm) {
-  for (uint32_t t = threadIdx.x; t < (uint32_t)EsShape<B>::kSlots; t += B) {
-    sm.skey[t] = kEmptyKey;
-    sm.ikey[t] = kEmptyKey;
-    sm.ihead[t] = kNil;
+__device__ __forceinline__ bool window_any(bool x) {
+  if constexpr (B == 32) {
+    __syncwarp();
+    return __any_sync(0xffffffffu, x);
+  } else {
+    return __syncthreads_or(x);
   }
 }
 
 // ---------------------------------------------------------------- kernels
 // H <- empty, for every job (blockIdx.y = job).
-__global__ void k_es_clear(const EsJob *jobs, uint32_t job_off, bool only_stopped) {
-  const EsJob jb = jobs[job_off + blockIdx.y];
+__global__ void k_es_clear(EsJob *jobs, uint32_t job_off, bool only_stopped) {
+  const EsJob &jb = jobs[job_off + blockIdx.y];
   if (jb.m < 2 || (only_stopped && !jb.stopped)) return;  // no list, no set; or a set that needs no rebuild
   const unsigned long long cap = 1ull << jb.hlog2;
   const unsigned long long nth = (unsigned long long)gridDim.x * blockDim.x;
+  unsigned long long *const H = jb.H;
   for (unsigned long long s = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; s < cap; s += nth)
-    jb.H[s] = kEmptyKey;
+    H[s] = kEmptyKey;
+  if (blockIdx.x == 0 && threadIdx.x == 0) jobs[job_off + blockIdx.y].tombs = 0;
 }
 
-// H <- the entries of E.
+// H <- the entries of E, each entry's slot into the list.
 __global__ void k_es_fill(const EsJob *jobs, uint32_t job_off, uint32_t *err, bool only_stopped) {
   const EsJob jb = jobs[job_off + blockIdx.y];
   if (jb.m < 2 || (only_stopped && !jb.stopped)) return;
   const uint32_t mask = (uint32_t)((1ull << jb.hlog2) - 1);
   for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < jb.m; s += gridDim.x * blockDim.x) {
-    const unsigned long long e = jb.E[s];
-    if (hset_insert(jb.H, mask, e, hash32(e)) < 0) atomicOr(err, kErrTableFull);
+    const unsigned long long e = rec_edge(jb.E[s]);
+    uint32_t tomb;
+    const uint32_t at = hset_insert(jb.H, mask, e, hash32(e) & mask, &tomb);
+    if (at == kNil) atomicOr(err, kErrTableFull);
+    else jb.E[s] = make_rec(e, at);
   }
 }
 
-// One CTA per job: switches k0 .. k0 + count - 1 of the job's chain, in
-// windows of B switches (thread x holds switch x of the window).
+// The switches off .. off + n - 1 of every job's call: positions and
+// direction, and for each the distance to the last switch before it, in this
+// batch and within a window, that shares a position with it (0xFFFF: none).
+// One CTA of C threads per C switches and job: it samples them and the W - 1
+// before them and chains the positions in a shared-memory hash table; a
+// position is in the table once for every switch that has it.
+template <int W, int C>
+__global__ void __launch_bounds__(C) k_es_sample(EsJob *jobs, uint32_t job_off, unsigned long long off, uint32_t n,
+                                                 uint2 *samples, uint16_t *dists) {
+  constexpr int kEntries = 2 * (C + W - 1);
+  constexpr int kLog2 = kEntries <= 512 ? 9 : kEntries <= 1024 ? 10 : kEntries <= 2048 ? 11 : 12;
+  static_assert(kEntries <= 4096, "table size");
+  __shared__ uint32_t pos[kEntries];
+  __shared__ uint16_t next[kEntries];
+  __shared__ __align__(4) uint16_t head[1 << kLog2];
+  EsJob &jb = jobs[job_off + blockIdx.y];
+  const uint32_t x = threadIdx.x, beg = blockIdx.x * C;
+  if (jb.m < 2) return;
+  if (blockIdx.x == 0 && x == 0) {  // the batch starts
+    jb.done = 0;
+    jb.stopped = 0;
+  }
+  const unsigned long long k0 = jb.k0 + off, seed = jb.seed, m = jb.m;
+  uint2 *const samp = samples + (size_t)jb.row * n;
+  uint16_t *const dist = dists + (size_t)jb.row * n;
+  for (uint32_t b = x; b < (1u << kLog2); b += C) head[b] = 0xFFFFu;
+  __syncthreads();
+  const uint32_t first = beg < W - 1 ? 0u : beg - (W - 1), end = min(beg + C, n);
+  for (uint32_t k = first + x; k < end; k += C) {
+    const U64x4 w = philox(k0 + k, 0, 2, 0, seed, 0);
+    const uint32_t i = (uint32_t)__umul64hi(w.w[0], m), jj = (uint32_t)__umul64hi(w.w[1], m - 1);
+    const uint32_t j = jj + (jj >= i ? 1u : 0u);
+    if (k >= beg) samp[k] = make_uint2(i, j | ((uint32_t)(w.w[2] >> 63) << 31));
+    const uint32_t t = 2 * (k - first);
+    pos[t] = i;
+    pos[t + 1] = j;
+  }
+  __syncthreads();
+  const uint32_t ne = 2 * (end - first);
+  for (uint32_t t = x; t < ne; t += C) {
+    // (16-bit exchange as a loop over the 32-bit word that holds the head)
+    const uint32_t b = (pos[t] * 0x9E3779B1u) >> (32 - kLog2);
+    uint32_t *const word = reinterpret_cast<uint32_t *>(head) + (b >> 1);
+    const uint32_t sh = (b & 1u) * 16;
+    uint32_t cur = *word, old;
+    do {
+      old = cur;
+      cur = atomicCAS(word, old, (old & ~(0xFFFFu << sh)) | (t << sh));
+    } while (cur != old);
+    next[t] = (uint16_t)(old >> sh);
+  }
+  __syncthreads();
+  const uint32_t k = beg + x;
+  if (k < end) {
+    const uint32_t own = k - first;
+    uint32_t last = 0;  // 1 + the last earlier switch with one of the two positions
+    for (int h = 0; h < 2; ++h) {
+      const uint32_t p = pos[2 * own + h];
+      for (uint32_t t = head[(p * 0x9E3779B1u) >> (32 - kLog2)]; t != 0xFFFFu; t = next[t]) {
+        const uint32_t v = t >> 1;
+        if (v < own && pos[t] == p) last = max(last, v + 1);
+      }
+    }
+    const uint32_t d = last ? own + 1 - last : 0xFFFFu;
+    dist[k] = (uint16_t)(d < (uint32_t)W ? d : 0xFFFFu);
+  }
+}
+
+// One CTA per job: the n switches of the batch from the job's last one
+// (done) on, in windows of B switches (thread x holds switch x of the window).
 // A CTA of the largest variant does not rebuild its chain's edge set itself
 // (one SM reinserting millions of ids): it stops after the superstep that
 // passes the tombstone limit (an eighth of the slots: rebuilds are cheap on
 // the whole GPU, and fewer tombstones keep the probe chains short), records
-// how far it got in jobs_out (k0, count advanced, stopped = 1, *nstop
-// counted), and the host rebuilds the set on the whole GPU and launches the
-// variant again; a finished job is left with count = 0, which a launch
-// again skips.  The smaller variants rebuild in place at a quarter.
+// how far it got (done, stopped = 1, *nstop counted), and the host rebuilds
+// the set on the whole GPU and launches the variant again; a job that is done
+// with the batch does nothing then.  The smaller variants rebuild in place at
+// a quarter.
+//
+// What bounds it: one chain's supersteps follow one another, each a chain of
+// dependent accesses (list entries, set slots, insertion) between a few
+// barriers; a window of 1024 switches is also bound by the 32-byte sectors
+// that one SM moves to and from L2 (about 11 a switch, and one every two
+// cycles or so at random addresses).  With sampling and first-touch tables in
+// every window, key tables for every superstep and separate searches to find,
+// erase and insert, 2^19 switches of a chain of 1e6 edges took 21.4 ms, now 7.2
+// (26 -> 8.9 us a superstep); 512 chains of 65 to 118,000 edges with 2^14
+// switches each 22.0 ms, now 8.9 (most are single warps: 2270 -> 430
+// instructions a superstep).
 template <int B, bool kStopToRebuild>
-__device__ __forceinline__ void es_run_body(const EsJob *jobs, uint32_t job_off, StatsDev *stats,
-                                            unsigned long long *chain_acc, uint32_t *err, EsJob *jobs_out,
-                                            uint32_t *nstop) {
-  constexpr int S = EsShape<B>::kSlots, LOG2 = EsShape<B>::kSlotsLog2;
-  const EsJob jb = jobs[job_off + blockIdx.x];
+__device__ __forceinline__ void es_run_body(EsJob *jobs, uint32_t job_off, uint32_t nsw, const uint2 *samples,
+                                            const uint16_t *dists, StatsDev *stats, unsigned long long *chain_acc,
+                                            uint32_t *err, uint32_t *nstop) {
+  constexpr int S = EsShape<B>::kSlots, PL = EsShape<B>::kPrintLog2;
+  constexpr bool kL1 = B <= 128;
+  constexpr uint32_t kPrintMask = EsShape<B>::kPrints - 1;
+  EsJob &job = jobs[job_off + blockIdx.x];
   const EsSmem<B> sm = es_smem<B>();
-  __shared__ uint32_t s_cut, s_tombs;
+  __shared__ uint32_t s_cut[2], s_tombs;
   const uint32_t x = threadIdx.x;
+  const uint32_t m = job.m;
   uint32_t acc = 0, rej_loop = 0, rej_exists = 0;
-  if (jb.m < 2) {  // no pair of positions: every requested switch is skipped
-    if (x == 0 && jb.count) atomicAdd(&stats->lazy, jb.count);
+  if (m < 2) {  // no pair of positions: every requested switch is skipped
+    if (x == 0) atomicAdd(&stats->lazy, (unsigned long long)nsw);
+    return;
+  }
+  uint4 *const E = job.E;
+  unsigned long long *const H = job.H;
+  const uint2 *const samp = samples + (size_t)job.row * nsw;
+  const uint16_t *const dist = dists + (size_t)job.row * nsw;
+  const uint32_t mask = (uint32_t)((1ull << job.hlog2) - 1);
+  uint32_t s = job.done;
+  if (s >= nsw) {
+    if (kStopToRebuild && x == 0) job.stopped = 0;
     return;
   }
   bool stop = false;
-  const uint32_t mask = (uint32_t)((1ull << jb.hlog2) - 1);
-  if (x == 0) s_tombs = 0;  // the set was built from the list just before
-  clear_touch(sm);
-  __syncthreads();
-  unsigned long long done = 0;  // switches run before a stop (largest variant)
-  for (unsigned long long s = 0; s < jb.count;) {
-    const uint32_t win = (uint32_t)min((unsigned long long)B, jb.count - s);
-    // sample the window and mark first touches (Algorithm 2's insert_if_min)
-    if (x == 0) s_cut = win;
-    uint32_t i = 0, j = 0, g = 0;
-    if (x < win) {
-      const U64x4 w = philox(jb.k0 + s + x, 0, 2, 0, jb.seed, 0);
-      i = (uint32_t)__umul64hi(w.w[0], (unsigned long long)jb.m);
-      const uint32_t jj = (uint32_t)__umul64hi(w.w[1], (unsigned long long)(jb.m - 1));
-      j = jj + (jj >= i ? 1u : 0u);
-      g = (uint32_t)(w.w[2] >> 63);
-      touch_first<S, LOG2>(sm.pkey, sm.pmin, i, x);
-      touch_first<S, LOG2>(sm.pkey, sm.pmin, j, x);
+  if (x == 0) {
+    s_tombs = job.tombs;
+    s_cut[0] = s_cut[1] = B;
+  }
+  for (uint32_t t = x; t <= kPrintMask; t += B) sm.print[t] = 0;
+  window_sync<B>();
+  // the first window's switch, and where its superstep ends
+  uint2 cur = make_uint2(0, 0);
+  uint32_t d = 0xFFFFu;
+  if (s + x < nsw) {
+    cur = __ldcs(&samp[s + x]);
+    d = __ldcs(&dist[s + x]);
+  }
+  uint32_t par = 0;
+  if constexpr (B > 32) {
+    if (d <= x) atomicMin(&s_cut[0], x);
+    __syncthreads();
+  }
+  while (s < nsw) {
+    uint32_t n = min((uint32_t)B, nsw - s);
+    if constexpr (B == 32) {
+      const unsigned hit = __ballot_sync(0xffffffffu, d <= x);
+      if (hit) n = min(n, (uint32_t)__ffs(hit) - 1);
+    } else {
+      n = min(n, s_cut[par]);
     }
-    __syncthreads();
-    // the superstep ends before the first switch that shares a position with an earlier one
-    if (x < win && (first_touch<S, LOG2>(sm.pkey, sm.pmin, i) < x || first_touch<S, LOG2>(sm.pkey, sm.pmin, j) < x))
-      atomicMin(&s_cut, x);
-    __syncthreads();
-    const uint32_t n = s_cut;
-    clear_tables(sm);  // the region becomes the key tables (the cut has read it)
+    const uint32_t i = cur.x, j = cur.y & 0x7FFFFFFFu, g = cur.y >> 31;
     // sources, targets and the outright rules
-    unsigned long long e1 = 0, e2 = 0, e3 = 0, e4 = 0;
-    uint32_t h1 = 0, h2 = 0, h3 = 0, h4 = 0, code = 1;
+    uint4 r1 = make_uint4(0, 0, 0, 0), r2 = r1;
     if (x < n) {
-      e1 = __ldcg(&jb.E[i]);
-      e2 = __ldcg(&jb.E[j]);
+      r1 = list_load<kL1>(&E[i]);
+      r2 = list_load<kL1>(&E[j]);
+    }
+    // the next window's switch, ahead of its use
+    d = 0xFFFFu;
+    if (s + n + x < nsw) {
+      cur = __ldcs(&samp[s + n + x]);
+      d = __ldcs(&dist[s + n + x]);
+    }
+    if (B > 32 && x == 0) s_cut[par ^ 1] = B;  // last read a superstep ago
+    const unsigned long long e1 = rec_edge(r1), e2 = rec_edge(r2);
+    unsigned long long e3 = 0, e4 = 0;
+    uint32_t code = 1;
+    if (x < n) {
       code = tau_g(g, e1, e2, e3, e4);
-      sm.st[x] = code ? kEsIllegal : kEsUndecided;
       if (code == kCodeLoop) ++rej_loop;
       else if (code) ++rej_exists;  // shared node: the targets re-create the sources
-      if (!code) {
-        h1 = hash32(e1);
-        h2 = hash32(e2);
-        h3 = hash32(e3);
-        h4 = hash32(e4);
+    }
+    // presence of the targets (the loads in flight while the fingerprints go
+    // in); a target's fingerprint is the high half of its hash
+    const bool live = code == 0;
+    bool dep = false;
+    uint32_t pres = 0, h3 = 0, h4 = 0, at3 = kNil, at4 = kNil, own3 = 0, own4 = 0;
+    unsigned long long was3 = kNoKey, was4 = kNoKey;  // what at3 and at4 held (kNoKey: no free slot was met)
+    if (live) {
+      const unsigned long long m3 = mix64(e3), m4 = mix64(e4);
+      h3 = (uint32_t)m3;
+      h4 = (uint32_t)m4;
+      uint32_t s3 = h3 & mask, s4 = h4 & mask;
+      unsigned long long c3 = set_load<kL1>(&H[s3]), c4 = set_load<kL1>(&H[s4]);
+      const uint32_t f3 = (uint32_t)(m3 >> 32) | 1u, f4 = (uint32_t)(m4 >> 32) | 1u;
+      own3 = f3 >> (32 - PL);
+      for (;;) {
+        const uint32_t old = atomicCAS(&sm.print[own3], 0u, f3);
+        if (old == 0) break;
+        if (old == f3) {
+          dep = true;
+          own3 = kNil;
+          break;
+        }
+        own3 = (own3 + 1) & kPrintMask;
       }
-    }
-    __syncthreads();
-    // erasers and inserters of the superstep; presence of the targets in E at its start (the first
-    // probes of the edge set are issued before the shared-memory tables are filled, so that they overlap)
-    uint32_t pres = 0;
-    if (x < n && code == 0) {
-      unsigned long long cur[2] = {__ldcg(&jb.H[h3 & mask]), __ldcg(&jb.H[h4 & mask])};
-      uint32_t t = table_slot<S>(sm.skey, e1, h1, true);
-      if (t != kNil) sm.sval[t] = x;
-      t = table_slot<S>(sm.skey, e2, h2, true);
-      if (t != kNil) sm.sval[t] = x;
-      const unsigned long long tk[2] = {e3, e4};
-      const uint32_t th[2] = {h3, h4};
-      t = table_slot<S>(sm.ikey, e3, h3, true);
-      if (t != kNil) sm.tnext[2 * x] = atomicExch(&sm.ihead[t], 2 * x);
-      else atomicOr(err, kErrTableFull);
-      t = table_slot<S>(sm.ikey, e4, h4, true);
-      if (t != kNil) sm.tnext[2 * x + 1] = atomicExch(&sm.ihead[t], 2 * x + 1);
-      else atomicOr(err, kErrTableFull);
-      pres = hset_contains2(jb.H, mask, tk, th, cur);
-    }
-    __syncthreads();
-    // waves (Algorithm 1): a switch decided in wave w only uses decisions of earlier waves
-    uint8_t dec = x < n ? sm.st[x] : kEsIllegal;
-    for (uint32_t wave = 1;; ++wave) {
-      if (dec == kEsUndecided) {
-        bool bad = false, wait = false;
-        for (uint32_t w = 0; w < 2 && !bad; ++w) {
-          const unsigned long long e = w ? e4 : e3;
-          const uint32_t h = w ? h4 : h3;
-          if ((pres >> w) & 1u) {  // in E at the start: present unless an earlier legal switch erased it
-            const uint32_t t = table_slot<S>(sm.skey, e, h, false);
-            const uint32_t p = t == kNil ? kNil : sm.sval[t];
-            if (p == kNil || p >= x || sm.st[p] == kEsIllegal) bad = true;
-            else if (sm.st[p] == kEsUndecided) wait = true;
-          }
-          if (bad) break;
-          const uint32_t t = table_slot<S>(sm.ikey, e, h, false);
-          for (uint32_t q = t == kNil ? kNil : sm.ihead[t]; q != kNil; q = sm.tnext[q]) {
-            const uint32_t k = q >> 1;  // an earlier switch that inserts e
-            if (k >= x) continue;
-            if (sm.st[k] == kEsLegal) {
-              bad = true;
-              break;
+      own4 = f4 >> (32 - PL);
+      for (;;) {
+        const uint32_t old = atomicCAS(&sm.print[own4], 0u, f4);
+        if (old == 0) break;
+        if (old == f4) {
+          dep = true;
+          own4 = kNil;
+          break;
+        }
+        own4 = (own4 + 1) & kPrintMask;
+      }
+      // both searches advance together; each ends at its key (present) or at
+      // an empty slot; at3, at4: the first slot that could take the key
+      uint32_t done = 0;
+      for (uint32_t q = 0; q <= mask; ++q) {
+        if (!(done & 1u)) {
+          if (c3 == e3) {
+            pres |= 1u;
+            done |= 1u;
+          } else {
+            if ((c3 == kEmptyKey || c3 == kTombKey) && at3 == kNil) {
+              at3 = s3;
+              was3 = c3;
             }
-            if (sm.st[k] == kEsUndecided) wait = true;
+            if (c3 == kEmptyKey) done |= 1u;
+            else s3 = (s3 + 1) & mask;
           }
         }
-        dec = bad ? kEsIllegal : (wait ? kEsUndecided : kEsLegal);
+        if (!(done & 2u)) {
+          if (c4 == e4) {
+            pres |= 2u;
+            done |= 2u;
+          } else {
+            if ((c4 == kEmptyKey || c4 == kTombKey) && at4 == kNil) {
+              at4 = s4;
+              was4 = c4;
+            }
+            if (c4 == kEmptyKey) done |= 2u;
+            else s4 = (s4 + 1) & mask;
+          }
+        }
+        if (done == 3u) break;
+        if (!(done & 1u)) c3 = set_load<kL1>(&H[s3]);
+        if (!(done & 2u)) c4 = set_load<kL1>(&H[s4]);
       }
-      __syncthreads();  // every read of this wave's states is done
-      if (x < n) sm.st[x] = dec;
-      const int left = __syncthreads_count(dec == kEsUndecided);
-      if (left == 0) break;
-      if (wave > (uint32_t)B) {  // every wave decides the smallest undecided switch: cannot happen
-        if (x == 0) atomicOr(err, kErrNoProgress);
-        return;
+      if (at3 == kNil) at3 = s3;  // present, or the table is full: insertion searches on from here
+      if (at4 == kNil) at4 = s4;
+    }
+    window_sync<B>();
+    if constexpr (B > 32) {  // where the next superstep ends, published by a barrier below
+      if (d <= x) atomicMin(&s_cut[par ^ 1], x);
+    }
+    // a source that is some target of the superstep
+    if (live) {
+#pragma unroll
+      for (int w = 0; w < 2; ++w) {
+        const uint32_t f = (uint32_t)(mix64(w ? e2 : e1) >> 32) | 1u;
+        uint32_t t = f >> (32 - PL);
+        for (;;) {
+          const uint32_t v = sm.print[t];
+          if (v == 0) break;
+          if (v == f) {
+            dep = true;
+            break;
+          }
+          t = (t + 1) & kPrintMask;
+        }
       }
     }
-    // apply: rewire, then erase the sources before inserting the targets
-    clear_touch(sm);  // the region becomes the next window's first-touch table (no table is read any more)
+    const bool some = window_any<B>(dep);
+    if (live) {  // the fingerprints have been read
+      if (own3 != kNil) sm.print[own3] = 0;
+      if (own4 != kNil) sm.print[own4] = 0;
+    }
+    uint8_t dec = !live ? kEsIllegal : pres ? kEsIllegal : kEsLegal;
+    if (some) {
+      // erasers and inserters of the superstep, and the waves of Algorithm 1
+      const uint32_t h1 = hash32(e1), h2 = hash32(e2);
+      for (uint32_t t = x; t < (uint32_t)S; t += B) {
+        sm.skey[t] = kEmptyKey;
+        sm.ikey[t] = kEmptyKey;
+        sm.ihead[t] = kNil;
+      }
+      if (x < n) sm.st[x] = live ? kEsUndecided : kEsIllegal;
+      window_sync<B>();
+      if (live) {
+        uint32_t t = table_slot<S>(sm.skey, e1, h1, true);
+        if (t != kNil) sm.sval[t] = x;
+        t = table_slot<S>(sm.skey, e2, h2, true);
+        if (t != kNil) sm.sval[t] = x;
+        t = table_slot<S>(sm.ikey, e3, h3, true);
+        if (t != kNil) sm.tnext[2 * x] = atomicExch(&sm.ihead[t], 2 * x);
+        else atomicOr(err, kErrTableFull);
+        t = table_slot<S>(sm.ikey, e4, h4, true);
+        if (t != kNil) sm.tnext[2 * x + 1] = atomicExch(&sm.ihead[t], 2 * x + 1);
+        else atomicOr(err, kErrTableFull);
+      }
+      window_sync<B>();
+      // a switch decided in wave w only uses decisions of earlier waves
+      dec = live ? kEsUndecided : kEsIllegal;
+      for (uint32_t wave = 1;; ++wave) {
+        if (dec == kEsUndecided) {
+          bool bad = false, wait = false;
+          for (uint32_t w = 0; w < 2 && !bad; ++w) {
+            const unsigned long long e = w ? e4 : e3;
+            const uint32_t h = w ? h4 : h3;
+            if ((pres >> w) & 1u) {  // in E at the start: present unless an earlier legal switch erased it
+              const uint32_t t = table_slot<S>(sm.skey, e, h, false);
+              const uint32_t p = t == kNil ? kNil : sm.sval[t];
+              if (p == kNil || p >= x || sm.st[p] == kEsIllegal) bad = true;
+              else if (sm.st[p] == kEsUndecided) wait = true;
+            }
+            if (bad) break;
+            const uint32_t t = table_slot<S>(sm.ikey, e, h, false);
+            for (uint32_t q = t == kNil ? kNil : sm.ihead[t]; q != kNil; q = sm.tnext[q]) {
+              const uint32_t k = q >> 1;  // an earlier switch that inserts e
+              if (k >= x) continue;
+              if (sm.st[k] == kEsLegal) {
+                bad = true;
+                break;
+              }
+              if (sm.st[k] == kEsUndecided) wait = true;
+            }
+          }
+          dec = bad ? kEsIllegal : (wait ? kEsUndecided : kEsLegal);
+        }
+        window_sync<B>();  // every read of this wave's states is done
+        if (x < n) sm.st[x] = dec;
+        if (!window_any<B>(dec == kEsUndecided)) break;
+        if (wave > (uint32_t)B) {  // every wave decides the smallest undecided switch: cannot happen
+          if (x == 0) atomicOr(err, kErrNoProgress);
+          return;
+        }
+      }
+    }
+    // apply: erase the sources where they are, insert the targets where their
+    // searches ended, rewire.  In no particular order: an insertion only takes
+    // empty slots and tombstones, and an erasure only its own edge's slot.
+    uint32_t tombs = 0;
     const bool legal = dec == kEsLegal;
     if (legal) {
-      jb.E[i] = e3;
-      jb.E[j] = e4;
-      const unsigned long long sk[2] = {e1, e2};
-      const uint32_t shh[2] = {h1, h2};
-      hset_erase2(jb.H, mask, sk, shh);
-      atomicAdd(&s_tombs, 2u);
+      H[r1.z] = kTombKey;
+      H[r2.z] = kTombKey;
+    }
+    uint32_t t3 = was3 == kTombKey, t4 = was4 == kTombKey, p3 = at3, p4 = at4;
+    if constexpr (B == 32) {
+      warp_insert(H, mask, legal, e3, e4, p3, p4, was3 != kNoKey, was4 != kNoKey, t3, t4, err);
+    } else if (legal) {
+      const unsigned long long g3 = atomicCAS(&H[at3], was3, e3), g4 = atomicCAS(&H[at4], was4, e4);
+      if (g3 != was3) p3 = hset_insert(H, mask, e3, at3, &t3);  // taken meanwhile, or no free slot was met
+      if (g4 != was4) p4 = hset_insert(H, mask, e4, at4, &t4);
+      if (p3 == kNil || p4 == kNil) atomicOr(err, kErrTableFull);
+    }
+    if (legal) {
+      E[i] = make_rec(e3, p3 & mask);  // (no slot, a full table, was reported: stay in bounds)
+      E[j] = make_rec(e4, p4 & mask);
+      tombs = 2u - t3 - t4;
       ++acc;
-    } else if (x < n && code == 0) {
+    } else if (live) {
       ++rej_exists;
     }
-    __syncthreads();
-    if (legal) {
-      const unsigned long long tk[2] = {e3, e4};
-      const uint32_t th[2] = {h3, h4};
-      int r[2];
-      hset_insert2(jb.H, mask, tk, th, r);
-      if (r[0] < 0 || r[1] < 0) atomicOr(err, kErrTableFull);
-      const uint32_t reused = (r[0] > 0 ? 1u : 0u) + (r[1] > 0 ? 1u : 0u);
-      if (reused) atomicSub(&s_tombs, reused);
+    tombs = __reduce_add_sync(0xffffffffu, tombs);
+    if ((x & 31u) == 0 && tombs) {
+      if constexpr (B == 32) s_tombs += tombs;
+      else atomicAdd(&s_tombs, tombs);
     }
-    __syncthreads();
+    window_sync<B>();
+    s += n;
+    par ^= 1u;
     if constexpr (kStopToRebuild) {
-      s += n;
       if (s_tombs > (mask >> 3)) {  // a rebuild on the whole GPU is cheap: keep the probe chains short
-        stop = s < jb.count;        // the same in every thread; a finished job needs no rebuild
-        done = s;
+        stop = s < nsw;             // the same in every thread; the batch's end needs no rebuild yet
         if (stop) break;
       }
     } else {
       if (s_tombs > (mask >> 2)) {  // rebuild the set from the list on this CTA
-        for (uint32_t t = x; t <= mask; t += B) jb.H[t] = kEmptyKey;
-        __syncthreads();
-        for (uint32_t t = x; t < jb.m; t += B) {
-          const unsigned long long e = __ldcg(&jb.E[t]);
-          if (hset_insert(jb.H, mask, e, hash32(e)) < 0) atomicOr(err, kErrTableFull);
+        window_sync<B>();           // every thread has read the count
+        for (uint32_t t = x; t <= mask; t += B) H[t] = kEmptyKey;
+        window_sync<B>();
+        for (uint32_t t = x; t < m; t += B) {
+          const unsigned long long e = rec_edge(list_load<kL1>(&E[t]));
+          uint32_t tomb;
+          const uint32_t at = hset_insert(H, mask, e, hash32(e) & mask, &tomb);
+          if (at == kNil) atomicOr(err, kErrTableFull);
+          else E[t] = make_rec(e, at);
         }
         if (x == 0) s_tombs = 0;
-        __syncthreads();
+        window_sync<B>();
       }
-      s += n;
     }
   }
-  if constexpr (kStopToRebuild) {
-    if (!stop) done = jb.count;
-    if (x == 0) {  // progress of the job (the host launches it again while stopped)
-      EsJob &out = jobs_out[job_off + blockIdx.x];
-      out.k0 = jb.k0 + done;
-      out.count = jb.count - done;
-      out.stopped = stop ? 1u : 0u;
+  if (x == 0) {  // progress of the job (the host launches it again while stopped)
+    job.tombs = s_tombs;
+    job.done = s;
+    if constexpr (kStopToRebuild) {
+      job.stopped = stop ? 1u : 0u;
       if (stop) atomicAdd(nstop, 1u);
     }
   }
@@ -470,7 +650,7 @@ __device__ __forceinline__ void es_run_body(const EsJob *jobs, uint32_t job_off,
   if ((x & 31) == 0) {
     if (a32) {
       atomicAdd(&stats->accepted, (unsigned long long)a32);
-      atomicAdd(&chain_acc[jb.chain], (unsigned long long)a32);
+      atomicAdd(&chain_acc[job.chain], (unsigned long long)a32);
     }
     if (l32) atomicAdd(&stats->rej_loop, (unsigned long long)l32);
     if (r32) atomicAdd(&stats->rej_exists, (unsigned long long)r32);
@@ -479,17 +659,20 @@ __device__ __forceinline__ void es_run_body(const EsJob *jobs, uint32_t job_off,
 
 // Windows of 32, 128 and 256 switches (the set rebuilt in place).
 template <int B, int MIN_BLOCKS>
-__global__ void __launch_bounds__(B, MIN_BLOCKS) k_es_run(const EsJob *jobs, uint32_t job_off, StatsDev *stats,
-                                                          unsigned long long *chain_acc, uint32_t *err) {
-  es_run_body<B, false>(jobs, job_off, stats, chain_acc, err, nullptr, nullptr);
+__global__ void __launch_bounds__(B, MIN_BLOCKS) k_es_run(EsJob *jobs, uint32_t job_off, uint32_t nsw,
+                                                          const uint2 *samples, const uint16_t *dists,
+                                                          StatsDev *stats, unsigned long long *chain_acc,
+                                                          uint32_t *err) {
+  es_run_body<B, false>(jobs, job_off, nsw, samples, dists, stats, chain_acc, err, nullptr);
 }
 
 // Windows of 1024 switches (chains of at least 2^19 edges: the set rebuilt
 // on the whole GPU between launches).
-__global__ void __launch_bounds__(1024, 1) k_es_run_big(EsJob *jobs, uint32_t job_off, StatsDev *stats,
+__global__ void __launch_bounds__(1024, 1) k_es_run_big(EsJob *jobs, uint32_t job_off, uint32_t nsw,
+                                                        const uint2 *samples, const uint16_t *dists, StatsDev *stats,
                                                         unsigned long long *chain_acc, uint32_t *err,
                                                         uint32_t *nstop) {
-  es_run_body<1024, true>(jobs, job_off, stats, chain_acc, err, jobs, nstop);
+  es_run_body<1024, true>(jobs, job_off, nsw, samples, dists, stats, chain_acc, err, nstop);
 }
 
 }  // namespace
@@ -506,7 +689,7 @@ cudaError_t prepare_es_kernels() {
                               (int)EsShape<256>::kBytes);
 }
 
-cudaError_t launch_es_set(const EsJob *jobs, uint32_t njobs, uint32_t *err, cudaStream_t s, int num_sms,
+cudaError_t launch_es_set(EsJob *jobs, uint32_t njobs, uint32_t *err, cudaStream_t s, int num_sms,
                           bool only_stopped) {
   for (uint32_t off = 0; off < njobs; off += 65535u) {
     const uint32_t nj = njobs - off < 65535u ? njobs - off : 65535u;
@@ -518,9 +701,26 @@ cudaError_t launch_es_set(const EsJob *jobs, uint32_t njobs, uint32_t *err, cuda
   return cudaGetLastError();
 }
 
-cudaError_t launch_es_run(EsJob *jobs, const uint32_t (&group)[4], StatsDev *stats,
-                          unsigned long long *chain_acc, uint32_t *err, uint32_t *nstop, cudaStream_t s,
-                          cudaStream_t s2, cudaEvent_t fork, cudaEvent_t join, uint32_t *launches) {
+cudaError_t launch_es_sample(EsJob *jobs, const uint32_t (&group)[4], unsigned long long off, uint32_t n,
+                             uint2 *samples, uint16_t *dists, cudaStream_t s, uint32_t *launches) {
+  uint32_t beg = 0;
+  for (int w = 0; w < 4; ++w) {
+    for (uint32_t o = beg; o < beg + group[w]; o += 65535u, ++*launches) {
+      const uint32_t nj = beg + group[w] - o < 65535u ? beg + group[w] - o : 65535u;
+      if (w == 0) k_es_sample<1024, 1024><<<dim3((n + 1023) / 1024, nj), 1024, 0, s>>>(jobs, o, off, n, samples, dists);
+      else if (w == 1) k_es_sample<256, 512><<<dim3((n + 511) / 512, nj), 512, 0, s>>>(jobs, o, off, n, samples, dists);
+      else if (w == 2) k_es_sample<128, 256><<<dim3((n + 255) / 256, nj), 256, 0, s>>>(jobs, o, off, n, samples, dists);
+      else k_es_sample<32, 128><<<dim3((n + 127) / 128, nj), 128, 0, s>>>(jobs, o, off, n, samples, dists);
+    }
+    beg += group[w];
+  }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_es_run(EsJob *jobs, const uint32_t (&group)[4], uint32_t nsw, const uint2 *samples,
+                          const uint16_t *dists, StatsDev *stats, unsigned long long *chain_acc, uint32_t *err,
+                          uint32_t *nstop, cudaStream_t s, cudaStream_t s2, cudaEvent_t fork, cudaEvent_t join,
+                          uint32_t *launches) {
   // group[w] jobs with windows of 1024, 256, 128 and 32 switches, in that
   // order; the two small-window groups run on s2 (after s, and joined back
   // into s) when there is one, beside the others
@@ -534,10 +734,16 @@ cudaError_t launch_es_run(EsJob *jobs, const uint32_t (&group)[4], StatsDev *sta
   auto run = [&](int w, cudaStream_t st) {
     for (uint32_t off = beg[w]; off < beg[w + 1]; off += 65535u, ++n) {
       const uint32_t nj = beg[w + 1] - off < 65535u ? beg[w + 1] - off : 65535u;
-      if (w == 0) k_es_run_big<<<nj, 1024, EsShape<1024>::kBytes, st>>>(jobs, off, stats, chain_acc, err, nstop);
-      else if (w == 1) k_es_run<256, 6><<<nj, 256, EsShape<256>::kBytes, st>>>(jobs, off, stats, chain_acc, err);
-      else if (w == 2) k_es_run<128, 12><<<nj, 128, EsShape<128>::kBytes, st>>>(jobs, off, stats, chain_acc, err);
-      else k_es_run<32, 32><<<nj, 32, EsShape<32>::kBytes, st>>>(jobs, off, stats, chain_acc, err);
+      if (w == 0)
+        k_es_run_big<<<nj, 1024, EsShape<1024>::kBytes, st>>>(jobs, off, nsw, samples, dists, stats, chain_acc, err,
+                                                              nstop);
+      else if (w == 1)
+        k_es_run<256, 6><<<nj, 256, EsShape<256>::kBytes, st>>>(jobs, off, nsw, samples, dists, stats, chain_acc, err);
+      else if (w == 2)
+        k_es_run<128, 12><<<nj, 128, EsShape<128>::kBytes, st>>>(jobs, off, nsw, samples, dists, stats, chain_acc,
+                                                                 err);
+      else
+        k_es_run<32, 32><<<nj, 32, EsShape<32>::kBytes, st>>>(jobs, off, nsw, samples, dists, stats, chain_acc, err);
     }
   };
   run(3, ss);

@@ -299,15 +299,20 @@ cudaError_t launch_duplicate_check(const unsigned long long *E, uint32_t m, unsi
                                    unsigned long long cap, uint32_t *flags, cudaStream_t s, int num_sms);
 
 // ParES (Algorithm 2) for one chain: its list in position order (in the
-// chain's tuple storage) and its edge set (open addressing, 2^hlog2 slots,
-// in the chain's permutation records), neither of which a round uses
-// between rounds; ES-MC switches k0 .. k0 + count - 1 with the chain's seed.
+// chain's tuple storage, {edge lo, edge hi, its slot in the edge set, 0} per
+// position) and its edge set (open addressing, 2^hlog2 slots, in the chain's
+// permutation records), neither of which a round uses between rounds; ES-MC
+// switches from number k0 on with the chain's seed.
 struct EsJob {
-  unsigned long long *E;
+  uint4 *E;
   unsigned long long *H;
-  unsigned long long seed, k0, count;  // the kernel advances k0 and count as it goes
+  unsigned long long seed, k0;  // k0: number of the call's first switch
   uint32_t m, hlog2, chain;
+  uint32_t row;      // place of the job's samples among the batch's
+  uint32_t done;     // switches of the batch that have run
+  uint32_t tombs;    // tombstones in the set
   uint32_t stopped;  // the kernel stopped this job for a rebuild of its set on the whole GPU
+  uint32_t pad;
 };
 
 // Shared-memory opt-in of the ParES kernels, once per device.
@@ -316,18 +321,24 @@ cudaError_t prepare_es_kernels();
 // 256, 128 or 32, by chain size).
 uint32_t es_window(uint32_t m);
 // Edge sets of all jobs (or only of the stopped ones) rebuilt from their lists.
-cudaError_t launch_es_set(const EsJob *jobs, uint32_t njobs, uint32_t *err, cudaStream_t s, int num_sms,
+cudaError_t launch_es_set(EsJob *jobs, uint32_t njobs, uint32_t *err, cudaStream_t s, int num_sms,
                           bool only_stopped);
-// All jobs' switches, one CTA per job: the first group[0] jobs with windows
-// of 1024, the next group[1] with windows of 256, then group[2] with 128 and
-// group[3] with 32 (these two on s2, forked from and joined back into s
-// through the two events, if given).  *launches receives the number of
+// A batch: the switches off .. off + n - 1 of the call, for every job with
+// m >= 2, sampled into row job.row (n entries each) of samples and dists.
+// group as for launch_es_run.
+cudaError_t launch_es_sample(EsJob *jobs, const uint32_t (&group)[4], unsigned long long off, uint32_t n,
+                             uint2 *samples, uint16_t *dists, cudaStream_t s, uint32_t *launches);
+// All jobs' switches of the batch, one CTA per job: the first group[0] jobs
+// with windows of 1024, the next group[1] with windows of 256, then group[2]
+// with 128 and group[3] with 32 (these two on s2, forked from and joined back
+// into s through the two events, if given).  *launches receives the number of
 // launches.
 // Jobs of the largest window stop when their set needs a rebuild (counted
 // in *nstop); the caller rebuilds those sets and launches again.
-cudaError_t launch_es_run(EsJob *jobs, const uint32_t (&group)[4], StatsDev *stats,
-                          unsigned long long *chain_acc, uint32_t *err, uint32_t *nstop, cudaStream_t s,
-                          cudaStream_t s2, cudaEvent_t fork, cudaEvent_t join, uint32_t *launches);
+cudaError_t launch_es_run(EsJob *jobs, const uint32_t (&group)[4], uint32_t nsw, const uint2 *samples,
+                          const uint16_t *dists, StatsDev *stats, unsigned long long *chain_acc, uint32_t *err,
+                          uint32_t *nstop, cudaStream_t s, cudaStream_t s2, cudaEvent_t fork, cudaEvent_t join,
+                          uint32_t *launches);
 // Lists of the chains with a job (job_of[chain] != kNoChain) out of their
 // slots into the jobs' position-order lists, and back (slots in position
 // order, nothing pending).

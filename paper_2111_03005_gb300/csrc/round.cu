@@ -1717,16 +1717,19 @@ __global__ void k_es_store(RoundArgs a, const EsJob *jobs, const uint32_t *job_o
     const uint32_t c = a.owner_slot[s0];
     if (c == kNoChain || job_of[c] == kNoChain) continue;
     const ChainDesc ch = a.chains[c];
-    unsigned long long *E = jobs[job_of[c]].E;
+    uint4 *E = jobs[job_of[c]].E;
+    auto put = [E](uint32_t pos, unsigned long long e) {
+      E[pos] = make_uint4((uint32_t)e, (uint32_t)(e >> 32), 0u, 0u);
+    };
     const uint32_t ls = s0 - ch.slot_base;
     if (ls + 1 < ch.m) {
       const uint32_t i = a.cpos[s0], j = a.cpos[s0 + 1];
       unsigned long long e1 = a.cedge[s0], e2 = a.cedge[s0 + 1];
       apply_last(a, ch, chain_apply(ch, R), ls >> 1, i, j, e1, e2);
-      E[i] = e1;
-      E[j] = e2;
+      put(i, e1);
+      put(j, e2);
     } else {
-      E[a.cpos[s0]] = a.cedge[s0];
+      put(a.cpos[s0], a.cedge[s0]);
     }
   }
 }
@@ -1738,7 +1741,7 @@ __global__ void k_es_load(RoundArgs a, const EsJob *jobs, const uint32_t *job_of
     const ChainDesc ch = a.chains[c];
     const uint32_t ls = s - ch.slot_base;
     a.cpos[s] = ls;
-    a.cedge[s] = jobs[job_of[c]].E[ls];
+    a.cedge[s] = *reinterpret_cast<const unsigned long long *>(&jobs[job_of[c]].E[ls]);
     if ((ls & 1u) == 0 && (ls >> 1) < ch.L) a.status[ch.switch_base + (ls >> 1)] = 0;  // nothing pending
   }
 }

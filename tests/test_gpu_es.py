@@ -183,3 +183,13 @@ def test_pool_mixes_window_sizes_with_rebuilds():
         x = oracle.validate(e, n)[1]
         x, _ = oracle.es_run(x, seed=600 + t, switches=1_200_000)
         assert np.array_equal(outs[t], x), t
+
+
+@pytest.mark.parametrize("m, switches", [(2, 1500), (5, 3000), (40, 5000), (300, 4000), (5000, 40_000),
+                                         (9000, 60_000), (70_000, 400_000)])
+def test_calls_longer_than_a_batch_of_samples(m, switches):
+    # a call samples its switches in batches of about three per edge (at least
+    # a few hundred): batches end inside windows of every size but the largest
+    n = max(8, int(3 * m ** 0.5) + 8)
+    edges = inputs.random_simple_graph(n, m, seed=m + 3)
+    es_compare(edges, n, seed=m, calls=[switches])
