@@ -61,10 +61,11 @@ enum {
                               starting degree sequence (gesmc_verify)        */
 };
 
-/* Rounds are replayed from a captured CUDA graph of one round (launched on
- * a private stream ordered after and before the caller's stream); this flag
- * launches the kernels one by one instead.  Stage timing always launches
- * them one by one. */
+/* Rounds run on a private stream ordered after and before the caller's
+ * stream, and once a handle has run a number of them with the same chains they
+ * are replayed from a captured CUDA graph of a few rounds; with this flag the
+ * kernels are launched one by one on the caller's stream instead.  Stage
+ * timing always launches them one by one. */
 #define GESMC_FLAG_NO_GRAPHS 1u
 /* Def. 2 as printed: each round draws l ~ Binom(floor(m/2), 1 - P_L) and
  * runs only its first l switches, l = the number of switches whose laziness

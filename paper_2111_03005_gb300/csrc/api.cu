@@ -287,13 +287,14 @@ struct gesmc_pool_ctx {
   RoundArgs args;
   uint64_t args_version = 1;  // bumped whenever args change (invalidates the graph)
   uint32_t wave_kernels = 0;  // whole-GPU wave kernel pairs per round (grows with the waves seen)
-  // captured round (CUDA graph), replayed on gstream
+  // captured rounds (a CUDA graph of kGraphRounds rounds), replayed on gstream
   bool use_graphs = true;
   cudaStream_t gstream = nullptr;
   cudaEvent_t ev_in = nullptr, ev_out = nullptr;
   cudaGraphExec_t gexec = nullptr;
   uint64_t graph_version = 0;
   uint32_t graph_launches = 0;
+  uint64_t warm_version = 0, warm_rounds = 0;  // rounds launched with the current arguments
   // one-launch rounds (k_round_fused) with this many CTAs; 0: the kernels of
   // a round one after another (replayed from the captured graph)
   uint32_t fused_ctas = 0;
@@ -316,6 +317,12 @@ struct gesmc_pool_ctx {
   double stage_ms[kNumStages] = {};
   uint64_t stage_rounds = 0;
 };
+
+// A round's 14 or more launches take the host about 30 us; a graph of them
+// replays without, but is worth its capture (about 0.1 ms a round) only for
+// pools whose arguments stay.
+constexpr uint32_t kGraphRounds = 4;
+constexpr uint64_t kGraphAfterRounds = 16;
 
 struct gesmc_ctx {
   gesmc_pool_t pool = nullptr;
@@ -838,53 +845,74 @@ int pool_run(gesmc_pool_t p, uint64_t rounds) {
         ++launches;
       }
     }
-  } else if (p->use_graphs && !p->profiling && rounds > 0) {
-    if (!p->gexec || p->graph_version != p->args_version) {
-      if (p->gexec) cudaGraphExecDestroy(p->gexec);
-      p->gexec = nullptr;
-      cudaGraph_t graph = nullptr;
-      uint32_t n = 0;
-      bool ok = cudaStreamBeginCapture(p->gstream, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-      if (ok) {
-        const bool launched = launch_round(a, p->gstream, p->num_sms, nullptr, &n) == cudaSuccess;
-        ok = cudaStreamEndCapture(p->gstream, &graph) == cudaSuccess && launched;
+  } else {
+    // the round's kernels one after another, on the private stream (ordered
+    // after and before the caller's), unless there is none or the stages are
+    // timed.  After kGraphAfterRounds rounds with the same arguments they are
+    // replayed from a graph of kGraphRounds rounds, if it is there or enough
+    // rounds are left to be worth its capture
+    const bool side = p->use_graphs && !p->profiling;
+    cudaStream_t gs = side ? p->gstream : s;
+    bool ok = true, after = false;
+    if (side)
+      ok = cudaEventRecord(p->ev_in, s) == cudaSuccess && cudaStreamWaitEvent(gs, p->ev_in, 0) == cudaSuccess;
+    if (p->warm_version != p->args_version) {
+      p->warm_version = p->args_version;
+      p->warm_rounds = 0;
+    }
+    auto direct = [&](uint64_t from, uint64_t to) {
+      for (uint64_t r = from; r < to && ok; ++r) {
+        cudaEvent_t *ev = stage_events ? &p->events[per_round * r] : nullptr;
+        nvtxRangePushA("gesmc round");
+        ok = launch_round(a, gs, p->num_sms, ev, after, &launches) == cudaSuccess;
+        nvtxRangePop();
+        after = true;
       }
-      ok = ok && cudaGraphInstantiate(&p->gexec, graph, 0) == cudaSuccess;
-      if (graph) cudaGraphDestroy(graph);
-      if (!ok) {
-        cudaGetLastError();
+    };
+    const uint64_t lead = p->warm_rounds < kGraphAfterRounds ? std::min(rounds, kGraphAfterRounds - p->warm_rounds) : 0;
+    const bool have = p->gexec && p->graph_version == p->args_version;
+    uint64_t done = rounds;  // rounds launched directly before the graph's
+    if (side && rounds - lead >= (have ? kGraphRounds : kGraphAfterRounds)) {
+      done = lead;
+      direct(0, done);
+      if (ok && !have) {
+        if (p->gexec) cudaGraphExecDestroy(p->gexec);
         p->gexec = nullptr;
-        p->broken = GESMC_E_CUDA;
-        return GESMC_E_CUDA;
+        cudaGraph_t graph = nullptr;
+        uint32_t n = 0;
+        ok = cudaStreamBeginCapture(gs, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+        if (ok) {
+          bool launched = true;
+          for (uint32_t r = 0; r < kGraphRounds && launched; ++r)
+            launched = launch_round(a, gs, p->num_sms, nullptr, r > 0, &n) == cudaSuccess;
+          ok = cudaStreamEndCapture(gs, &graph) == cudaSuccess && launched;
+        }
+        ok = ok && cudaGraphInstantiate(&p->gexec, graph, 0) == cudaSuccess;
+        if (graph) cudaGraphDestroy(graph);
+        if (!ok) p->gexec = nullptr;
+        p->graph_version = p->args_version;
+        p->graph_launches = n;
       }
-      p->graph_version = p->args_version;
-      p->graph_launches = n;
+      while (ok && rounds - done >= kGraphRounds) {
+        nvtxRangePushA("gesmc rounds");
+        ok = cudaGraphLaunch(p->gexec, gs) == cudaSuccess;
+        nvtxRangePop();
+        launches += p->graph_launches;
+        done += kGraphRounds;
+      }
+      after = false;  // a graph launch ended: nothing to overlap with
+      direct(done, rounds);
+    } else {
+      direct(0, rounds);
     }
-    bool ok = cudaEventRecord(p->ev_in, s) == cudaSuccess && cudaStreamWaitEvent(p->gstream, p->ev_in, 0) == cudaSuccess;
-    for (uint64_t r = 0; r < rounds && ok; ++r) {
-      nvtxRangePushA("gesmc round");
-      ok = cudaGraphLaunch(p->gexec, p->gstream) == cudaSuccess;
-      nvtxRangePop();
-    }
-    ok = ok && cudaEventRecord(p->ev_out, p->gstream) == cudaSuccess &&
-         cudaStreamWaitEvent(s, p->ev_out, 0) == cudaSuccess;
+    if (side && ok)
+      ok = cudaEventRecord(p->ev_out, gs) == cudaSuccess && cudaStreamWaitEvent(s, p->ev_out, 0) == cudaSuccess;
     if (!ok) {
       cudaGetLastError();
       p->broken = GESMC_E_CUDA;
       return GESMC_E_CUDA;
     }
-    launches = (uint32_t)(rounds * p->graph_launches);
-  } else {
-    for (uint64_t r = 0; r < rounds; ++r) {
-      cudaEvent_t *ev = p->profiling ? &p->events[per_round * r] : nullptr;
-      nvtxRangePushA("gesmc round");
-      const cudaError_t e = launch_round(a, s, p->num_sms, ev, &launches);
-      nvtxRangePop();
-      if (e != cudaSuccess) {
-        p->broken = GESMC_E_CUDA;
-        return GESMC_E_CUDA;
-      }
-    }
+    p->warm_rounds += rounds;
   }
   Counters ctl;
   if (cudaMemcpyAsync(&ctl, a.ctl, sizeof(Counters), cudaMemcpyDeviceToHost, s) != cudaSuccess ||

@@ -267,8 +267,11 @@ size_t group_smem_bytes(uint32_t group_log2);
 cudaError_t prepare_kernels(uint32_t group_log2, int num_sms, LaunchShapes *shapes);
 
 // One pool round.  ev (optional) receives kNumStages + 1 events around the
-// stages; *launches (optional) counts the kernels launched.
-cudaError_t launch_round(const RoundArgs &a, cudaStream_t s, int num_sms, cudaEvent_t *ev, uint32_t *launches);
+// stages; after_round: the launch before this one on the stream is another
+// round's last (this round's first kernel may then start while it ends);
+// *launches (optional) counts the kernels launched.
+cudaError_t launch_round(const RoundArgs &a, cudaStream_t s, int num_sms, cudaEvent_t *ev, bool after_round,
+                         uint32_t *launches);
 
 // The one-launch round: every stage of a pool round in one cooperative launch
 // of `ctas` CTAs (at most fused_max_ctas() of them), the stages separated by

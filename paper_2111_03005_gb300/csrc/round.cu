@@ -295,6 +295,10 @@ __device__ __forceinline__ void clear_body(const RoundArgs &a) {
   for (uint32_t p = tid; p < a.part_hw; p += nth) a.ocount[p] = 0;
   for (uint32_t p = tid; p < a.tcount_hw; p += nth) a.tcount[p] = 0;
   for (uint32_t c = tid; c < a.chain_hw; c += nth) a.chain_ell[c] = 0;
+  if (a.any_work) {  // the target filter: at least 2^12 bits
+    uint4 *const f = reinterpret_cast<uint4 *>(a.tfilter);
+    for (uint32_t w = tid; w <= (a.tfilter_mask >> 7); w += nth) f[w] = make_uint4(0, 0, 0, 0);
+  }
   if (tid == 0) {
     a.ctl->pending[0] = 0;
     a.ctl->pending[1] = 0;
@@ -308,7 +312,20 @@ __device__ __forceinline__ void clear_body(const RoundArgs &a) {
   }
 }
 
-__global__ void k_clear(RoundArgs a) { clear_body(a); }
+// The kernels of a round follow one another by programmatic dependent launch:
+// each lets the next one start as soon as its own CTAs are all on the GPU
+// (dep_launch) and reads and writes nothing that changes during a round before
+// the one before it has ended (dep_wait).  A kernel waits for the one before
+// it even where it does nothing else, so that "the one before has ended"
+// means all of them.  Chain descriptors and owner maps do not change while
+// rounds run.  A round of G(1000, 0.01) took 69 us replayed from a plain graph,
+// 61 us so, and 53 us with the scatter on more SMs and the statistics closed by
+// several warps (18 kernels: what is left is their own chains of L2 accesses).
+__global__ void k_clear(RoundArgs a) {
+  dep_launch();
+  dep_wait();
+  clear_body(a);
+}
 
 __device__ __forceinline__ void store_record(const RoundArgs &a, uint32_t b, uint32_t idx, uint32_t keybits,
                                              uint32_t pos, unsigned long long e) {
@@ -319,86 +336,72 @@ __device__ __forceinline__ void store_record(const RoundArgs &a, uint32_t b, uin
 }
 
 // The positions of the chain with few buckets (a pool of one chain with at
-// most kAggBuckets buckets), each CTA taking kAggThreads * kAggPairs
-// consecutive pairs of slots: the CTA counts its records per bucket in
-// shared memory (a record's rank among the CTA's records of its bucket comes
-// with it), takes each bucket's range with one cursor atomic, then stores
-// its records (keys recomputed).  With few buckets every cursor takes
-// thousands of same-address atomics per round, which serialise in L2; here
-// it takes one per CTA.  The order of records inside a bucket does not
-// matter: the sort orders them by key and position.
-constexpr int kAggThreads = 1024, kAggPairs = 2;
-
-// The pair of slots x of the chain (its position and edge pair with the last
-// round's decision applied, and the keys).
-__device__ __forceinline__ void agg_pair(const RoundArgs &a, const ChainDesc &ch, unsigned long long R,
-                                         unsigned long long round, uint32_t x, bool &two, uint32_t (&pos)[2],
-                                         unsigned long long (&e)[2], unsigned long long (&K)[2]) {
-  const uint32_t gx = (ch.slot_base >> 1) + x;  // pair index in the pool's slots
-  two = 2 * x + 1 < ch.m;
-  if (two) {
-    const uint2 ij = __ldcs(reinterpret_cast<const uint2 *>(a.cpos) + gx);
-    const ulonglong2 ee = __ldcs(reinterpret_cast<const ulonglong2 *>(a.cedge) + gx);
-    e[0] = ee.x;
-    e[1] = ee.y;
-    apply_last(a, ch, chain_apply(ch, R), x, ij.x, ij.y, e[0], e[1]);
-    pos[0] = ij.x;
-    pos[1] = ij.y;
-  } else {  // odd m: the chain's last slot has no partner
-    pos[0] = a.cpos[2 * gx];
-    e[0] = a.cedge[2 * gx];
-    pos[1] = 0;
-    e[1] = 0;
-  }
-  K[0] = perm_key(ch.seed, round, pos[0]);
-  K[1] = two ? perm_key(ch.seed, round, pos[1]) : 0ull;
-}
-
-__global__ void __launch_bounds__(kAggThreads, 1) k_permute_agg(RoundArgs a) {
+// most kAggBuckets buckets), each CTA taking kThreads * kPairs consecutive
+// pairs of slots: the CTA counts its records per bucket in shared memory (a
+// record's rank among the CTA's records of its bucket comes with it), takes
+// each bucket's range with one cursor atomic, then stores its records, which
+// stay in registers meanwhile.  With few buckets every cursor takes thousands
+// of same-address atomics per round, which serialise in L2; here it takes one
+// per CTA.  The order of records inside a bucket does not matter: the sort
+// orders them by key and position.  Bound by the generator (a Philox block per
+// position, about 400 instructions): with the keys computed again for the
+// second pass it took 38 us for 9.5e5 positions and, on two CTAs of 2048 pairs, 19 us
+// for 5,000; now 28 us, and 5.4 us on ten CTAs of 256 pairs.
+template <int kThreads, int kPairs>
+__global__ void __launch_bounds__(kThreads, 1024 / kThreads) k_permute_agg(RoundArgs a) {
   __shared__ uint32_t sc[kAggBuckets];  // per bucket: the CTA's count, then its base
+  dep_launch();
   const ChainDesc ch = a.chains[a.agg_chain];
+  const uint32_t tid = threadIdx.x, nb = 1u << ch.B, npair = (ch.m + 1) >> 1;
+  for (uint32_t b = tid; b < nb; b += kThreads) sc[b] = 0;
+  dep_wait();
   const unsigned long long R = a.ctl->pool_round;
   const unsigned long long round = chain_round(ch, R);
-  const uint32_t tid = threadIdx.x, nb = 1u << ch.B, npair = (ch.m + 1) >> 1;
-  const uint32_t x0 = blockIdx.x * (kAggThreads * kAggPairs) + tid;
-  for (uint32_t b = tid; b < nb; b += kAggThreads) sc[b] = 0;
+  const bool apply = chain_apply(ch, R);
+  const uint32_t x0 = blockIdx.x * (kThreads * kPairs) + tid;
   __syncthreads();
-  uint32_t bk[2 * kAggPairs], rk[2 * kAggPairs];
+  uint32_t pos[2 * kPairs], mid[2 * kPairs], br[2 * kPairs];  // br: bucket, and the rank in the high half
+  unsigned long long e[2 * kPairs];
 #pragma unroll
-  for (int j = 0; j < kAggPairs; ++j) {
-    const uint32_t x = x0 + j * kAggThreads;
-    bk[2 * j] = bk[2 * j + 1] = kNoChain;
+  for (int j = 0; j < kPairs; ++j) {
+    const uint32_t x = x0 + j * kThreads;
+    br[2 * j] = br[2 * j + 1] = kNoChain;
     if (x >= npair) continue;
-    bool two;
-    uint32_t pos[2];
-    unsigned long long e[2], K[2];
-    agg_pair(a, ch, R, round, x, two, pos, e, K);
-    bk[2 * j] = bucket_of(K[0], ch.B);
-    rk[2 * j] = atomicAdd(&sc[bk[2 * j]], 1u);
+    const uint32_t gx = (ch.slot_base >> 1) + x;  // pair index in the pool's slots
+    const bool two = 2 * x + 1 < ch.m;
     if (two) {
-      bk[2 * j + 1] = bucket_of(K[1], ch.B);
-      rk[2 * j + 1] = atomicAdd(&sc[bk[2 * j + 1]], 1u);
+      const uint2 ij = __ldcs(reinterpret_cast<const uint2 *>(a.cpos) + gx);
+      const ulonglong2 ee = __ldcs(reinterpret_cast<const ulonglong2 *>(a.cedge) + gx);
+      e[2 * j] = ee.x;
+      e[2 * j + 1] = ee.y;
+      apply_last(a, ch, apply, x, ij.x, ij.y, e[2 * j], e[2 * j + 1]);
+      pos[2 * j] = ij.x;
+      pos[2 * j + 1] = ij.y;
+    } else {  // odd m: the chain's last slot has no partner
+      pos[2 * j] = a.cpos[2 * gx];
+      e[2 * j] = a.cedge[2 * gx];
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (h == 1 && !two) continue;
+      const unsigned long long K = perm_key(ch.seed, round, pos[2 * j + h]);
+      const uint32_t b = bucket_of(K, ch.B);
+      mid[2 * j + h] = mid_of(K, ch.B);
+      br[2 * j + h] = b | (atomicAdd(&sc[b], 1u) << 16);
     }
   }
   __syncthreads();
-  for (uint32_t b = tid; b < nb; b += kAggThreads) {
+  for (uint32_t b = tid; b < nb; b += kThreads) {
     const uint32_t n = sc[b];
     if (n) sc[b] = atomicAdd(&a.pcount[ch.bucket_base + b], n);
   }
   __syncthreads();
 #pragma unroll
-  for (int j = 0; j < kAggPairs; ++j) {
-    const uint32_t x = x0 + j * kAggThreads;
-    if (x >= npair) continue;
-    bool two;
-    uint32_t pos[2];
-    unsigned long long e[2], K[2];
-    agg_pair(a, ch, R, round, x, two, pos, e, K);
-    store_record(a, ch.bucket_base + bk[2 * j], sc[bk[2 * j]] + rk[2 * j], mid_of(K[0], ch.B), pos[0], e[0]);
-    if (two)
-      store_record(a, ch.bucket_base + bk[2 * j + 1], sc[bk[2 * j + 1]] + rk[2 * j + 1], mid_of(K[1], ch.B), pos[1],
-                   e[1]);
-  }
+  for (int j = 0; j < 2 * kPairs; ++j)
+    if (br[j] != kNoChain) {
+      const uint32_t b = br[j] & 0xFFFFu;
+      store_record(a, ch.bucket_base + b, sc[b] + (br[j] >> 16), mid[j], pos[j], e[j]);
+    }
 }
 
 // Exact l (Def. 2 as printed): per chain in that mode, the number of its
@@ -426,7 +429,11 @@ __device__ __forceinline__ void lazy_count_body(const RoundArgs &a) {
   if (n) atomicAdd(&a.chain_ell[cur], n);
 }
 
-__global__ void k_lazy_count(RoundArgs a) { lazy_count_body(a); }
+__global__ void k_lazy_count(RoundArgs a) {
+  dep_launch();
+  dep_wait();
+  lazy_count_body(a);
+}
 
 // Append every position, with its current edge, to its chain's bucket.
 // Five CTAs of 256 per SM (48 registers, no spills): 3.16 ms per round on
@@ -477,7 +484,9 @@ __device__ __forceinline__ uint32_t scrambled_cta(uint32_t stride) {
 
 // One pair of slots per thread, CTAs in scrambled order.
 __global__ void __launch_bounds__(256, 5) k_permute(RoundArgs a) {
+  dep_launch();
   const uint32_t x = scrambled_cta(a.permute_stride) * blockDim.x + threadIdx.x;
+  dep_wait();
   if (x < (a.slot_hw + 1) >> 1) permute_pair(a, x, a.ctl->pool_round);
 }
 
@@ -516,6 +525,8 @@ __device__ __forceinline__ void cta_scan_1024(const uint32_t *count, uint32_t *o
 // pblk[b / 1024] + poff[b].
 __global__ void __launch_bounds__(1024) k_scan_perm(RoundArgs a) {
   __shared__ uint32_t warp_tot[32];
+  dep_launch();
+  dep_wait();
   const uint32_t b = blockIdx.x * 1024 + threadIdx.x;
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t v = b < a.bucket_hw ? min(a.pcount[b], 1u << a.bucket_log2) : 0u;
@@ -542,6 +553,8 @@ __global__ void __launch_bounds__(1024) k_scan_perm(RoundArgs a) {
 }
 
 __global__ void __launch_bounds__(1024) k_scan_blocks(RoundArgs a) {
+  dep_launch();
+  dep_wait();
   const uint32_t nblk = (a.bucket_hw + 1023) / 1024;
   cta_scan_1024(a.pblk, a.pblk, nullptr, nblk, 0xFFFFFFFFu);
 }
@@ -563,9 +576,15 @@ __device__ __forceinline__ void overflow_count_body(const RoundArgs &a) {
     atomicAdd(&a.ocount[a.otup[t].w], 1u);
 }
 
-__global__ void k_overflow_count(RoundArgs a) { overflow_count_body(a); }
+__global__ void k_overflow_count(RoundArgs a) {
+  dep_launch();
+  dep_wait();
+  overflow_count_body(a);
+}
 
 __global__ void __launch_bounds__(1024) k_overflow_scan_blocks(RoundArgs a) {
+  dep_launch();
+  dep_wait();
   if (a.ctl->ovf_count == 0) return;
   __shared__ uint32_t warp_tot[32];
   const uint32_t p = blockIdx.x * 1024 + threadIdx.x;
@@ -598,6 +617,8 @@ __global__ void __launch_bounds__(1024) k_overflow_scan_blocks(RoundArgs a) {
 }
 
 __global__ void __launch_bounds__(1024) k_overflow_scan_top(RoundArgs a) {
+  dep_launch();
+  dep_wait();
   if (a.ctl->ovf_count == 0) return;
   const uint32_t nblk = (a.part_hw + 1023) / 1024;
   cta_scan_1024(a.oblk, a.oblk, nullptr, nblk, 0xFFFFFFFFu);  // oblk[nblk] = all overflow tuples
@@ -617,7 +638,11 @@ __device__ __forceinline__ void overflow_scatter_body(const RoundArgs &a) {
   }
 }
 
-__global__ void k_overflow_scatter(RoundArgs a) { overflow_scatter_body(a); }
+__global__ void k_overflow_scatter(RoundArgs a) {
+  dep_launch();
+  dep_wait();
+  overflow_scatter_body(a);
+}
 
 // In-place exclusive scan of 2^kLog2 counters by a CTA of kThreads.
 template <int kThreads, int kLog2>
@@ -628,10 +653,22 @@ __device__ __forceinline__ void cta_exclusive_scan(uint32_t *h, uint32_t *warp_t
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   uint32_t loc[per];
   uint32_t sum = 0;
+  if constexpr (per % 4 == 0) {  // (word by word, a warp's lanes would share few banks)
 #pragma unroll
-  for (int r = 0; r < per; ++r) {
-    loc[r] = h[tid * per + r];
-    sum += loc[r];
+    for (int r = 0; r < per; r += 4) {
+      const uint4 v = reinterpret_cast<const uint4 *>(h)[(tid * per + r) / 4];
+      loc[r] = v.x;
+      loc[r + 1] = v.y;
+      loc[r + 2] = v.z;
+      loc[r + 3] = v.w;
+      sum += v.x + v.y + v.z + v.w;
+    }
+  } else {
+#pragma unroll
+    for (int r = 0; r < per; ++r) {
+      loc[r] = h[tid * per + r];
+      sum += loc[r];
+    }
   }
   uint32_t incl = sum;
 #pragma unroll
@@ -654,8 +691,17 @@ __device__ __forceinline__ void cta_exclusive_scan(uint32_t *h, uint32_t *warp_t
   uint32_t run = incl - sum + (warp ? warp_tot[warp - 1] : 0);
 #pragma unroll
   for (int r = 0; r < per; ++r) {
-    h[tid * per + r] = run;
-    run += loc[r];
+    const uint32_t c = loc[r];
+    loc[r] = run;
+    run += c;
+  }
+  if constexpr (per % 4 == 0) {
+#pragma unroll
+    for (int r = 0; r < per; r += 4)
+      reinterpret_cast<uint4 *>(h)[(tid * per + r) / 4] = make_uint4(loc[r], loc[r + 1], loc[r + 2], loc[r + 3]);
+  } else {
+#pragma unroll
+    for (int r = 0; r < per; ++r) h[tid * per + r] = loc[r];
   }
 }
 
@@ -842,11 +888,13 @@ __global__ void __launch_bounds__(1 << (kLog2 - 3), kMin) k_sortpair(RoundArgs a
   constexpr int kThreads = 1 << (kLog2 - 3);
   __shared__ __align__(128) uint4 srec[1 << kLog2];
   __shared__ uint16_t sidx[1 << kLog2];
-  __shared__ uint32_t hist[1 << kLog2];
+  __shared__ __align__(16) uint32_t hist[1 << kLog2];
   __shared__ uint32_t warp_tot[kThreads / 32];
   __shared__ __align__(8) unsigned long long bar;
+  dep_launch();
   if (threadIdx.x == 0) mbar_init(&bar, 1);
   __syncthreads();
+  dep_wait();
   const SortSmem sm{srec, sidx, hist, warp_tot, &bar};
   uint32_t parity = 0;
   if (sort_bucket<kThreads, kLog2>(a, blockIdx.x, sm, parity) && threadIdx.x == 0) mbar_inval(&bar);
@@ -876,7 +924,11 @@ __device__ __forceinline__ void boundary_body(const RoundArgs &a) {
   }
 }
 
-__global__ void k_boundary(RoundArgs a) { boundary_body(a); }
+__global__ void k_boundary(RoundArgs a) {
+  dep_launch();
+  dep_wait();
+  boundary_body(a);
+}
 
 // The chain of a thread's current pair, kept while its consecutive pairs
 // stay in it: pairs [lo, hi) are chain c's.
@@ -990,7 +1042,9 @@ __device__ __forceinline__ void source_pairs(const RoundArgs &a, uint32_t x, uin
 // One launch of short-lived CTAs, two pairs per thread (measured faster than
 // a grid-stride loop over a resident grid).
 __global__ void __launch_bounds__(256, 4) k_sources(RoundArgs a) {
+  dep_launch();
   const uint32_t end = a.slot_hw >> 1;
+  dep_wait();
   const uint32_t x = scrambled_cta(a.sources_stride) * 2 * blockDim.x + threadIdx.x;
   if (x < end) source_pairs(a, x, x + blockDim.x, end);
 }
@@ -1120,9 +1174,10 @@ __device__ __forceinline__ void group_body(const RoundArgs &a) {
   __shared__ int stk_top;
   __shared__ uint32_t overflow;
   const int tid = threadIdx.x;
-  const bool ovf = a.ctl->ovf_count != 0;
   for (uint32_t s = tid; s < S; s += T) group_reset_slot(g, s);
   if (tid == 0) overflow = 0;
+  dep_wait();  // (does nothing in the one-launch round)
+  const bool ovf = a.ctl->ovf_count != 0;
   __syncthreads();
   for (uint32_t part = blockIdx.x; part < a.part_hw; part += gridDim.x) {
     const uint32_t c = a.owner_part[part];
@@ -1231,7 +1286,10 @@ __device__ __forceinline__ void group_body(const RoundArgs &a) {
   }
 }
 
-__global__ void __launch_bounds__(kGroupThreads, 2) k_group(RoundArgs a) { group_body<kGroupThreads, kGroupR>(a); }
+__global__ void __launch_bounds__(kGroupThreads, 2) k_group(RoundArgs a) {
+  dep_launch();
+  group_body<kGroupThreads, kGroupR>(a);
+}
 
 // Each CTA takes a contiguous range of switches, so that a thread's running
 // per-chain count changes chain only at chain boundaries.
@@ -1274,7 +1332,11 @@ __device__ __forceinline__ void wave1_body(const RoundArgs &a) {
   flush_count(a, cc);
 }
 
-__global__ void k_wave1(RoundArgs a) { wave1_body(a); }
+__global__ void k_wave1(RoundArgs a) {
+  dep_launch();
+  dep_wait();
+  wave1_body(a);
+}
 
 __device__ __forceinline__ uint32_t wave_cap(const RoundArgs &a) {
   return a.max_waves ? a.max_waves : kDefaultWaveCap;
@@ -1286,6 +1348,8 @@ __device__ __forceinline__ uint32_t wave_cap(const RoundArgs &a) {
 // Nothing to do once no switch is undecided, or past the wave cap (k_tail
 // reports that).
 __global__ void k_wave_register(RoundArgs a) {
+  dep_launch();
+  dep_wait();
   const uint32_t cur = a.ctl->cur, wave = a.ctl->wave_next;
   const uint32_t n = a.ctl->pending[cur];
   if (n == 0 || wave > wave_cap(a)) return;
@@ -1307,9 +1371,12 @@ __global__ void k_wave_register(RoundArgs a) {
 // finish moves the wave number on and switches lists.
 __global__ void k_wave_decide(RoundArgs a) {
   __shared__ bool last;
+  dep_launch();
+  dep_wait();
   const uint32_t cur = a.ctl->cur, wave = a.ctl->wave_next;
   const uint32_t n = a.ctl->pending[cur];
-  if (n == 0 || wave > wave_cap(a)) return;
+  const uint32_t active = min(gridDim.x, (n + blockDim.x - 1) / blockDim.x);  // CTAs with a switch
+  if (blockIdx.x >= active || wave > wave_cap(a)) return;
   Tally t;
   ChainCount cc;
   const uint32_t *in = cur ? a.list1 : a.list0;
@@ -1341,7 +1408,7 @@ __global__ void k_wave_decide(RoundArgs a) {
   flush_count(a, cc);
   __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) last = atomicAdd(&a.ctl->wave_blocks, 1u) == gridDim.x - 1;
+  if (threadIdx.x == 0) last = atomicAdd(&a.ctl->wave_blocks, 1u) == active - 1;
   __syncthreads();
   if (last && threadIdx.x == 0) {
     __threadfence();
@@ -1351,12 +1418,47 @@ __global__ void k_wave_decide(RoundArgs a) {
   }
 }
 
+// End of a pool round: wave telemetry, statistics, and the pool's round
+// counter.  Called by every thread of a CTA of 256 or more: each word is one
+// warp's, so that their loads are in flight together (by one thread, one after
+// another, they took k_tail 5 of its 7.5 us).
+__device__ __forceinline__ void close_round(const RoundArgs &a, uint32_t wave) {
+  const uint32_t waves = a.any_work ? wave - 1 : 0, tid = threadIdx.x;
+  for (uint32_t w = wave + tid; w < kWaveHist; w += blockDim.x) a.st->last_pending[w] = 0;
+  if (tid & 31u) return;
+  switch (tid >> 5) {
+    case 0:
+      a.ctl->pool_round += 1;
+      break;
+    case 1:
+      a.ctl->waves = waves;
+      a.st->last_pending[1] = a.switch_hw;
+      break;
+    case 2:
+      if (a.any_work) a.st->waves_total += waves;
+      break;
+    case 3:
+      if (a.any_work && waves > a.st->waves_max) a.st->waves_max = waves;
+      break;
+    case 4:
+      if (a.any_work) a.st->wave_hist[waves < kWaveHist ? waves : kWaveHist - 1] += 1;
+      break;
+    case 5:
+      a.st->overflow_tuples += a.ctl->ovf_count;
+      break;
+    default:
+      break;
+  }
+}
+
 // Waves 2, 3, ... on one CTA: undecided switches re-register as inserters
 // (the q fields of illegal minima were cleared), then decide.  The kernel
 // also closes the pool round (the round counter every chain derives its own
 // round number from).
 __global__ void __launch_bounds__(1024) k_tail(RoundArgs a) {
   __shared__ uint32_t s_n;
+  dep_launch();
+  dep_wait();
   Tally t;
   ChainCount cc;
   uint32_t cur = a.ctl->cur, wave = a.ctl->wave_next, prev_n = a.switch_hw + 1;
@@ -1415,21 +1517,11 @@ __global__ void __launch_bounds__(1024) k_tail(RoundArgs a) {
     cur ^= 1;
     ++wave;
   }
-  flush_tally(a, t);
-  flush_count(a, cc);
-  if (threadIdx.x == 0) {
-    const uint32_t waves = a.any_work ? wave - 1 : 0;
-    a.ctl->waves = waves;
-    if (a.any_work) {
-      a.st->waves_total += waves;
-      if (waves > a.st->waves_max) a.st->waves_max = waves;
-      a.st->wave_hist[waves < kWaveHist ? waves : kWaveHist - 1] += 1;
-    }
-    a.st->last_pending[1] = a.switch_hw;
-    a.st->overflow_tuples += a.ctl->ovf_count;
-    for (uint32_t w = wave; w < kWaveHist; ++w) a.st->last_pending[w] = 0;
-    a.ctl->pool_round += 1;
+  if (prev_n <= a.switch_hw) {  // some waves ran here
+    flush_tally(a, t);
+    flush_count(a, cc);
   }
+  close_round(a, wave);
 }
 
 // ---------------------------------------------------------------- one-launch round
@@ -1508,22 +1600,6 @@ __device__ __forceinline__ uint32_t cta_scan_full(const uint32_t *count, uint32_
   return tot;
 }
 
-// End of a pool round (the work of k_tail after its waves): wave telemetry,
-// statistics, and the pool's round counter.  One thread.
-__device__ __forceinline__ void close_round(const RoundArgs &a, uint32_t wave) {
-  const uint32_t waves = a.any_work ? wave - 1 : 0;
-  a.ctl->waves = waves;
-  if (a.any_work) {
-    a.st->waves_total += waves;
-    if (waves > a.st->waves_max) a.st->waves_max = waves;
-    a.st->wave_hist[waves < kWaveHist ? waves : kWaveHist - 1] += 1;
-  }
-  a.st->last_pending[1] = a.switch_hw;
-  a.st->overflow_tuples += a.ctl->ovf_count;
-  for (uint32_t w = wave; w < kWaveHist; ++w) a.st->last_pending[w] = 0;
-  a.ctl->pool_round += 1;
-}
-
 // The whole round of a pool in one cooperative launch of kFusedThreads-thread
 // CTAs: the same stages as the multi-kernel round, in the same order, each
 // spread over the launch's CTAs, with a grid barrier where the multi-kernel
@@ -1552,7 +1628,6 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_round_fused(RoundArgs a) {
   __syncthreads();
   unsigned long long target = start_count;
   clear_body(a);
-  for (uint32_t w = gtid; w <= (a.tfilter_mask >> 5); w += nth) a.tfilter[w] = 0;
   if (!grid_sync(ctl, target)) return;
   uint32_t wave = 2;
   if (a.any_work) {
@@ -1575,9 +1650,9 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_round_fused(RoundArgs a) {
       const size_t room = size_t(1) << a.bucket_log2;
       SortSmem sm;
       sm.srec = reinterpret_cast<uint4 *>(base);
-      sm.sidx = reinterpret_cast<uint16_t *>(base + sizeof(uint4) * room);
-      sm.hist = reinterpret_cast<uint32_t *>(base + (sizeof(uint4) + sizeof(uint16_t)) * room);
-      sm.warp_tot = sm.hist + room;
+      sm.hist = reinterpret_cast<uint32_t *>(base + sizeof(uint4) * room);
+      sm.sidx = reinterpret_cast<uint16_t *>(sm.hist + room);
+      sm.warp_tot = reinterpret_cast<uint32_t *>(sm.sidx + room);
       sm.bar = reinterpret_cast<unsigned long long *>(sm.warp_tot + 32);
       if (tid == 0) mbar_init(sm.bar, 1);
       __syncthreads();
@@ -1677,7 +1752,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_round_fused(RoundArgs a) {
     flush_tally(a, t);
     flush_count(a, cc);
   }
-  if (gtid == 0) close_round(a, wave);
+  if (blockIdx.x == 0) close_round(a, wave);
 }
 
 // ---------------------------------------------------------------- state in / out
@@ -1871,7 +1946,8 @@ cudaError_t launch_round_fused(const RoundArgs &a, cudaStream_t s, uint32_t ctas
                                      fused_smem_bytes(a.group_log2), s);
 }
 
-cudaError_t launch_round(const RoundArgs &a, cudaStream_t s, int num_sms, cudaEvent_t *ev, uint32_t *launches) {
+cudaError_t launch_round(const RoundArgs &a, cudaStream_t s, int num_sms, cudaEvent_t *ev, bool after_round,
+                         uint32_t *launches) {
   // ev (optional) receives kNumStages + 1 stage boundaries; stages that do
   // not run (no chain with two edges) still get both events (zero duration)
   auto mark = [&](int stage) {
@@ -1879,68 +1955,80 @@ cudaError_t launch_round(const RoundArgs &a, cudaStream_t s, int num_sms, cudaEv
   };
   uint32_t n = 0;
   const bool work = a.any_work != 0;
+  // programmatic dependent launch, but for the first kernel unless the one
+  // before it is a round's too (what came before may not wait as they do), and
+  // not between the events of stage timing
+  cudaError_t bad = cudaSuccess;
+  auto go = [&](void (*fn)(RoundArgs), uint32_t ctas, uint32_t threads, size_t smem = 0) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = !ev && (n > 0 || after_round) ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, fn, a);
+    if (e != cudaSuccess && bad == cudaSuccess) bad = e;
+    ++n;
+  };
   mark(kStageClear);
-  if (work) cudaMemsetAsync(a.tfilter, 0, 4ull * ((a.tfilter_mask >> 5) + 1), s);
-  k_clear<<<grid_for(max(max(a.bucket_hw, a.part_hw), a.tcount_hw), 256, num_sms, 4), 256, 0, s>>>(a);
-  ++n;
-  if (work && a.any_exact) { k_lazy_count<<<grid_for(a.switch_hw, 256, num_sms, 8), 256, 0, s>>>(a); ++n; }
+  const uint32_t clear = max(max(max(a.bucket_hw, a.part_hw), a.tcount_hw), work ? a.tfilter_mask >> 7 : 0u);
+  go(k_clear, grid_for(clear, 256, num_sms, 4), 256);
+  if (work && a.any_exact) go(k_lazy_count, grid_for(a.switch_hw, 256, num_sms, 8), 256);
   mark(kStagePermute);
-  if (work && a.agg_chain != kNoChain) {
-    k_permute_agg<<<(a.agg_pairs + kAggThreads * kAggPairs - 1) / (kAggThreads * kAggPairs), kAggThreads, 0, s>>>(a);
-    ++n;
-  } else if (work) {
-    k_permute<<<a.permute_ctas, 256, 0, s>>>(a);
-    ++n;
-  }
+  if (work && a.agg_chain != kNoChain)
+    // few pairs: spread over the SMs; more: more records per cursor atomic
+    if (a.agg_pairs <= (uint32_t)num_sms * 512) go(k_permute_agg<256, 1>, (a.agg_pairs + 255) / 256, 256);
+    else go(k_permute_agg<1024, 2>, (a.agg_pairs + 2047) / 2048, 1024);
+  else if (work)
+    go(k_permute, a.permute_ctas, 256);
   mark(kStageScanPerm);
   if (work) {
-    k_scan_perm<<<a.bucket_hw ? (a.bucket_hw + 1023) / 1024 : 1, 1024, 0, s>>>(a);
-    k_scan_blocks<<<1, 1024, 0, s>>>(a);
-    n += 2;
+    go(k_scan_perm, a.bucket_hw ? (a.bucket_hw + 1023) / 1024 : 1, 1024);
+    go(k_scan_blocks, 1, 1024);
   }
   mark(kStageSortPair);
   if (work) {
     if (a.bucket_log2 == kBucketLog2Small)
-      k_sortpair<kBucketLog2Small, 7><<<a.bucket_hw, 1 << (kBucketLog2Small - 3), 0, s>>>(a);
+      go(k_sortpair<kBucketLog2Small, 7>, a.bucket_hw, 1 << (kBucketLog2Small - 3));
     else
-      k_sortpair<kBucketLog2Large, 4><<<a.bucket_hw, 1 << (kBucketLog2Large - 3), 0, s>>>(a);
-    ++n;
+      go(k_sortpair<kBucketLog2Large, 4>, a.bucket_hw, 1 << (kBucketLog2Large - 3));
   }
   mark(kStageBoundary);
-  if (work) { k_boundary<<<grid_for(a.bucket_hw, 256, num_sms, 2), 256, 0, s>>>(a); ++n; }
+  if (work) go(k_boundary, grid_for(a.bucket_hw, 256, num_sms, 2), 256);
   mark(kStageSources);
-  if (work) { k_sources<<<a.sources_ctas, 256, 0, s>>>(a); ++n; }
+  if (work) go(k_sources, a.sources_ctas, 256);
   mark(kStageOverflow);
   if (work) {
     const int g = grid_for(a.ovf_cap, 256, num_sms, 2);
-    k_overflow_count<<<g, 256, 0, s>>>(a);
-    k_overflow_scan_blocks<<<(a.part_hw + 1023) / 1024 ? (a.part_hw + 1023) / 1024 : 1, 1024, 0, s>>>(a);
-    k_overflow_scan_top<<<1, 1024, 0, s>>>(a);
-    k_overflow_scatter<<<g, 256, 0, s>>>(a);
-    n += 4;
+    go(k_overflow_count, g, 256);
+    go(k_overflow_scan_blocks, (a.part_hw + 1023) / 1024 ? (a.part_hw + 1023) / 1024 : 1, 1024);
+    go(k_overflow_scan_top, 1, 1024);
+    go(k_overflow_scatter, g, 256);
   }
   mark(kStageGroup);
   if (work) {
     const uint32_t ctas = a.group_grid ? a.group_grid : (uint32_t)num_sms;
-    k_group<<<ctas < a.part_hw ? ctas : a.part_hw, kGroupThreads, group_smem_bytes(a.group_log2), s>>>(a);
-    ++n;
+    go(k_group, ctas < a.part_hw ? ctas : a.part_hw, kGroupThreads, group_smem_bytes(a.group_log2));
   }
   mark(kStageWave1);
-  if (work) { k_wave1<<<grid_for(a.switch_hw, 256, num_sms, 16), 256, 0, s>>>(a); ++n; }
+  if (work) go(k_wave1, grid_for(a.switch_hw, 256, num_sms, 16), 256);
   mark(kStageWaves);
   if (work) {
     for (uint32_t w = 0; w < a.wave_kernels && w < kMaxWaveKernels; ++w) {
-      k_wave_register<<<num_sms * 4, 256, 0, s>>>(a);
-      k_wave_decide<<<num_sms * 4, 256, 0, s>>>(a);
-      n += 2;
+      go(k_wave_register, num_sms * 4, 256);
+      go(k_wave_decide, num_sms * 4, 256);
     }
   }
   mark(kStageTail);
-  k_tail<<<1, 1024, 0, s>>>(a);
-  ++n;
+  go(k_tail, 1, 1024);
   mark(kNumStages);
   if (launches) *launches += n;
-  return cudaGetLastError();
+  const cudaError_t last = cudaGetLastError();
+  return bad != cudaSuccess ? bad : last;
 }
 
 cudaError_t launch_load_chain(const RoundArgs &a, const ChainDesc &ch, const unsigned long long *E, cudaStream_t s,

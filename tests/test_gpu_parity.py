@@ -343,3 +343,32 @@ def test_gnp_2p27_largest_size_keeps_degrees_and_simplicity():
     assert not bool((srt[1:] == srt[:-1]).any())                # no repeated edge
     assert st["accepted"] + st["rejected_exists"] + st["rejected_loop"] + st["lazy"] == 2 * (m // 2)
     assert st["accepted"] > 0.99 * 2 * (m // 2)
+
+
+def test_replayed_rounds_after_direct_ones():
+    # the first rounds with the same chains are launched directly, later ones
+    # replayed from a graph of a few rounds, with a remainder launched directly
+    edges, n = inputs.workload_gnp_small(seed=8)
+    with gesmc.Chain(edges, n=n) as a, gesmc.Chain(edges, n=n, graphs=False) as b:
+        total = 0
+        for rounds in (3, 30, 7, 1, 40, 18):
+            a.run(rounds, 9)
+            b.run(rounds, 9)
+            total += rounds
+            assert np.array_equal(a.edges(), b.edges())
+        sa, sb = a.stats(), b.stats()
+    assert all(sa[k] == sb[k] for k in ("rounds", "accepted", "rejected_exists", "waves_total", "wave_hist"))
+    want, st = oracle.run(edges, seed=9, rounds=total)
+    assert st["accepted"] == sa["accepted"]
+    with gesmc.Chain(edges, n=n) as c:
+        assert np.array_equal(c.run(total, 9).edges(), want)
+
+
+@pytest.mark.parametrize("m", [155_647, 155_648, 155_649, 4_194_303, 4_194_305])
+def test_scatter_variants_at_their_limits(m):
+    # one chain: the shape of the aggregated scatter changes with the pairs per
+    # SM, and above 8192 buckets every record takes its own cursor atomic
+    edges, n = inputs.gnp(m, 2.4 / (m - 1), seed=m), m
+    edges = np.random.default_rng(m).permutation(edges)[:m]
+    assert len(edges) == m
+    run_and_compare(edges, n, seed=3, rounds=2)
