@@ -181,10 +181,10 @@ int gesmc_reset_stats(gesmc_t h);
  * profiled rounds into *rounds.  Stage i is named by gesmc_stage_name(i);
  * GESMC_NUM_STAGES stages exist, in launch order, each one kernel except
  * "overflow" (three kernels that return at once when nothing overflowed)
- * and "waves" (a pair of kernels per wave after the first, run on the whole
- * GPU; as many pairs as the handle's rounds have needed extra waves so far,
- * at most 8, none while every round needed one wave; "tail" runs any waves
- * beyond those on one CTA). */
+ * and "waves" (a pair of kernels per wave after the first that more than
+ * 2048 undecided switches enter, run on the whole GPU; as many pairs as the
+ * handle's rounds have needed such waves so far, at most 8, none while no
+ * round needed one; "tail" runs the other waves on one CTA). */
 #define GESMC_NUM_STAGES 11
 int gesmc_set_profiling(gesmc_t h, int enable);
 int gesmc_stage_times(gesmc_t h, double *ms, int n_stages, uint64_t *rounds);

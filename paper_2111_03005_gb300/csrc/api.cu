@@ -286,7 +286,7 @@ struct gesmc_pool_ctx {
   int broken = 0;
   RoundArgs args;
   uint64_t args_version = 1;  // bumped whenever args change (invalidates the graph)
-  uint32_t wave_kernels = 0;  // whole-GPU wave kernel pairs per round (grows with the waves seen)
+  uint32_t wave_kernels = 0;  // whole-GPU wave kernel pairs per round (grows with the wide waves seen)
   // captured rounds (a CUDA graph of kGraphRounds rounds), replayed on gstream
   bool use_graphs = true;
   cudaStream_t gstream = nullptr;
@@ -793,6 +793,7 @@ int pool_run(gesmc_pool_t p, uint64_t rounds) {
       done += r;
     }
   } else if (p->fused_ctas && !p->profiling) {
+    if (cudaMemsetAsync(&a.ctl->clean, 0, sizeof(uint32_t), s) != cudaSuccess) return GESMC_E_CUDA;
     // one cooperative launch per round, replayed from a captured graph when
     // the driver captures it (else launched directly)
     if (p->use_graphs && !p->fused_graph_refused &&
@@ -940,8 +941,8 @@ int pool_run(gesmc_pool_t p, uint64_t rounds) {
   p->switches_run += rounds * sw;
   const int rc = map_device_errors(ctl.err);
   if (rc != GESMC_OK) p->broken = rc;
-  // rounds that needed more than one wave: run that many on the whole GPU from now on
-  const uint32_t want = ctl.waves > 1 ? std::min<uint32_t>(ctl.waves - 1, kMaxWaveKernels) : 0u;
+  // waves after the first that many switches entered: run as many on the whole GPU from now on
+  const uint32_t want = std::min<uint32_t>(ctl.wide, kMaxWaveKernels);
   if (rc == GESMC_OK && want > p->wave_kernels) {
     p->wave_kernels = want;
     refresh_args(p);

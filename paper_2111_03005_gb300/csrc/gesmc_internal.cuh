@@ -83,9 +83,9 @@ constexpr uint32_t kErrTableFull = 1u, kErrBucket = 2u, kErrWaveCap = 4u, kErrNo
                    kErrGroup = 32u, kErrCopy = 64u, kErrGridSync = 128u;
 
 // Polls of the one-launch round's grid barrier before a CTA gives up (sets
-// kErrGridSync and leaves the kernel); each poll sleeps about 64 ns, so the
-// wait is bounded at about a second.
-constexpr uint32_t kGridWaitPolls = 1u << 24;
+// kErrGridSync and leaves the kernel); each poll is an access to L2 of half a
+// microsecond or more, so the wait is bounded at about a second.
+constexpr uint32_t kGridWaitPolls = 1u << 21;
 
 // Polls of an mbarrier before a kernel gives up on a bulk copy (sets
 // kErrCopy and returns instead of waiting on).
@@ -97,9 +97,10 @@ constexpr uint32_t kCopyWaitPolls = 1u << 22;
 // The cap bounds the time a faulty input or build can spend in one round.
 constexpr uint32_t kDefaultWaveCap = 10000;
 
-// Waves after the first run on the whole GPU as pairs of kernels (register,
-// decide), as many pairs as the pool's rounds have needed so far, at most
-// kMaxWaveKernels; k_tail runs any remaining waves on one CTA.
+// Waves after the first that many switches enter run on the whole GPU as pairs
+// of kernels (register, decide), as many pairs as the pool's rounds have
+// needed so far, at most kMaxWaveKernels; k_tail runs the other waves on one
+// CTA.
 constexpr uint32_t kMaxWaveKernels = 8;
 
 // Permutation buckets: a chain's positions go to 2^B buckets by the top B
@@ -167,6 +168,10 @@ struct Counters {
   // launches of the same CTA count (each launch leaves it at a multiple of
   // its CTA count; the host zeroes it when the count changes)
   unsigned long long gbar_arrived;
+  // the last one-launch round left the arrays that a round counts in cleared
+  // (the host zeroes it before a call's first round)
+  uint32_t clean;
+  uint32_t wide;  // waves of the round that more than kSoloPending switches entered
 };
 
 // Device-resident statistics, accumulated over rounds (all chains).

@@ -198,14 +198,13 @@ __device__ __forceinline__ bool decided_before(uint32_t st, uint32_t wave) {
 // Algorithm 1's test of one target edge of switch k in wave `wave` >= 2,
 // from its dependency entry (p, q): kBad if the edge exists when k runs,
 // kOk if it certainly does not, kWait if that depends on an undecided switch.
-__device__ __forceinline__ int check_target(const RoundArgs &a, uint32_t k, uint32_t d, uint32_t wave) {
-  if (d == kTrivial) return kOk;
-  const uint2 pq = __ldcg(&a.dep[d]);
-  const uint32_t p = pq.x, q = pq.y;
+// The test, given the entry and the statuses of the eraser p and of the
+// smallest inserter q (looked at only where they come before k).
+__device__ __forceinline__ int judge_target(uint32_t k, uint32_t p, uint32_t q, uint32_t sp, uint32_t sq,
+                                            uint32_t wave) {
   int res = kOk;
   if (p != kPNone) {             // the edge is in E at the start of the round
     if (p >= k) return kBad;     // erased later than k, or never
-    const uint32_t sp = __ldcg(&a.status[p]);
     if (decided_before(sp, wave)) {
       if ((sp & 3u) == kIllegal) return kBad;  // its eraser failed: still there
     } else {
@@ -213,13 +212,18 @@ __device__ __forceinline__ int check_target(const RoundArgs &a, uint32_t k, uint
     }
   }
   if (q != k) {
-    if (q < k) {                 // an earlier switch may insert it first
-      const uint32_t sq = __ldcg(&a.status[q]);
-      if (decided_before(sq, wave) && (sq & 3u) == kLegal) return kBad;
-    }
+    // an earlier switch may insert it first
+    if (q < k && decided_before(sq, wave) && (sq & 3u) == kLegal) return kBad;
     res = kWait;                 // q undecided, illegal but not yet replaced, or being replaced
   }
   return res;
+}
+
+__device__ __forceinline__ int check_target(const RoundArgs &a, uint32_t k, uint32_t d, uint32_t wave) {
+  if (d == kTrivial) return kOk;
+  const uint2 pq = __ldcg(&a.dep[d]);
+  return judge_target(k, pq.x, pq.y, pq.x < k ? __ldcg(&a.status[pq.x]) : 0u,
+                      pq.y < k ? __ldcg(&a.status[pq.y]) : 0u, wave);
 }
 
 struct Tally {
@@ -289,7 +293,7 @@ __device__ __forceinline__ void append_if(bool take, uint32_t k, uint32_t *list,
 
 // ---------------------------------------------------------------- kernels
 
-__device__ __forceinline__ void clear_body(const RoundArgs &a) {
+__device__ __forceinline__ void clear_arrays(const RoundArgs &a) {
   const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
   for (uint32_t b = tid; b < a.bucket_hw; b += nth) a.pcount[b] = 0;
   for (uint32_t p = tid; p < a.part_hw; p += nth) a.ocount[p] = 0;
@@ -299,17 +303,20 @@ __device__ __forceinline__ void clear_body(const RoundArgs &a) {
     uint4 *const f = reinterpret_cast<uint4 *>(a.tfilter);
     for (uint32_t w = tid; w <= (a.tfilter_mask >> 7); w += nth) f[w] = make_uint4(0, 0, 0, 0);
   }
-  if (tid == 0) {
-    a.ctl->pending[0] = 0;
-    a.ctl->pending[1] = 0;
-    a.ctl->boundary = 0;
-    a.ctl->waves = 0;
-    a.ctl->dep_count = 0;
-    a.ctl->ovf_count = 0;
-    a.ctl->cur = 0;
-    a.ctl->wave_next = 2;
-    a.ctl->wave_blocks = 0;
-  }
+}
+
+// One thread.
+__device__ __forceinline__ void clear_counters(Counters *ctl) {
+  ctl->pending[0] = 0;
+  ctl->pending[1] = 0;
+  ctl->boundary = 0;
+  ctl->waves = 0;
+  ctl->dep_count = 0;
+  ctl->ovf_count = 0;
+  ctl->cur = 0;
+  ctl->wave_next = 2;
+  ctl->wave_blocks = 0;
+  ctl->wide = 0;
 }
 
 // The kernels of a round follow one another by programmatic dependent launch:
@@ -324,7 +331,8 @@ __device__ __forceinline__ void clear_body(const RoundArgs &a) {
 __global__ void k_clear(RoundArgs a) {
   dep_launch();
   dep_wait();
-  clear_body(a);
+  clear_arrays(a);
+  if (blockIdx.x == 0 && threadIdx.x == 0) clear_counters(a.ctl);
 }
 
 __device__ __forceinline__ void store_record(const RoundArgs &a, uint32_t b, uint32_t idx, uint32_t keybits,
@@ -735,6 +743,10 @@ struct SortSmem {
   uint32_t *hist;    // one counter per sub-bucket (as many as the bucket has room for records)
   uint32_t *warp_tot;
   unsigned long long *bar;
+  // the one-launch round's straddling pairs (second bucket, first slot) of the
+  // buckets sorted so far
+  uint2 *meet = nullptr;
+  uint32_t *meets = nullptr;
 };
 
 // Shared memory of a sort of buckets with room for 2^log2 records (the
@@ -752,8 +764,10 @@ constexpr size_t sort_smem_bytes(uint32_t log2) {
 // the switches of all pairs of consecutive slots inside the bucket are
 // built.  Returns false (with kErrCopy set) if the copy did not land in time;
 // the caller must stop then.  Every thread of the CTA calls it; `parity`
-// tracks the barrier's phase across the buckets a CTA sorts.
-template <int kThreads, int kLog2>
+// tracks the barrier's phase across the buckets a CTA sorts.  A pair that
+// straddles two buckets is listed for k_boundary, or (kMeet, the one-launch
+// round, where that stage would cost a grid barrier) for meet_pairs.
+template <int kThreads, int kLog2, bool kMeet = false>
 __device__ __forceinline__ bool sort_bucket(const RoundArgs &a, uint32_t b, const SortSmem &sm, uint32_t &parity,
                                             bool local_offsets = false) {
   constexpr uint32_t kCap = 1u << kLog2;
@@ -864,9 +878,17 @@ __device__ __forceinline__ bool sort_bucket(const RoundArgs &a, uint32_t b, cons
       const uint4 r = srec[sidx[t]];
       a.cpos[goff + t] = r.y;
       a.cedge[goff + t] = ((unsigned long long)r.w << 32) | r.z;
+      if (kMeet && (tid == 0 || loff + cnt < ch.m)) {
+        // the bucket with the pair's second slot (there is one unless a bucket
+        // overflowed, which was reported), and the pair's first slot
+        const uint32_t end = ch.bucket_base + (1u << ch.B);
+        uint32_t second = b;
+        if (tid == 1) do { ++second; } while (second < end && a.pcount[second] == 0);
+        if (second < end) sm.meet[atomicAdd(sm.meets, 1u)] = make_uint2(second, tid == 0 ? goff - 1 : goff + t);
+      }
     }
   }
-  if (tid == 0 && t0 == 1 && cnt > 0) {
+  if (!kMeet && tid == 0 && t0 == 1 && cnt > 0) {
     // this bucket's first slot is the second of a pair started in an
     // earlier bucket: k_boundary builds that switch from the list
     const uint32_t idx = atomicAdd(&a.ctl->boundary, 1u);
@@ -874,6 +896,31 @@ __device__ __forceinline__ bool sort_bucket(const RoundArgs &a, uint32_t b, cons
   }
   __syncthreads();  // the CTA's shared memory may take the next bucket's copy
   return true;
+}
+
+// The straddling pairs a CTA of the one-launch round has a slot of: the later
+// of a pair's two CTAs to get here, which the count bnd[second bucket] tells,
+// builds it, both slots being written then.  Every thread of the CTA calls it.
+constexpr uint32_t kMeets = 256;
+__device__ __forceinline__ void meet_pairs(const RoundArgs &a, const SortSmem &sm) {
+  __syncthreads();
+  const uint32_t n = *sm.meets;
+  for (uint32_t x = threadIdx.x; x < n; x += blockDim.x) {
+    const uint32_t second = sm.meet[x].x, g = sm.meet[x].y;
+    __threadfence();
+    if (atomicAdd(&a.bnd[second], 1u) == 0) continue;
+    __threadfence();
+    const uint32_t c = a.owner_bucket[second];
+    const ChainDesc ch = a.chains[c];
+    const bool valid[1] = {true};
+    const uint32_t k[1] = {(g - ch.slot_base) >> 1}, i[1] = {__ldcg(&a.cpos[g])}, j[1] = {__ldcg(&a.cpos[g + 1])};
+    const unsigned long long e1[1] = {__ldcg(&a.cedge[g])}, e2[1] = {__ldcg(&a.cedge[g + 1])};
+    build_switches<1>(a, ch, chain_round(ch, a.ctl->pool_round), ch.exact_ell ? a.chain_ell[c] : 0u, valid, k, i, e1,
+                      j, e2);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) *sm.meets = 0;
+  __syncthreads();
 }
 
 // One CTA per bucket (the round's launch over all buckets): buckets with
@@ -1342,17 +1389,97 @@ __device__ __forceinline__ uint32_t wave_cap(const RoundArgs &a) {
   return a.max_waves ? a.max_waves : kDefaultWaveCap;
 }
 
+// Waves from `wave` on over the n <= kSoloPending undecided switches of `in`,
+// by one CTA of T threads (every thread calls it).  A switch stays with its
+// thread, with its dependency entries and their erasers, until it is decided,
+// so that a wave is a registration, two dependent accesses to L2 (the smallest
+// inserters, then their statuses) and a decision: about 1.8 us, where the same
+// from a list in memory took 5.7 us and a pair of whole-GPU kernels 6.  Returns
+// the number after the last wave.
+constexpr uint32_t kSoloPending = 2048;
+
+template <int T>
+__device__ __forceinline__ uint32_t solo_waves(const RoundArgs &a, const uint32_t *in, uint32_t n, uint32_t wave) {
+  constexpr int R = (int)kSoloPending / T;
+  const uint32_t tid = threadIdx.x;
+  Tally t;
+  ChainCount cc;
+  uint32_t k[R], live = 0, prev_n = n + 1;
+  uint2 d[R], p[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    if (tid + r * T >= n) continue;
+    live |= 1u << r;
+    k[r] = __ldcg(&in[tid + r * T]);
+    d[r] = __ldcg(&a.sw[k[r]]);
+    p[r].x = d[r].x != kTrivial ? __ldcg(&a.dep[d[r].x].x) : kPNone;
+    p[r].y = d[r].y != kTrivial ? __ldcg(&a.dep[d[r].y].x) : kPNone;
+  }
+  while (n != 0) {
+    if (wave > wave_cap(a)) {
+      if (tid == 0) atomicOr(&a.ctl->err, kErrWaveCap);
+      break;
+    }
+    if (n >= prev_n) {  // no switch was decided in the last wave: impossible
+      if (tid == 0) atomicOr(&a.ctl->err, kErrNoProgress);
+      break;
+    }
+    prev_n = n;
+    if (tid == 0 && wave < kWaveHist) a.st->last_pending[wave] = n;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      if (!((live >> r) & 1u)) continue;
+      if (d[r].x != kTrivial) atomicMin(&a.dep[d[r].x].y, k[r]);
+      if (d[r].y != kTrivial) atomicMin(&a.dep[d[r].y].y, k[r]);
+    }
+    __syncthreads();
+    uint32_t left = live;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      if (!((live >> r) & 1u)) continue;
+      // the inserters and the erasers' statuses first, then the inserters'
+      const bool x = d[r].x != kTrivial, y = d[r].y != kTrivial;
+      const uint32_t qx = x ? __ldcg(&a.dep[d[r].x].y) : k[r], qy = y ? __ldcg(&a.dep[d[r].y].y) : k[r];
+      const uint32_t ex = p[r].x < k[r] ? __ldcg(&a.status[p[r].x]) : 0u;
+      const uint32_t ey = p[r].y < k[r] ? __ldcg(&a.status[p[r].y]) : 0u;
+      const uint32_t ix = qx < k[r] ? __ldcg(&a.status[qx]) : 0u, iy = qy < k[r] ? __ldcg(&a.status[qy]) : 0u;
+      const int r3 = x ? judge_target(k[r], p[r].x, qx, ex, ix, wave) : kOk;
+      const int r4 = y ? judge_target(k[r], p[r].y, qy, ey, iy, wave) : kOk;
+      if (r3 == kBad || r4 == kBad) {
+        a.status[k[r]] = (wave << 2) | kIllegal;
+        if (x && qx == k[r]) atomicCAS(&a.dep[d[r].x].y, k[r], kQNone);  // no longer an inserter
+        if (y && qy == k[r]) atomicCAS(&a.dep[d[r].y].y, k[r], kQNone);
+        ++t.rej_exists;
+        left &= ~(1u << r);
+      } else if (r3 == kOk && r4 == kOk) {
+        a.status[k[r]] = (wave << 2) | kLegal;
+        ++t.accepted;
+        count_accepted(a, cc, a.owner_switch[k[r]]);
+        left &= ~(1u << r);
+      }
+    }
+    live = left;
+    n = 0;
+#pragma unroll
+    for (int r = 0; r < R; ++r) n += __syncthreads_count((live >> r) & 1u);
+    ++wave;
+  }
+  flush_tally(a, t);
+  flush_count(a, cc);
+  return wave;
+}
+
 // One wave after the first, on the whole GPU.  Registration: every
 // undecided switch becomes an inserter of its targets again (the q fields
 // of illegal minima were cleared); also empties the list of the next wave.
-// Nothing to do once no switch is undecided, or past the wave cap (k_tail
-// reports that).
+// Nothing to do once few switches are undecided (k_tail takes those), or past
+// the wave cap (k_tail reports that).
 __global__ void k_wave_register(RoundArgs a) {
   dep_launch();
   dep_wait();
   const uint32_t cur = a.ctl->cur, wave = a.ctl->wave_next;
   const uint32_t n = a.ctl->pending[cur];
-  if (n == 0 || wave > wave_cap(a)) return;
+  if (n <= kSoloPending || wave > wave_cap(a)) return;
   const uint32_t *in = cur ? a.list1 : a.list0;
   for (uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x; idx < n; idx += gridDim.x * blockDim.x) {
     const uint32_t k = in[idx];
@@ -1376,7 +1503,7 @@ __global__ void k_wave_decide(RoundArgs a) {
   const uint32_t cur = a.ctl->cur, wave = a.ctl->wave_next;
   const uint32_t n = a.ctl->pending[cur];
   const uint32_t active = min(gridDim.x, (n + blockDim.x - 1) / blockDim.x);  // CTAs with a switch
-  if (blockIdx.x >= active || wave > wave_cap(a)) return;
+  if (n <= kSoloPending || blockIdx.x >= active || wave > wave_cap(a)) return;
   Tally t;
   ChainCount cc;
   const uint32_t *in = cur ? a.list1 : a.list0;
@@ -1415,6 +1542,7 @@ __global__ void k_wave_decide(RoundArgs a) {
     a.ctl->wave_blocks = 0;
     a.ctl->cur = cur ^ 1;
     a.ctl->wave_next = wave + 1;
+    a.ctl->wide += 1;
   }
 }
 
@@ -1451,10 +1579,10 @@ __device__ __forceinline__ void close_round(const RoundArgs &a, uint32_t wave) {
   }
 }
 
-// Waves 2, 3, ... on one CTA: undecided switches re-register as inserters
-// (the q fields of illegal minima were cleared), then decide.  The kernel
-// also closes the pool round (the round counter every chain derives its own
-// round number from).
+// The remaining waves, on one CTA: from a list as the pairs of wave kernels do
+// while many switches are undecided (waves that the pool's rounds have not
+// needed before), then solo_waves.  The kernel also closes the pool round (the
+// round counter every chain derives its own round number from).
 __global__ void __launch_bounds__(1024) k_tail(RoundArgs a) {
   __shared__ uint32_t s_n;
   dep_launch();
@@ -1468,7 +1596,10 @@ __global__ void __launch_bounds__(1024) k_tail(RoundArgs a) {
     if (threadIdx.x == 0) s_n = pend[cur];
     __syncthreads();
     const uint32_t n = s_n;
-    if (n == 0) break;
+    if (n <= kSoloPending) {
+      if (n) wave = solo_waves<1024>(a, cur ? a.list1 : a.list0, n, wave);
+      break;
+    }
     if (wave > wave_cap(a)) {
       if (threadIdx.x == 0) atomicOr(&a.ctl->err, kErrWaveCap);
       break;
@@ -1516,6 +1647,7 @@ __global__ void __launch_bounds__(1024) k_tail(RoundArgs a) {
     }
     cur ^= 1;
     ++wave;
+    if (threadIdx.x == 0) a.ctl->wide += 1;
   }
   if (prev_n <= a.switch_hw) {  // some waves ran here
     flush_tally(a, t);
@@ -1532,7 +1664,7 @@ __global__ void __launch_bounds__(1024) k_tail(RoundArgs a) {
 // at this barrier, i.e. the count has reached `target`, which every thread
 // advances by the CTA count per barrier.  With the CTA barriers on both
 // sides, every write before the barrier is visible after it.  The wait is
-// bounded (kGridWaitPolls): a CTA that gives up sets kErrGridSync and
+// bounded (kGridWaitPolls, each an access to L2): a CTA that gives up sets kErrGridSync and
 // returns false, and its caller leaves the kernel; the other CTAs see the
 // error bit while they wait and leave too.
 __device__ __forceinline__ bool grid_sync(Counters *ctl, unsigned long long &target) {
@@ -1546,7 +1678,6 @@ __device__ __forceinline__ bool grid_sync(Counters *ctl, unsigned long long &tar
     uint32_t it = 0;
     while (v < target && it < kGridWaitPolls) {
       if (*(volatile uint32_t *)&ctl->err & kErrGridSync) break;
-      __nanosleep(20);
       asm volatile("ld.acquire.gpu.u64 %0, [%1];" : "=l"(v) : "l"(&ctl->gbar_arrived) : "memory");
       ++it;
     }
@@ -1605,8 +1736,14 @@ __device__ __forceinline__ uint32_t cta_scan_full(const uint32_t *count, uint32_
 // spread over the launch's CTAs, with a grid barrier where the multi-kernel
 // round has a kernel boundary.  The offset scans run on CTA 0 (the pools this
 // launch is for have few buckets and partitions), and the waves after the
-// first repeat register / decide until no switch is undecided.  The shared
-// memory holds the sort's arrays and, later, the grouping table.
+// first repeat register / decide until no switch is undecided, on CTA 0 alone
+// once they are few.  The shared memory holds the sort's arrays and, later, the
+// grouping table.  What bounds it: a grid barrier is about 1.5 us, a stage of a
+// small chain a few dependent accesses to L2.  The arrays a round counts in
+// are cleared by the round before (ctl->clean; the first round of a call
+// clears its own), the straddling pairs are built in the sort and the last
+// waves take no grid barriers: five barriers a round for a chain of 10,000
+// edges where there were 13 to 17 (53 -> 44 us a round on 32 CTAs).
 __global__ void __launch_bounds__(kFusedThreads, 1) k_round_fused(RoundArgs a) {
   extern __shared__ __align__(128) uint4 fused_dyn[];
   const uint32_t tid = threadIdx.x;
@@ -1627,8 +1764,12 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_round_fused(RoundArgs a) {
   }
   __syncthreads();
   unsigned long long target = start_count;
-  clear_body(a);
-  if (!grid_sync(ctl, target)) return;
+  if (!*(volatile uint32_t *)&ctl->clean) {
+    clear_arrays(a);
+    for (uint32_t b = gtid; b < a.bucket_hw; b += nth) a.bnd[b] = 0;
+    if (gtid == 0) clear_counters(ctl);
+    if (!grid_sync(ctl, target)) return;
+  }
   uint32_t wave = 2;
   if (a.any_work) {
     if (a.any_exact) {
@@ -1654,20 +1795,27 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_round_fused(RoundArgs a) {
       sm.sidx = reinterpret_cast<uint16_t *>(sm.hist + room);
       sm.warp_tot = reinterpret_cast<uint32_t *>(sm.sidx + room);
       sm.bar = reinterpret_cast<unsigned long long *>(sm.warp_tot + 32);
-      if (tid == 0) mbar_init(sm.bar, 1);
+      __shared__ uint2 meet[kMeets];
+      __shared__ uint32_t meets;
+      sm.meet = meet;
+      sm.meets = &meets;
+      if (tid == 0) {
+        mbar_init(sm.bar, 1);
+        meets = 0;
+      }
       __syncthreads();
       uint32_t parity = 0;
       const bool local = a.fused_local_offsets != 0;
-      for (uint32_t b = blockIdx.x; b < a.bucket_hw; b += gridDim.x)
+      for (uint32_t b = blockIdx.x; b < a.bucket_hw; b += gridDim.x) {
         if (!(a.bucket_log2 == kBucketLog2Small
-                  ? sort_bucket<kFusedThreads, kBucketLog2Small>(a, b, sm, parity, local)
-                  : sort_bucket<kFusedThreads, kBucketLog2Large>(a, b, sm, parity, local)))
+                  ? sort_bucket<kFusedThreads, kBucketLog2Small, true>(a, b, sm, parity, local)
+                  : sort_bucket<kFusedThreads, kBucketLog2Large, true>(a, b, sm, parity, local)))
           return;
-      __syncthreads();
+        if (meets > kMeets - 2) meet_pairs(a, sm);  // (the same for every thread: read after a barrier)
+      }
+      meet_pairs(a, sm);
       if (tid == 0) mbar_inval(sm.bar);  // the grouping table takes these bytes next
     }
-    if (!grid_sync(ctl, target)) return;
-    boundary_body(a);
     if (!grid_sync(ctl, target)) return;
     const uint32_t npair = a.slot_hw >> 1;
     for (uint32_t base = blockIdx.x * 2 * blockDim.x; base < npair; base += 2 * nth) {
@@ -1691,15 +1839,22 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_round_fused(RoundArgs a) {
     group_body<kFusedThreads, 2048 / kFusedThreads>(a);
     if (!grid_sync(ctl, target)) return;
     wave1_body(a);
+    // what the stages so far counted in is not needed any more
+    clear_arrays(a);
+    for (uint32_t b = gtid; b < a.bucket_hw; b += nth) a.bnd[b] = 0;
     if (!grid_sync(ctl, target)) return;
-    // waves 2, 3, ...: undecided switches re-register as inserters, then decide
+    // waves 2, 3, ...: undecided switches re-register as inserters, then
+    // decide; from kSoloPending undecided switches on by CTA 0 alone
     Tally t;
     ChainCount cc;
     uint32_t cur = 0, prev_n = a.switch_hw + 1;
     volatile uint32_t *pend = ctl->pending;
     for (;;) {
       const uint32_t n = pend[cur];  // the same for every thread: read after a barrier
-      if (n == 0) break;
+      if (n <= kSoloPending) {
+        if (n && blockIdx.x == 0) wave = solo_waves<kFusedThreads>(a, cur ? a.list1 : a.list0, n, wave);
+        break;
+      }
       if (wave > wave_cap(a)) {
         if (gtid == 0) atomicOr(&ctl->err, kErrWaveCap);
         break;
@@ -1712,7 +1867,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_round_fused(RoundArgs a) {
       const uint32_t *in = cur ? a.list1 : a.list0;
       uint32_t *out = cur ? a.list0 : a.list1;
       for (uint32_t idx = gtid; idx < n; idx += nth) {
-        const uint32_t k = in[idx];
+        const uint32_t k = __ldcg(&in[idx]);
         const uint2 sv = __ldcg(&a.sw[k]);
         if (sv.x != kTrivial) atomicMin(&a.dep[sv.x].y, k);
         if (sv.y != kTrivial) atomicMin(&a.dep[sv.y].y, k);
@@ -1727,7 +1882,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_round_fused(RoundArgs a) {
         bool wait = false;
         uint32_t k = 0;
         if (idx < n) {
-          k = in[idx];
+          k = __ldcg(&in[idx]);
           const uint2 sv = __ldcg(&a.sw[k]);
           const int r3 = check_target(a, k, sv.x, wave);
           const int r4 = check_target(a, k, sv.y, wave);
@@ -1752,7 +1907,17 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_round_fused(RoundArgs a) {
     flush_tally(a, t);
     flush_count(a, cc);
   }
-  if (blockIdx.x == 0) close_round(a, wave);
+  if (blockIdx.x == 0) {
+    __syncthreads();  // CTA 0's threads have read the counters
+    close_round(a, wave);
+    __syncthreads();
+    if (tid == 0) {
+      const uint32_t waves = ctl->waves;
+      clear_counters(ctl);
+      ctl->waves = waves;  // (the host reads it)
+      ctl->clean = a.any_work;
+    }
+  }
 }
 
 // ---------------------------------------------------------------- state in / out

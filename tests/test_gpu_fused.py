@@ -109,3 +109,38 @@ def test_one_launch_rounds_replayed_or_launched_directly(graphs):
         c.run(2, 5)
         assert np.array_equal(c.edges(), want)
         assert c.stats()["kernel_launches"] == 9
+
+
+@pytest.mark.parametrize("ctas", [1, 3, 32, 152])
+@pytest.mark.parametrize("m", [513, 1024, 5001, 70_000])
+def test_pairs_that_straddle_buckets_on_different_ctas(ctas, m):
+    # a straddling pair is built by the later of its two CTAs; one CTA has both
+    # sides of every pair, more CTAs than buckets never have more than one
+    edges = inputs.gnp(m, 2.4 / (m - 1), seed=m)
+    edges = np.random.default_rng(m).permutation(edges)[:m]
+    with gesmc.Chain(edges, n=m) as c:
+        c.set_round_launch(ctas)
+        c.run(3, 21)
+        c.run(2, 21)
+        got, st = c.edges(), c.stats()
+    want, want_st = oracle.run(edges, seed=21, rounds=5)
+    assert np.array_equal(got, want)
+    assert st["accepted"] == want_st["accepted"] and st["rejected_exists"] == want_st["rejected_exists"]
+
+
+@pytest.mark.parametrize("ctas", [0, 8])
+@pytest.mark.parametrize("k", [4200, 10500, 20000])
+def test_waves_on_both_sides_of_the_single_cta_limit(ctas, k):
+    # hubs in a small node set: second waves of a few hundred to several
+    # thousand switches, above and below what one CTA takes
+    edges = inputs.pld_graph(k, 2.01, 1, k // 10, seed=23)
+    want, want_w, want_ent = oracle.run_rounds(edges, seed=4, rounds=3)
+    with gesmc.Chain(edges, n=k) as c:
+        if ctas:
+            c.set_round_launch(ctas)
+        for r in range(3):
+            c.run(1, 4)
+            pend = c.stats()["last_round_pending"]
+            for v in range(2, int(want_w[r]) + 1):
+                assert pend[v] == want_ent[r][v], (r, v)
+        assert np.array_equal(c.edges(), want)
