@@ -57,6 +57,18 @@ bool chain_shape(uint64_t m, uint32_t tuple_log2, uint32_t bucket_log2, ChainSha
   return true;
 }
 
+// Layout where the caller leaves it open.  Pools of many chains and large
+// chains run partitions of 2^11 tuples on tables of 2^12 slots: half the
+// cursors for the sort to append to, and two tuples a thread for the grouping
+// (ms per round against 2^10 and 2^11: 11.14 / 12.20 for one chain of 1.3e8
+// edges, 2.46 / 2.61 for 3.4e7, 0.73 / 0.80 for 256 mixed chains of 9e6 edges,
+// 0.244 / 0.263 for 1024 small ones).  Single chains of up to 2^24 edges keep
+// 2^10 and 2^11 (0.661 / 0.655 for 8e6 edges, 0.066 / 0.064 for 5,000).
+constexpr uint64_t kWideLayoutEdges = 1ull << 24;
+bool wide_layout(uint64_t M, uint64_t C) { return C > 1 || M > kWideLayoutEdges; }
+uint32_t default_tuple_log2(uint64_t M, uint64_t C) { return wide_layout(M, C) ? 11 : kDefaultTupleLog2; }
+uint32_t default_group_log2(uint64_t M, uint64_t C) { return wide_layout(M, C) ? 12 : kDefaultGroupLog2; }
+
 // Capacities of a pool's index spaces for at most M edges in at most C
 // chains; each bound holds for any split of the edges into chains.
 struct Capacity {
@@ -464,7 +476,9 @@ int pool_init(gesmc_pool_t p, const gesmc_pool_opts &o) {
     a.dep_cap = std::min<uint32_t>(a.dep_cap, 16u);
   }
   a.max_waves = o.max_waves;
-  a.group_log2 = o.group_log2 ? o.group_log2 : kDefaultGroupLog2;
+  a.group_log2 = o.group_log2   ? o.group_log2
+                 : o.tuple_log2 ? kDefaultGroupLog2
+                                : default_group_log2(p->max_edges, p->max_chains);
   LaunchShapes shapes;
   if (prepare_kernels(a.group_log2, p->num_sms, &shapes) != cudaSuccess) {
     cudaGetLastError();
@@ -1083,7 +1097,7 @@ void gesmc_pool_opts_default(gesmc_pool_opts *o) {
 
 size_t gesmc_pool_device_bytes(uint64_t max_edges, uint32_t max_chains, uint32_t tuple_log2) {
   if (max_edges > kMaxEdges || max_chains == 0) return 0;
-  if (!tuple_log2) tuple_log2 = kDefaultTupleLog2;
+  if (!tuple_log2) tuple_log2 = default_tuple_log2(max_edges, max_chains);
   const Capacity c = pool_capacity(max_edges, max_chains, tuple_log2);
   return capacity_fits(c) ? pool_layout(c, max_edges, max_chains).total : 0;
 }
@@ -1127,7 +1141,7 @@ int gesmc_pool_create(const gesmc_pool_opts *opts, gesmc_pool_t *out) {
   p->alloc_ctx = o.alloc_ctx;
   p->max_edges = o.max_edges;
   p->max_chains = o.max_chains;
-  p->tuple_log2 = o.tuple_log2 ? o.tuple_log2 : kDefaultTupleLog2;
+  p->tuple_log2 = o.tuple_log2 ? o.tuple_log2 : default_tuple_log2(p->max_edges, p->max_chains);
   p->use_graphs = !(o.flags & GESMC_FLAG_NO_GRAPHS);
   p->verify_rounds = (o.flags & GESMC_FLAG_VERIFY_ROUNDS) != 0;
   p->cap = pool_capacity(p->max_edges, p->max_chains, p->tuple_log2);
@@ -1573,7 +1587,7 @@ extern "C" int gesmc_run_noalloc(uint64_t *edges, uint64_t m, uint64_t n, uint64
   p.stream = (cudaStream_t)stream;
   p.max_edges = GESMC_NOALLOC_MAX_EDGES;
   p.max_chains = 1;
-  p.tuple_log2 = kDefaultTupleLog2;
+  p.tuple_log2 = default_tuple_log2(p.max_edges, 1);
   p.cap = pool_capacity(p.max_edges, 1, p.tuple_log2);
   p.lay = pool_layout(p.cap, p.max_edges, 1);
   if (p.lay.total > GESMC_NOALLOC_SCRATCH_BYTES) return GESMC_E_INTERNAL;

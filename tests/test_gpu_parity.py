@@ -372,3 +372,19 @@ def test_scatter_variants_at_their_limits(m):
     edges = np.random.default_rng(m).permutation(edges)[:m]
     assert len(edges) == m
     run_and_compare(edges, n, seed=3, rounds=2)
+
+
+@pytest.mark.slow
+def test_large_lists_are_read_out_in_two_passes():
+    # just above the size from which the list is binned by position on the way
+    # out; odd, so that the last slot has no partner
+    m, n = (1 << 24) + 1, 1 << 21
+    edges = np.random.default_rng(5).permutation(inputs.gnp(n, (m + 40_000) / (n * (n - 1) / 2), seed=5))[:m]
+    assert len(edges) == m
+    with gesmc.Chain(edges, n=n) as c:
+        assert first_diff(c.edges(), edges) < 0
+        c.run(1, 3)
+        got = c.edges()
+        out = torch.empty(m, dtype=torch.int64, device="cuda")
+        assert np.array_equal(c.edges(out).cpu().numpy().view(np.uint64), got)
+    assert first_diff(got, oracle.run(edges, seed=3, rounds=1)[0]) < 0
