@@ -57,17 +57,14 @@ bool chain_shape(uint64_t m, uint32_t tuple_log2, uint32_t bucket_log2, ChainSha
   return true;
 }
 
-// Layout where the caller leaves it open.  Pools of many chains and large
-// chains run partitions of 2^11 tuples on tables of 2^12 slots: half the
-// cursors for the sort to append to, and two tuples a thread for the grouping
-// (ms per round against 2^10 and 2^11: 11.14 / 12.20 for one chain of 1.3e8
-// edges, 2.46 / 2.61 for 3.4e7, 0.73 / 0.80 for 256 mixed chains of 9e6 edges,
-// 0.244 / 0.263 for 1024 small ones).  Single chains of up to 2^24 edges keep
-// 2^10 and 2^11 (0.661 / 0.655 for 8e6 edges, 0.066 / 0.064 for 5,000).
-constexpr uint64_t kWideLayoutEdges = 1ull << 24;
-bool wide_layout(uint64_t M, uint64_t C) { return C > 1 || M > kWideLayoutEdges; }
-uint32_t default_tuple_log2(uint64_t M, uint64_t C) { return wide_layout(M, C) ? 11 : kDefaultTupleLog2; }
-uint32_t default_group_log2(uint64_t M, uint64_t C) { return wide_layout(M, C) ? 12 : kDefaultGroupLog2; }
+// Mean tuples per partition where the caller leaves it open: 2^11 for pools of
+// many chains and for single chains above 2^18 edges (half the cursors for the
+// sort to append to; ms per round against 2^10: 10.2 / 11.3 for 1.3e8 edges,
+// 2.25 / 2.40 for 3.4e7, 0.607 / 0.604 for 8e6, 0.119 / 0.122 for a power law of
+// 1e6, 0.67 / 0.71 for 256 mixed chains), 2^10 for smaller chains (0.043 / 0.041
+// for 5,000 edges: the more partitions, the more SMs have one).
+constexpr uint64_t kWideLayoutEdges = 1ull << 18;
+uint32_t default_tuple_log2(uint64_t M, uint64_t C) { return C > 1 || M > kWideLayoutEdges ? 11 : kDefaultTupleLog2; }
 
 // Capacities of a pool's index spaces for at most M edges in at most C
 // chains; each bound holds for any split of the edges into chains.
@@ -476,9 +473,7 @@ int pool_init(gesmc_pool_t p, const gesmc_pool_opts &o) {
     a.dep_cap = std::min<uint32_t>(a.dep_cap, 16u);
   }
   a.max_waves = o.max_waves;
-  a.group_log2 = o.group_log2   ? o.group_log2
-                 : o.tuple_log2 ? kDefaultGroupLog2
-                                : default_group_log2(p->max_edges, p->max_chains);
+  a.group_log2 = o.group_log2 ? o.group_log2 : kDefaultGroupLog2;
   LaunchShapes shapes;
   if (prepare_kernels(a.group_log2, p->num_sms, &shapes) != cudaSuccess) {
     cudaGetLastError();

@@ -118,12 +118,13 @@ inline uint32_t bucket_log2(unsigned long long max_edges) {
 
 // Tuple partitions: a chain's tuples go to 2^P partitions by the top P bits
 // of the hash of the edge id (about 2^tuple_log2 tuples each, room for
-// twice that); one CTA groups a partition by edge id in a shared-memory
-// table of 2^group_log2 slots of 20 bytes.
+// twice that); one CTA groups a partition by edge id, the few ids that may have
+// a dependency in a shared-memory table of 2^group_log2 slots of 20 bytes.
 constexpr int kDefaultTupleLog2 = 10;
-constexpr int kDefaultGroupLog2 = 11;
+constexpr int kDefaultGroupLog2 = 11;  // as many slots as a partition of the fast path has tuples
 constexpr int kMaxGroupLog2 = 13;
-constexpr int kGroupThreads = 1024;
+constexpr int kGroupThreads = 512;
+constexpr int kGroupMin = 3;  // CTAs per SM
 constexpr int kGroupSlotBytes = 20;
 
 constexpr int kWaveHist = 64;

@@ -1097,24 +1097,34 @@ __global__ void __launch_bounds__(256, 4) k_sources(RoundArgs a) {
 }
 
 // Grouping of one tuple partition by edge id (Algorithm 1's table T for the
-// partition's edge ids) in a shared-memory table of S slots: slot[s] =
-// {key lo, key hi, p, q} with p the eraser (from the source tuple) and q
-// the smallest inserter, and aux[s] = 1 once a second inserter arrives.
-// Then wave 1 for every target: present when k runs (p >= k), dependent on
-// an undecided switch (p < k, or an earlier inserter q < k), or free.  Edge
-// ids with a dependency get an entry {p, q} for the later waves, whose index
-// replaces aux[s].  Slots are probed from the low bits of the id's hash,
-// which the tuple carries.
+// partition's edge ids).  Most targets are proposed by no other switch and
+// equal no edge of the graph: two bitmaps over 15 bits of the ids' hashes tell
+// them.  Every target sets its bit of `seen`; a bit met twice, or met by a
+// source, is also set in `marked`; a target whose bit is not marked is free.
+// The other targets, and the sources that met a target's bit, go into a
+// shared-memory table of S slots: slot[s] = {key lo, key hi, p, q} with p the
+// eraser (from the source tuple) and q the smallest inserter, and aux[s] = 1
+// once a second inserter arrives.  Then wave 1 for each of these targets:
+// present when k runs (p >= k), dependent on an undecided switch (p < k, or an
+// earlier inserter q < k), or free.  Edge ids with a dependency get an entry
+// {p, q} for the later waves, whose index replaces aux[s].  Slots are probed
+// from the low bits of the id's hash, which the tuple carries; the bitmaps use
+// other bits of it.
 struct GroupSmem {
   uint4 *slot;
   uint32_t *aux;
+  uint32_t *seen, *marked;
 };
+
+constexpr uint32_t kGroupBitsLog2 = 15, kGroupWords = 1u << (kGroupBitsLog2 - 5);
 
 __device__ __forceinline__ GroupSmem group_smem(uint32_t S) {
   extern __shared__ uint4 group_dyn[];
   GroupSmem g;
   g.slot = group_dyn;
   g.aux = reinterpret_cast<uint32_t *>(group_dyn + S);
+  g.seen = g.aux + S;
+  g.marked = g.seen + kGroupWords;
   return g;
 }
 
@@ -1189,18 +1199,18 @@ __device__ __forceinline__ void group_decide(const RoundArgs &a, const GroupSmem
   }
 }
 
-// Tuples a thread holds in registers on the fast path: 2 in the grouping
-// kernel's 1024-thread CTAs (measured 7% faster than 4 in 512-thread CTAs:
-// fewer probe loops in a row per thread before each barrier), 4 in the
-// one-launch round's 512-thread CTAs; both take partitions of up to 2048
-// tuples on the fast path.
-constexpr int kGroupR = 2;
-
-// Persistent CTAs over the partitions.  Fast path: the partition's tuples
-// stay in registers, and each thread later visits and clears the slots it
-// claimed.  Partitions with more tuples than fit, or more distinct ids than
-// slots, take the sub-pass path: the ids whose hash bits 16.. select them,
-// split further until each sub-pass fits.
+// Persistent CTAs over the partitions.  Fast path: a thread keeps the hash
+// and the value of its (at most kR) tuples in registers, reads the ids of
+// those that go into the table again, and clears the slots it claimed.
+// Partitions with more tuples than that, or more distinct marked ids than
+// slots, take the sub-pass path, all tuples into the table: the ids whose hash
+// bits 16.. select them, split further until each sub-pass fits.
+//
+// What bounds it: the barriers and shared-memory latency of one partition
+// after another, about a third of it the wait for its tuples.  With every tuple
+// in a table of 64-bit keys, 1024-thread CTAs took 2.31 ms per round of G(2^24)
+// and 0.169 of 256 mixed chains; so, 512-thread CTAs, three per SM, take 1.47
+// and 0.123 (256 threads: 1.35, but the round 0.15 ms longer; 128: 2.84).
 // Bring the own tuples of partition `part` (if it exists and is owned) into
 // L2 with one bulk prefetch (the TMA engine), so that the CTA finds them
 // there when it gets to that partition.
@@ -1222,6 +1232,7 @@ __device__ __forceinline__ void group_body(const RoundArgs &a) {
   __shared__ uint32_t overflow;
   const int tid = threadIdx.x;
   for (uint32_t s = tid; s < S; s += T) group_reset_slot(g, s);
+  for (uint32_t w = tid; w < 2 * kGroupWords; w += T) g.seen[w] = 0;
   if (tid == 0) overflow = 0;
   dep_wait();  // (does nothing in the one-launch round)
   const bool ovf = a.ctl->ovf_count != 0;
@@ -1238,41 +1249,71 @@ __device__ __forceinline__ void group_body(const RoundArgs &a) {
     const uint32_t obeg = ovf ? overflow_offset(a, part) : 0, oend = ovf ? overflow_offset(a, part + 1) : 0;
     const uint32_t ntup = nprim + (oend - obeg);
     if (ntup <= (uint32_t)(R * T)) {
-      uint4 r[R];
-      uint32_t slot[R];
+      uint32_t h[R], v[R], todo = 0;  // todo: this thread's tuples that go into the table
 #pragma unroll
       for (int j = 0; j < R; ++j) {
         const uint32_t t = tid + j * T;
-        r[j] = make_uint4(0, 0, 0, 0);
-        if (t < ntup) r[j] = t < nprim ? __ldcs(&prim[t]) : a.stup[obeg + (t - nprim)];
-      }
-#pragma unroll
-      for (int j = 0; j < R; ++j) {
-        const uint32_t t = tid + j * T;
-        slot[j] = S;
+        v[j] = kTupleSource;
         if (t < ntup) {
-          slot[j] = group_insert(g, S, ((unsigned long long)r[j].y << 32) | r[j].x, r[j].w, r[j].z);
-          if (slot[j] == S) overflow = 1;
+          const uint2 zw = __ldcs(reinterpret_cast<const uint2 *>(t < nprim ? &prim[t] : &a.stup[obeg + (t - nprim)]) + 1);
+          v[j] = zw.x;
+          h[j] = zw.y;
+          if (!(zw.x & kTupleSource)) {
+            const uint32_t bit = h[j] >> (32 - kGroupBitsLog2), m = 1u << (bit & 31);
+            if (atomicOr(&g.seen[bit >> 5], m) & m) atomicOr(&g.marked[bit >> 5], m);
+          }
         }
-      }
-      __syncthreads();
-      const bool full = overflow != 0;
-      if (!full) {
-#pragma unroll
-        for (int j = 0; j < R; ++j)
-          if (slot[j] != S && (slot[j] & kClaimed)) group_alloc(a, g, slot[j] & ~kClaimed);
-        __syncthreads();
-#pragma unroll
-        for (int j = 0; j < R; ++j)
-          if (slot[j] != S && !(r[j].z & kTupleSource)) group_decide(a, g, slot[j] & ~kClaimed, r[j].z);
       }
       __syncthreads();
 #pragma unroll
       for (int j = 0; j < R; ++j)
-        if (slot[j] != S && (slot[j] & kClaimed)) group_reset_slot(g, slot[j] & ~kClaimed);
+        if (tid + j * T < ntup && (v[j] & kTupleSource)) {
+          const uint32_t bit = h[j] >> (32 - kGroupBitsLog2), m = 1u << (bit & 31);
+          if (g.seen[bit >> 5] & m) {
+            atomicOr(&g.marked[bit >> 5], m);
+            todo |= 1u << j;
+          }
+        }
+      __syncthreads();
+#pragma unroll
+      for (int j = 0; j < R; ++j)
+        if (!(v[j] & kTupleSource)) {
+          const uint32_t bit = h[j] >> (32 - kGroupBitsLog2);
+          if ((g.marked[bit >> 5] >> (bit & 31)) & 1u) todo |= 1u << j;
+        }
+      // h of a tuple that goes into the table becomes its slot
+#pragma unroll
+      for (int j = 0; j < R; ++j)
+        if ((todo >> j) & 1u) {
+          const uint32_t t = tid + j * T;
+          const uint2 id = *reinterpret_cast<const uint2 *>(t < nprim ? &prim[t] : &a.stup[obeg + (t - nprim)]);
+          h[j] = group_insert(g, S, ((unsigned long long)id.y << 32) | id.x, h[j], v[j]);
+          if (h[j] == S) {
+            overflow = 1;
+            todo &= ~(1u << j);
+          }
+        }
+      __syncthreads();
+      const bool full = overflow != 0;
+      for (uint32_t w = tid; w < 2 * kGroupWords / 4; w += T)  // both bitmaps
+        reinterpret_cast<uint4 *>(g.seen)[w] = make_uint4(0, 0, 0, 0);
+      if (!full) {
+#pragma unroll
+        for (int j = 0; j < R; ++j)
+          if (((todo >> j) & 1u) && (h[j] & kClaimed)) group_alloc(a, g, h[j] & ~kClaimed);
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < R; ++j)
+          if (((todo >> j) & 1u) && !(v[j] & kTupleSource)) group_decide(a, g, h[j] & ~kClaimed, v[j]);
+      }
+      __syncthreads();
+      // (the next partition's first table access comes two barriers later)
+#pragma unroll
+      for (int j = 0; j < R; ++j)
+        if (((todo >> j) & 1u) && (h[j] & kClaimed)) group_reset_slot(g, h[j] & ~kClaimed);
+      if (!full) continue;
       if (tid == 0) overflow = 0;
       __syncthreads();
-      if (!full) continue;
     }
     // sub-pass path
     if (tid == 0) {
@@ -1333,9 +1374,9 @@ __device__ __forceinline__ void group_body(const RoundArgs &a) {
   }
 }
 
-__global__ void __launch_bounds__(kGroupThreads, 2) k_group(RoundArgs a) {
+__global__ void __launch_bounds__(kGroupThreads, kGroupMin) k_group(RoundArgs a) {
   dep_launch();
-  group_body<kGroupThreads, kGroupR>(a);
+  group_body<kGroupThreads, 2048 / kGroupThreads>(a);
 }
 
 // Each CTA takes a contiguous range of switches, so that a thread's running
@@ -2142,7 +2183,7 @@ inline int grid_for(unsigned long long work, int threads, int num_sms, int per_s
 
 }  // namespace
 
-size_t group_smem_bytes(uint32_t group_log2) { return (size_t)kGroupSlotBytes << group_log2; }
+size_t group_smem_bytes(uint32_t group_log2) { return ((size_t)kGroupSlotBytes << group_log2) + 8 * kGroupWords; }
 
 cudaError_t prepare_kernels(uint32_t group_log2, int num_sms, LaunchShapes *shapes) {
   // opt in to the largest table any pool may use, so that pools with

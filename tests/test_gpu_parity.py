@@ -388,3 +388,12 @@ def test_large_lists_are_read_out_in_two_passes():
         out = torch.empty(m, dtype=torch.int64, device="cuda")
         assert np.array_equal(c.edges(out).cpu().numpy().view(np.uint64), got)
     assert first_diff(got, oracle.run(edges, seed=3, rounds=1)[0]) < 0
+
+
+@pytest.mark.parametrize("tuple_log2,group_log2", [(0, 0), (11, 10), (11, 11), (10, 10)])
+@pytest.mark.parametrize("n,m", [(200, 10_000), (300, 40_000), (3000, 40_001)])
+def test_grouping_with_few_and_many_marked_ids(n, m, tuple_log2, group_log2):
+    # dense graphs: nearly every target is an edge, so that a partition's marked
+    # ids outnumber the slots of a small table; sparse ones: few are marked
+    edges = inputs.random_simple_graph(n, m, seed=m + n)
+    run_and_compare(edges, n, seed=31, rounds=2, tuple_log2=tuple_log2, group_log2=group_log2)
