@@ -395,14 +395,17 @@ void refresh_args(gesmc_pool_t p) {
   a.fused_local_offsets = most_buckets <= kLocalOffsetBuckets ? 1u : 0u;
   a.permute_stride = spread ? coprime_stride(a.permute_ctas) : 1;
   a.sources_stride = spread ? coprime_stride(a.sources_ctas) : 1;
-  a.agg_chain = kNoChain;
+  a.agg_chain = a.solo_chain = kNoChain;
   a.agg_pairs = 0;
   if (p->live_chains == 1)
-    for (uint32_t c = 0; c < p->max_chains; ++c)
-      if (p->chains[c].live && p->chains[c].shape.m >= 2 && p->chains[c].shape.nb <= kAggBuckets) {
+    for (uint32_t c = 0; c < p->max_chains; ++c) {
+      if (!p->chains[c].live) continue;
+      a.solo_chain = c;
+      if (p->chains[c].shape.m >= 2 && p->chains[c].shape.nb <= kAggBuckets) {
         a.agg_chain = c;
         a.agg_pairs = (p->chains[c].shape.m + 1) / 2;
       }
+    }
 }
 
 // Point the round arguments at the pieces of the pool's memory.
@@ -570,7 +573,7 @@ int verify_chain(gesmc_pool_t p, uint32_t chain) {
   const uint64_t m = hc.shape.m;
   unsigned long long *E = at<unsigned long long>(p->base, p->lay.E);
   uint32_t *words = at<uint32_t>(p->base, p->lay.scratch) + 4;
-  if (m > 0 && launch_store_chain(p->args, hc.d, E, p->stream, p->num_sms) != cudaSuccess) {
+  if (m > 0 && launch_store_chain(p->args, hc.d, p->pool_round, E, p->stream, p->num_sms) != cudaSuccess) {
     cudaGetLastError();
     return GESMC_E_CUDA;
   }
@@ -1292,7 +1295,7 @@ int gesmc_pool_edges(gesmc_pool_t p, uint32_t chain, uint64_t *out, uint64_t cap
   // the list is kept in the last round's slot order: write it by position
   unsigned long long *E = out_on_device ? reinterpret_cast<unsigned long long *>(out)
                                         : at<unsigned long long>(p->base, p->lay.E);
-  bool ok = launch_store_chain(p->args, p->chains[chain].d, E, p->stream, p->num_sms) == cudaSuccess;
+  bool ok = launch_store_chain(p->args, p->chains[chain].d, p->pool_round, E, p->stream, p->num_sms) == cudaSuccess;
   if (ok && !out_on_device) ok = cudaMemcpyAsync(out, E, 8 * m, cudaMemcpyDeviceToHost, p->stream) == cudaSuccess;
   ok = ok && cudaStreamSynchronize(p->stream) == cudaSuccess;
   if (!ok) {
@@ -1596,8 +1599,8 @@ extern "C" int gesmc_run_noalloc(uint64_t *edges, uint64_t m, uint64_t n, uint64
     rc = pool_add_device(&p, reinterpret_cast<unsigned long long *>(edges), m, n, seed, start_round, 0, 0u, &chain);
   if (rc == GESMC_OK) rc = pool_run(&p, global_switches);
   if (rc == GESMC_OK &&
-      (launch_store_chain(p.args, p.chains[chain].d, reinterpret_cast<unsigned long long *>(edges), p.stream,
-                          p.num_sms) != cudaSuccess ||
+      (launch_store_chain(p.args, p.chains[chain].d, p.pool_round, reinterpret_cast<unsigned long long *>(edges),
+                          p.stream, p.num_sms) != cudaSuccess ||
        cudaStreamSynchronize(p.stream) != cudaSuccess)) {
     cudaGetLastError();
     rc = GESMC_E_CUDA;

@@ -20,7 +20,8 @@
 //   prec         uint4[buckets * cap]     permutation bucket records:
 //                                         {32 key bits, position, edge lo, hi}
 //   word         u32[switches]            outright-reject code | flags
-//   sw           uint2[switches]          dependency entries of e3, e4
+//   sw           uint2[switches]          dependency entries of e3, e4 (where
+//                                         word says that there is one)
 //   status       u32[switches]            (wave << 2) | state
 //   ptup         uint4[tuple storage]     Algorithm 1's tuples (four per
 //                                         switch) in fixed-capacity hash
@@ -74,6 +75,7 @@ constexpr uint32_t kTrivial = 0xFFFFFFFFu;  // sw entry: target without a depend
 constexpr uint32_t kCodeLoop = 1u, kCodeShared = 2u, kCodeLazy = 3u, kCodeMask = 3u;
 constexpr uint32_t kFlagBad = 4u;  // a target is in E when k runs, certainly
 constexpr uint32_t kFlagDep = 8u;  // a target depends on an undecided switch
+constexpr uint32_t kFlagEntry3 = 16u, kFlagEntry4 = 32u;  // sw holds e3's / e4's dependency entry
 
 // Switch status word: (wave << 2) | state.  Wave 0 means "not decided".
 constexpr uint32_t kUndecided = 0, kLegal = 1, kIllegal = 2;
@@ -238,6 +240,7 @@ struct RoundArgs {
   // kAggBuckets buckets (kNoChain otherwise): its positions are appended by
   // k_permute_agg, one cursor atomic per bucket and CTA instead of per record
   uint32_t agg_chain, agg_pairs;  // and its pairs of slots, (m + 1) / 2
+  uint32_t solo_chain;  // the only chain of the pool (kNoChain if there are more)
 };
 
 constexpr uint32_t kAggBuckets = 8192;
@@ -292,8 +295,9 @@ cudaError_t launch_round_fused(const RoundArgs &a, cudaStream_t s, uint32_t ctas
 // its slots, and write its current list by position.
 cudaError_t launch_load_chain(const RoundArgs &a, const ChainDesc &ch, const unsigned long long *E, cudaStream_t s,
                               int num_sms);
-cudaError_t launch_store_chain(const RoundArgs &a, const ChainDesc &ch, unsigned long long *E, cudaStream_t s,
-                               int num_sms);
+// (pool_round: rounds the pool has completed).
+cudaError_t launch_store_chain(const RoundArgs &a, const ChainDesc &ch, uint64_t pool_round, unsigned long long *E,
+                               cudaStream_t s, int num_sms);
 // Fill n u32 words with v.
 cudaError_t launch_fill_u32(uint32_t *p, uint32_t n, uint32_t v, cudaStream_t s, int num_sms);
 cudaError_t launch_canonicalise(unsigned long long *E, uint32_t m, unsigned long long n_bound, uint32_t *flags,

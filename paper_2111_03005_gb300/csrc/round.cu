@@ -168,7 +168,6 @@ __device__ __forceinline__ void build_switches(const RoundArgs &a, const ChainDe
     if (valid[t]) {
       const uint32_t code = is_lazy(ch, round, k[t], ell) ? kCodeLazy : tau(i[t], j[t], e1[t], e2[t], e3, e4);
       a.word[kg] = code;
-      a.sw[kg] = make_uint2(kTrivial, kTrivial);
       if (code) e3 = e4 = kEmptyKey;
     }
     key[2 * t] = e3;
@@ -224,6 +223,18 @@ __device__ __forceinline__ int check_target(const RoundArgs &a, uint32_t k, uint
   const uint2 pq = __ldcg(&a.dep[d]);
   return judge_target(k, pq.x, pq.y, pq.x < k ? __ldcg(&a.status[pq.x]) : 0u,
                       pq.y < k ? __ldcg(&a.status[pq.y]) : 0u, wave);
+}
+
+// The dependency entries of switch k's targets, given its word (sw holds an
+// entry only where the word says so: most switches have none, and their sw is
+// not written at all).
+__device__ __forceinline__ uint2 entries_of(uint32_t word, uint2 s) {
+  if (!(word & kFlagEntry3)) s.x = kTrivial;
+  if (!(word & kFlagEntry4)) s.y = kTrivial;
+  return s;
+}
+__device__ __forceinline__ uint2 switch_entries(const RoundArgs &a, uint32_t k) {
+  return entries_of(__ldcg(&a.word[k]), __ldcg(&a.sw[k]));
 }
 
 struct Tally {
@@ -344,8 +355,8 @@ __device__ __forceinline__ void store_record(const RoundArgs &a, uint32_t b, uin
 }
 
 // The positions of the chain with few buckets (a pool of one chain with at
-// most kAggBuckets buckets), each CTA taking kThreads * kPairs consecutive
-// pairs of slots: the CTA counts its records per bucket in shared memory (a
+// most kAggBuckets buckets), each CTA taking `tile` (at most kThreads * kPairs)
+// consecutive pairs of slots: the CTA counts its records per bucket in shared memory (a
 // record's rank among the CTA's records of its bucket comes with it), takes
 // each bucket's range with one cursor atomic, then stores its records, which
 // stay in registers meanwhile.  With few buckets every cursor takes thousands
@@ -354,9 +365,10 @@ __device__ __forceinline__ void store_record(const RoundArgs &a, uint32_t b, uin
 // orders them by key and position.  Bound by the generator (a Philox block per
 // position, about 400 instructions): with the keys computed again for the
 // second pass it took 38 us for 9.5e5 positions and, on two CTAs of 2048 pairs, 19 us
-// for 5,000; now 28 us, and 5.4 us on ten CTAs of 256 pairs.
+// for 5,000; now 22 us (in full waves of equal CTAs), and 5.4 us on ten CTAs of
+// 256 pairs.
 template <int kThreads, int kPairs>
-__global__ void __launch_bounds__(kThreads, 1024 / kThreads) k_permute_agg(RoundArgs a) {
+__global__ void __launch_bounds__(kThreads, 1024 / kThreads) k_permute_agg(RoundArgs a, uint32_t tile) {
   __shared__ uint32_t sc[kAggBuckets];  // per bucket: the CTA's count, then its base
   dep_launch();
   const ChainDesc ch = a.chains[a.agg_chain];
@@ -366,7 +378,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) k_permute_agg(Round
   const unsigned long long R = a.ctl->pool_round;
   const unsigned long long round = chain_round(ch, R);
   const bool apply = chain_apply(ch, R);
-  const uint32_t x0 = blockIdx.x * (kThreads * kPairs) + tid;
+  const uint32_t x0 = blockIdx.x * tile + tid, x1 = min(blockIdx.x * tile + tile, npair);
   __syncthreads();
   uint32_t pos[2 * kPairs], mid[2 * kPairs], br[2 * kPairs];  // br: bucket, and the rank in the high half
   unsigned long long e[2 * kPairs];
@@ -374,7 +386,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) k_permute_agg(Round
   for (int j = 0; j < kPairs; ++j) {
     const uint32_t x = x0 + j * kThreads;
     br[2 * j] = br[2 * j + 1] = kNoChain;
-    if (x >= npair) continue;
+    if (x >= x1) continue;
     const uint32_t gx = (ch.slot_base >> 1) + x;  // pair index in the pool's slots
     const bool two = 2 * x + 1 < ch.m;
     if (two) {
@@ -978,7 +990,9 @@ __global__ void k_boundary(RoundArgs a) {
 }
 
 // The chain of a thread's current pair, kept while its consecutive pairs
-// stay in it: pairs [lo, hi) are chain c's.
+// stay in it: pairs [lo, hi) are chain c's.  The only chain of a pool needs no
+// owner map (G(2^24): k_sources 1.54 -> 1.48 ms, k_wave1 0.27 -> 0.17 with its
+// counts summed per CTA; k_permute got slower by 3% and keeps the map).
 struct PairChain {
   uint32_t c = kNoChain, lo = 1, hi = 0;
 };
@@ -986,6 +1000,12 @@ struct PairChain {
 // Make pc the chain of pair x; false if no chain owns it.
 __device__ __forceinline__ bool pair_chain(const RoundArgs &a, uint32_t x, PairChain &pc) {
   if (x >= pc.lo && x < pc.hi) return true;
+  if (a.solo_chain != kNoChain) {
+    pc.c = a.solo_chain;
+    pc.lo = a.chains[pc.c].slot_base >> 1;
+    pc.hi = pc.lo + ((a.chains[pc.c].m + 1) >> 1);
+    return x >= pc.lo && x < pc.hi;
+  }
   pc.c = a.owner_slot[2 * x];
   if (pc.c == kNoChain) {
     pc.lo = 1;
@@ -1189,14 +1209,16 @@ __device__ __forceinline__ void group_alloc(const RoundArgs &a, const GroupSmem 
 // Wave 1 for target tuple v in slot s.
 __device__ __forceinline__ void group_decide(const RoundArgs &a, const GroupSmem &g, uint32_t s, uint32_t v) {
   const uint32_t k = v & kTupleK;
-  const uint32_t p = g.slot[s].z, q = g.slot[s].w;
-  if (p != kPNone && p >= k) atomicOr(&a.word[k], kFlagBad);       // present when k runs
-  else if (p != kPNone || q != k) atomicOr(&a.word[k], kFlagDep);  // erased or inserted earlier, maybe
-  const uint32_t d = g.aux[s];
+  const uint32_t p = g.slot[s].z, q = g.slot[s].w, d = g.aux[s];
+  uint32_t flags = 0;
+  if (p != kPNone && p >= k) flags = kFlagBad;                // present when k runs
+  else if (p != kPNone || q != k) flags = kFlagDep;           // erased or inserted earlier, maybe
   if (d != kTrivial) {
+    flags |= v & kTupleWhich ? kFlagEntry4 : kFlagEntry3;
     if (v & kTupleWhich) a.sw[k].y = d;
     else a.sw[k].x = d;
   }
+  if (flags) atomicOr(&a.word[k], flags);
 }
 
 // Persistent CTAs over the partitions.  Fast path: a thread keeps the hash
@@ -1380,18 +1402,25 @@ __global__ void __launch_bounds__(kGroupThreads, kGroupMin) k_group(RoundArgs a)
 }
 
 // Each CTA takes a contiguous range of switches, so that a thread's running
-// per-chain count changes chain only at chain boundaries.
+// per-chain count changes chain only at chain boundaries.  The counts leave the
+// CTA once: by the warp, their atomics on a handful of words took 15 of the 20
+// us of a power law of 1e6 edges.
 __device__ __forceinline__ void wave1_body(const RoundArgs &a) {
   Tally t;
   ChainCount cc;
   const uint32_t per = (a.switch_hw + gridDim.x - 1) / gridDim.x;
   const uint32_t chunk = (per + blockDim.x - 1) / blockDim.x * blockDim.x;
-  const uint32_t beg = min(blockIdx.x * chunk, a.switch_hw), end = min(beg + chunk, a.switch_hw);
+  uint32_t beg = min(blockIdx.x * chunk, a.switch_hw), end = min(beg + chunk, a.switch_hw);
+  if (a.solo_chain != kNoChain) {  // its switches only
+    const uint32_t lo = a.chains[a.solo_chain].switch_base, hi = lo + a.chains[a.solo_chain].L;
+    beg = max(beg, lo);
+    end = min(end, hi);
+  }
   for (uint32_t base = beg; base < end; base += blockDim.x) {
     const uint32_t k = base + threadIdx.x;
     bool wait = false;
     uint32_t c = kNoChain;
-    if (k < a.switch_hw) c = a.owner_switch[k];
+    if (k < end) c = a.solo_chain != kNoChain ? a.solo_chain : a.owner_switch[k];
     if (c != kNoChain) {
       const uint32_t w = __ldcs(&a.word[k]);
       const uint32_t code = w & kCodeMask;
@@ -1404,7 +1433,7 @@ __device__ __forceinline__ void wave1_body(const RoundArgs &a) {
       } else if (w & kFlagBad) {
         state = kIllegal;
         ++t.rej_exists;
-        drop_inserter(a, k, a.sw[k]);
+        drop_inserter(a, k, entries_of(w, a.sw[k]));
       } else if (w & kFlagDep) {
         state = kUndecided;
         wait = true;
@@ -1416,8 +1445,35 @@ __device__ __forceinline__ void wave1_body(const RoundArgs &a) {
     }
     append_if(wait, k, a.list0, &a.ctl->pending[0]);
   }
-  flush_tally(a, t);
-  flush_count(a, cc);
+  __shared__ uint32_t sums[5], chain0;
+  if (threadIdx.x < 5) sums[threadIdx.x] = 0;
+  if (threadIdx.x == 5) chain0 = kNoChain;
+  __syncthreads();
+  const uint32_t counts[4] = {t.accepted, t.rej_loop, t.rej_exists, t.lazy};
+  const bool lead = (threadIdx.x & 31) == 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t n = __reduce_add_sync(0xffffffffu, counts[i]);
+    if (lead && n) atomicAdd(&sums[i], n);
+  }
+  const uint32_t first = __reduce_min_sync(0xffffffffu, cc.n ? cc.chain : kNoChain);
+  if (lead && first != kNoChain) atomicMin(&chain0, first);
+  __syncthreads();
+  // the CTA's first chain, usually its only one, in one sum; other chains by the warp
+  const bool own = cc.n && cc.chain == chain0;
+  const uint32_t n0 = __reduce_add_sync(0xffffffffu, own ? cc.n : 0u);
+  if (lead && n0) atomicAdd(&sums[4], n0);
+  if (own) cc.n = 0;
+  if (__any_sync(0xffffffffu, cc.n != 0)) flush_count(a, cc);
+  __syncthreads();
+  if (threadIdx.x < 4 && sums[threadIdx.x]) {
+    unsigned long long *const to = threadIdx.x == 0   ? &a.st->accepted
+                                   : threadIdx.x == 1 ? &a.st->rej_loop
+                                   : threadIdx.x == 2 ? &a.st->rej_exists
+                                                      : &a.st->lazy;
+    atomicAdd(to, (unsigned long long)sums[threadIdx.x]);
+  }
+  if (threadIdx.x == 4 && sums[4]) atomicAdd(&a.chain_accepted[chain0], (unsigned long long)sums[4]);
 }
 
 __global__ void k_wave1(RoundArgs a) {
@@ -1452,7 +1508,7 @@ __device__ __forceinline__ uint32_t solo_waves(const RoundArgs &a, const uint32_
     if (tid + r * T >= n) continue;
     live |= 1u << r;
     k[r] = __ldcg(&in[tid + r * T]);
-    d[r] = __ldcg(&a.sw[k[r]]);
+    d[r] = switch_entries(a, k[r]);
     p[r].x = d[r].x != kTrivial ? __ldcg(&a.dep[d[r].x].x) : kPNone;
     p[r].y = d[r].y != kTrivial ? __ldcg(&a.dep[d[r].y].x) : kPNone;
   }
@@ -1524,7 +1580,7 @@ __global__ void k_wave_register(RoundArgs a) {
   const uint32_t *in = cur ? a.list1 : a.list0;
   for (uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x; idx < n; idx += gridDim.x * blockDim.x) {
     const uint32_t k = in[idx];
-    const uint2 s = __ldcg(&a.sw[k]);
+    const uint2 s = switch_entries(a, k);
     if (s.x != kTrivial) atomicMin(&a.dep[s.x].y, k);
     if (s.y != kTrivial) atomicMin(&a.dep[s.y].y, k);
   }
@@ -1555,7 +1611,7 @@ __global__ void k_wave_decide(RoundArgs a) {
     uint32_t k = 0;
     if (idx < n) {
       k = in[idx];
-      const uint2 s = __ldcg(&a.sw[k]);
+      const uint2 s = switch_entries(a, k);
       const int r3 = check_target(a, k, s.x, wave);
       const int r4 = check_target(a, k, s.y, wave);
       if (r3 == kBad || r4 == kBad) {
@@ -1654,7 +1710,7 @@ __global__ void __launch_bounds__(1024) k_tail(RoundArgs a) {
     uint32_t *out = cur ? a.list0 : a.list1;
     for (uint32_t idx = threadIdx.x; idx < n; idx += blockDim.x) {
       const uint32_t k = in[idx];
-      const uint2 s = __ldcg(&a.sw[k]);
+      const uint2 s = switch_entries(a, k);
       if (s.x != kTrivial) atomicMin(&a.dep[s.x].y, k);
       if (s.y != kTrivial) atomicMin(&a.dep[s.y].y, k);
     }
@@ -1669,7 +1725,7 @@ __global__ void __launch_bounds__(1024) k_tail(RoundArgs a) {
       uint32_t k = 0;
       if (idx < n) {
         k = in[idx];
-        const uint2 s = __ldcg(&a.sw[k]);
+        const uint2 s = switch_entries(a, k);
         const int r3 = check_target(a, k, s.x, wave);
         const int r4 = check_target(a, k, s.y, wave);
         if (r3 == kBad || r4 == kBad) {
@@ -1909,7 +1965,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_round_fused(RoundArgs a) {
       uint32_t *out = cur ? a.list0 : a.list1;
       for (uint32_t idx = gtid; idx < n; idx += nth) {
         const uint32_t k = __ldcg(&in[idx]);
-        const uint2 sv = __ldcg(&a.sw[k]);
+        const uint2 sv = switch_entries(a, k);
         if (sv.x != kTrivial) atomicMin(&a.dep[sv.x].y, k);
         if (sv.y != kTrivial) atomicMin(&a.dep[sv.y].y, k);
       }
@@ -1924,7 +1980,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_round_fused(RoundArgs a) {
         uint32_t k = 0;
         if (idx < n) {
           k = __ldcg(&in[idx]);
-          const uint2 sv = __ldcg(&a.sw[k]);
+          const uint2 sv = switch_entries(a, k);
           const int r3 = check_target(a, k, sv.x, wave);
           const int r4 = check_target(a, k, sv.y, wave);
           if (r3 == kBad || r4 == kBad) {
@@ -1970,19 +2026,24 @@ __global__ void k_load_chain(RoundArgs a, ChainDesc ch, const unsigned long long
   }
 }
 
-__global__ void k_store_chain(RoundArgs a, ChainDesc ch, unsigned long long *E) {
-  const bool apply = chain_apply(ch, a.ctl->pool_round);
-  const uint32_t npair = (ch.m + 1) >> 1;
+// A chain's list by position, with its last round's legal switches applied
+// (status; null if there is nothing to apply).  The host says so: with the round
+// counter read first, every access would wait for it (11.3 us a call for a
+// small chain, with launch and synchronisation; 10.9 so).
+__global__ void k_store_chain(const uint2 *cpos, const ulonglong2 *cedge, const uint32_t *status, uint32_t m,
+                              unsigned long long *E) {
+  const uint32_t npair = (m + 1) >> 1, L = m >> 1;
   for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < npair; k += gridDim.x * blockDim.x) {
-    const uint32_t s0 = ch.slot_base + 2 * k;
-    if (2 * k + 1 < ch.m) {
-      const uint32_t i = a.cpos[s0], j = a.cpos[s0 + 1];
-      unsigned long long e1 = a.cedge[s0], e2 = a.cedge[s0 + 1];
-      apply_last(a, ch, apply, k, i, j, e1, e2);
-      E[i] = e1;
-      E[j] = e2;
-    } else {
-      E[a.cpos[s0]] = a.cedge[s0];
+    if (k < L) {
+      const uint32_t st = status ? __ldcs(&status[k]) : 0u;
+      const uint2 ij = __ldcs(&cpos[k]);
+      const ulonglong2 ee = __ldcs(&cedge[k]);
+      unsigned long long e1 = ee.x, e2 = ee.y;
+      if ((st & 3u) == kLegal) tau(ij.x, ij.y, ee.x, ee.y, e1, e2);
+      E[ij.x] = e1;
+      E[ij.y] = e2;
+    } else {  // odd m: the last slot has no partner
+      E[reinterpret_cast<const uint32_t *>(cpos)[2 * k]] = reinterpret_cast<const unsigned long long *>(cedge)[2 * k];
     }
   }
 }
@@ -2238,7 +2299,7 @@ cudaError_t launch_round(const RoundArgs &a, cudaStream_t s, int num_sms, cudaEv
   // before it is a round's too (what came before may not wait as they do), and
   // not between the events of stage timing
   cudaError_t bad = cudaSuccess;
-  auto go = [&](void (*fn)(RoundArgs), uint32_t ctas, uint32_t threads, size_t smem = 0) {
+  auto go = [&](auto fn, uint32_t ctas, uint32_t threads, size_t smem = 0, auto... more) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ctas);
     cfg.blockDim = dim3(threads);
@@ -2249,7 +2310,7 @@ cudaError_t launch_round(const RoundArgs &a, cudaStream_t s, int num_sms, cudaEv
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = !ev && (n > 0 || after_round) ? 1 : 0;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, fn, a);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, fn, a, more...);
     if (e != cudaSuccess && bad == cudaSuccess) bad = e;
     ++n;
   };
@@ -2258,12 +2319,17 @@ cudaError_t launch_round(const RoundArgs &a, cudaStream_t s, int num_sms, cudaEv
   go(k_clear, grid_for(clear, 256, num_sms, 4), 256);
   if (work && a.any_exact) go(k_lazy_count, grid_for(a.switch_hw, 256, num_sms, 8), 256);
   mark(kStagePermute);
-  if (work && a.agg_chain != kNoChain)
-    // few pairs: spread over the SMs; more: more records per cursor atomic
-    if (a.agg_pairs <= (uint32_t)num_sms * 512) go(k_permute_agg<256, 1>, (a.agg_pairs + 255) / 256, 256);
-    else go(k_permute_agg<1024, 2>, (a.agg_pairs + 2047) / 2048, 1024);
-  else if (work)
+  if (work && a.agg_chain != kNoChain) {
+    if (a.agg_pairs <= (uint32_t)num_sms * 512) {  // few pairs: spread over the SMs
+      go(k_permute_agg<256, 1>, (a.agg_pairs + 255) / 256, 256, 0, 256u);
+    } else {  // more records per cursor atomic; one CTA per SM at a time, so full waves of equal CTAs
+      const uint32_t wave = (uint32_t)num_sms * 2048, ctas = (a.agg_pairs + wave - 1) / wave * num_sms;
+      const uint32_t tile = (a.agg_pairs + ctas - 1) / ctas;
+      go(k_permute_agg<1024, 2>, (a.agg_pairs + tile - 1) / tile, 1024, 0, tile);
+    }
+  } else if (work) {
     go(k_permute, a.permute_ctas, 256);
+  }
   mark(kStageScanPerm);
   if (work) {
     go(k_scan_perm, a.bucket_hw ? (a.bucket_hw + 1023) / 1024 : 1, 1024);
@@ -2317,11 +2383,15 @@ cudaError_t launch_load_chain(const RoundArgs &a, const ChainDesc &ch, const uns
   return cudaGetLastError();
 }
 
-cudaError_t launch_store_chain(const RoundArgs &a, const ChainDesc &ch, unsigned long long *E, cudaStream_t s,
-                               int num_sms) {
+cudaError_t launch_store_chain(const RoundArgs &a, const ChainDesc &ch, uint64_t pool_round, unsigned long long *E,
+                               cudaStream_t s, int num_sms) {
   if (ch.m == 0) return cudaSuccess;
   if (ch.m < kStoreMinEdges) {
-    k_store_chain<<<grid_for((ch.m + 1) / 2, 256, num_sms, 8), 256, 0, s>>>(a, ch, E);
+    // (slot ranges start on even slots)
+    k_store_chain<<<grid_for((ch.m + 1) / 2, 256, num_sms, 8), 256, 0, s>>>(
+        reinterpret_cast<const uint2 *>(a.cpos + ch.slot_base),
+        reinterpret_cast<const ulonglong2 *>(a.cedge + ch.slot_base),
+        pool_round > ch.added ? a.status + ch.switch_base : nullptr, ch.m, E);
     return cudaGetLastError();
   }
   // between rounds the permutation records and the bucket counts are free (at
