@@ -460,7 +460,7 @@ bool valid_opts(const gesmc_pool_opts &o) {
 }
 
 // Host state and device memory (owner maps, counters) of an empty pool whose
-// memory is bound at p->base.
+// memory is bound at p->base.  Does not wait for the device.
 int pool_init(gesmc_pool_t p, const gesmc_pool_opts &o) {
   p->slots.reset(p->cap.slots);
   p->switches.reset(p->cap.switches);
@@ -493,17 +493,13 @@ int pool_init(gesmc_pool_t p, const gesmc_pool_opts &o) {
   }
   cudaStream_t s = p->stream;
   const int sms = p->num_sms;
-  bool ok = launch_fill_u32(const_cast<uint32_t *>(a.owner_slot), (uint32_t)p->cap.slots, kNoChain, s, sms) ==
-            cudaSuccess;
-  ok &= launch_fill_u32(const_cast<uint32_t *>(a.owner_switch), (uint32_t)p->cap.switches, kNoChain, s, sms) ==
-        cudaSuccess;
-  ok &= launch_fill_u32(const_cast<uint32_t *>(a.owner_bucket), (uint32_t)p->cap.buckets, kNoChain, s, sms) ==
-        cudaSuccess;
-  ok &= launch_fill_u32(const_cast<uint32_t *>(a.owner_part), (uint32_t)p->cap.parts, kNoChain, s, sms) ==
-        cudaSuccess;
+  const FillRanges all = {{const_cast<uint32_t *>(a.owner_slot), const_cast<uint32_t *>(a.owner_switch),
+                           const_cast<uint32_t *>(a.owner_bucket), const_cast<uint32_t *>(a.owner_part)},
+                          {(uint32_t)p->cap.slots, (uint32_t)p->cap.switches, (uint32_t)p->cap.buckets,
+                           (uint32_t)p->cap.parts}};
+  bool ok = launch_fill_ranges(all, kNoChain, s, sms) == cudaSuccess;
   ok &= cudaMemsetAsync(a.ctl, 0, sizeof(Counters), s) == cudaSuccess;
   ok &= cudaMemsetAsync(a.st, 0, sizeof(StatsDev), s) == cudaSuccess;
-  ok &= cudaStreamSynchronize(s) == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
     return GESMC_E_CUDA;
@@ -514,34 +510,38 @@ int pool_init(gesmc_pool_t p, const gesmc_pool_opts &o) {
 
 // Validate and canonicalise the list at E (device, m edges) in place: loops,
 // ids >= n_bound, repeated edges, in that precedence.  *n_out receives
-// n_bound, or largest id + 1 if n_bound is 0.  Synchronises the stream.
-int validate_list(gesmc_pool_t p, unsigned long long *E, uint64_t m, uint64_t n_bound, uint64_t *n_out) {
+// n_bound, or largest id + 1 if n_bound is 0, *fp_out the list's degree
+// fingerprint.  Synchronises the stream, once: the repeated edges are looked
+// for before the host knows about the rest.
+int validate_list(gesmc_pool_t p, unsigned long long *E, uint64_t m, uint64_t n_bound, uint64_t *n_out,
+                  unsigned long long *fp_out) {
   cudaStream_t s = p->stream;
-  uint32_t *flags = at<uint32_t>(p->base, p->lay.scratch);
-  uint32_t host_flags[2] = {0, 0};
-  bool ok = cudaMemsetAsync(flags, 0, 8, s) == cudaSuccess;
-  if (ok && m > 0) ok &= launch_canonicalise(E, (uint32_t)m, n_bound, flags, flags + 1, s, p->num_sms) == cudaSuccess;
-  ok &= cudaMemcpyAsync(host_flags, flags, 8, cudaMemcpyDeviceToHost, s) == cudaSuccess;
-  ok &= cudaStreamSynchronize(s) == cudaSuccess;
-  if (!ok) {
-    cudaGetLastError();
-    return GESMC_E_CUDA;
+  struct {
+    uint32_t flags, max_id;
+    unsigned long long fp;
+  } host = {0, 0, 0};
+  char *words = at<char>(p->base, p->lay.scratch);
+  uint32_t *flags = reinterpret_cast<uint32_t *>(words);
+  if (m > 0) {
+    bool ok = cudaMemsetAsync(words, 0, sizeof(host), s) == cudaSuccess;
+    ok &= launch_canonicalise(E, (uint32_t)m, n_bound, flags, flags + 1, reinterpret_cast<unsigned long long *>(words + 8),
+                              s, p->num_sms) == cudaSuccess;
+    // between rounds the overflow-tuple array is free: it holds the set
+    ok &= launch_duplicate_check(E, (uint32_t)m, reinterpret_cast<unsigned long long *>(p->args.otup), 2 * p->cap.ovf,
+                                 flags, s, p->num_sms) == cudaSuccess;
+    ok &= cudaMemcpyAsync(&host, words, sizeof(host), cudaMemcpyDeviceToHost, s) == cudaSuccess;
+    ok &= cudaStreamSynchronize(s) == cudaSuccess;
+    if (!ok) {
+      cudaGetLastError();
+      return GESMC_E_CUDA;
+    }
   }
-  if (host_flags[0] & kFlagLoop) return GESMC_E_LOOP;
-  if (host_flags[0] & kFlagRange) return GESMC_E_RANGE;
-  *n_out = n_bound ? n_bound : (m ? (uint64_t)host_flags[1] + 1 : 0);
-  if (m == 0) return GESMC_OK;
-  // between rounds the overflow-tuple array is free: it holds the set
-  ok &= launch_duplicate_check(E, (uint32_t)m, reinterpret_cast<unsigned long long *>(p->args.otup), 2 * p->cap.ovf,
-                               flags, s, p->num_sms) == cudaSuccess;
-  ok &= cudaMemcpyAsync(host_flags, flags, 4, cudaMemcpyDeviceToHost, s) == cudaSuccess;
-  ok &= cudaStreamSynchronize(s) == cudaSuccess;
-  if (!ok) {
-    cudaGetLastError();
-    return GESMC_E_CUDA;
-  }
-  if (host_flags[0] & kFlagMulti) return GESMC_E_MULTI;
-  if (host_flags[0] & kFlagTableFull) return GESMC_E_INTERNAL;
+  if (host.flags & kFlagLoop) return GESMC_E_LOOP;
+  if (host.flags & kFlagRange) return GESMC_E_RANGE;
+  if (host.flags & kFlagMulti) return GESMC_E_MULTI;
+  if (host.flags & kFlagTableFull) return GESMC_E_INTERNAL;
+  *n_out = n_bound ? n_bound : (m ? (uint64_t)host.max_id + 1 : 0);
+  *fp_out = host.fp;
   return GESMC_OK;
 }
 
@@ -644,17 +644,12 @@ bool alloc_ranges(gesmc_pool_t p, HostChain &hc) {
 // Set the owner maps of a chain's ranges to `c` (kNoChain to remove it).
 bool set_owners(gesmc_pool_t p, const HostChain &hc, uint32_t c) {
   RoundArgs &a = p->args;
-  cudaStream_t s = p->stream;
-  const int sms = p->num_sms;
-  bool ok = launch_fill_u32(const_cast<uint32_t *>(a.owner_slot) + hc.d.slot_base, hc.shape.slots(), c, s, sms) ==
-            cudaSuccess;
-  ok &= launch_fill_u32(const_cast<uint32_t *>(a.owner_switch) + hc.d.switch_base, hc.shape.L, c, s, sms) ==
-        cudaSuccess;
-  ok &= launch_fill_u32(const_cast<uint32_t *>(a.owner_bucket) + hc.d.bucket_base, hc.shape.nb, c, s, sms) ==
-        cudaSuccess;
-  ok &= launch_fill_u32(const_cast<uint32_t *>(a.owner_part) + hc.d.part_base, hc.shape.np, c, s, sms) ==
-        cudaSuccess;
-  return ok;
+  const FillRanges own = {
+      {const_cast<uint32_t *>(a.owner_slot) + hc.d.slot_base, const_cast<uint32_t *>(a.owner_switch) + hc.d.switch_base,
+       const_cast<uint32_t *>(a.owner_bucket) + hc.d.bucket_base,
+       const_cast<uint32_t *>(a.owner_part) + hc.d.part_base},
+      {hc.shape.slots(), hc.shape.L, hc.shape.nb, hc.shape.np}};
+  return launch_fill_ranges(own, c, p->stream, p->num_sms) == cudaSuccess;
 }
 
 // Add a chain whose list is already on the device at E (the pool's staging
@@ -670,15 +665,10 @@ int pool_add_device(gesmc_pool_t p, unsigned long long *E, uint64_t m, uint64_t 
   std::memset(&hc.d, 0, sizeof(hc.d));
   if (!chain_shape(m, p->tuple_log2, p->cap.bucket_log2, &hc.shape)) return GESMC_E_INVALID;
   uint64_t n_eff = 0;
-  int rc = validate_list(p, E, m, n, &n_eff);
+  // (with the starting list's degree fingerprint, which gesmc_verify compares against)
+  const int rc = validate_list(p, E, m, n, &n_eff, &hc.fp);
   if (rc != GESMC_OK) return rc;
   if (p->resident && !resident_fits(m, n_eff)) return GESMC_E_TOO_LARGE;
-  {  // the starting list's degree fingerprint (gesmc_verify compares against it)
-    uint32_t flags = 0;
-    rc = list_check(E, m, 0, nullptr, 0, at<uint32_t>(p->base, p->lay.scratch) + 4, p->stream, p->num_sms, &flags,
-                    &hc.fp);
-    if (rc != GESMC_OK) return rc;
-  }
   if (!alloc_ranges(p, hc)) return GESMC_E_NOMEM;
   ChainDesc &d = hc.d;
   d.m = hc.shape.m;
@@ -721,7 +711,7 @@ int pool_run(gesmc_pool_t p, uint64_t rounds) {
   DeviceGuard g(p->device);
   cudaStream_t s = p->stream;
   const RoundArgs a = p->args;
-  if (cudaMemsetAsync(&a.ctl->err, 0, sizeof(uint32_t), s) != cudaSuccess) return GESMC_E_CUDA;
+  // (the device's error word is zero: a call that sets it breaks the pool)
   const size_t per_round = kNumStages + 1;
   const bool stage_events = p->profiling && !p->resident;  // resident rounds have no separate stages
   if (stage_events) {
@@ -1023,8 +1013,7 @@ int pool_es_run(gesmc_pool_t p, uint64_t switches, uint32_t only) {
   uint32_t *djob_of = at<uint32_t>(p->base, p->lay.es_job_of);
   uint32_t *err = &a.ctl->err;
   const uint32_t nj = (uint32_t)jobs.size();
-  bool ok = cudaMemsetAsync(err, 0, sizeof(uint32_t), s) == cudaSuccess;
-  ok &= cudaMemcpyAsync(djob_of, job_of.data(), 4ull * p->max_chains, cudaMemcpyHostToDevice, s) == cudaSuccess;
+  bool ok = cudaMemcpyAsync(djob_of, job_of.data(), 4ull * p->max_chains, cudaMemcpyHostToDevice, s) == cudaSuccess;
   ok &= cudaMemcpyAsync(djobs, jobs.data(), sizeof(EsJob) * nj, cudaMemcpyHostToDevice, s) == cudaSuccess;
   ok &= launch_es_store(a, djobs, djob_of, s, p->num_sms) == cudaSuccess;
   const uint64_t set_launches = 2ull * ((nj + 65534) / 65535);
@@ -1119,7 +1108,8 @@ void gesmc_pool_destroy(gesmc_pool_t p) {
   delete p;
 }
 
-int gesmc_pool_create(const gesmc_pool_opts *opts, gesmc_pool_t *out) {
+// Without waiting for the device (gesmc_create's next step does).
+static int pool_create(const gesmc_pool_opts *opts, gesmc_pool_t *out) {
   if (!out || !opts) return GESMC_E_INVALID;
   *out = nullptr;
   const gesmc_pool_opts o = *opts;
@@ -1167,6 +1157,19 @@ int gesmc_pool_create(const gesmc_pool_opts *opts, gesmc_pool_t *out) {
     return rc;
   }
   *out = p;
+  return GESMC_OK;
+}
+
+int gesmc_pool_create(const gesmc_pool_opts *opts, gesmc_pool_t *out) {
+  const int rc = pool_create(opts, out);
+  if (rc != GESMC_OK) return rc;
+  DeviceGuard g((*out)->device);
+  if (cudaStreamSynchronize((*out)->stream) != cudaSuccess) {
+    cudaGetLastError();
+    gesmc_pool_destroy(*out);
+    *out = nullptr;
+    return GESMC_E_CUDA;
+  }
   return GESMC_OK;
 }
 
@@ -1451,7 +1454,7 @@ int gesmc_create(const uint64_t *edges, uint64_t m, int edges_on_device, const g
   po.alloc_ctx = o.alloc_ctx;
   gesmc_ctx *h = new (std::nothrow) gesmc_ctx();
   if (!h) return GESMC_E_NOMEM;
-  int rc = gesmc_pool_create(&po, &h->pool);
+  int rc = pool_create(&po, &h->pool);
   // the seed is given to gesmc_run; the chain starts with seed 0
   if (rc == GESMC_OK)
     rc = gesmc_pool_add(h->pool, edges, m, edges_on_device, o.n, 0, o.start_round, o.lazy_threshold,

@@ -298,10 +298,16 @@ cudaError_t launch_load_chain(const RoundArgs &a, const ChainDesc &ch, const uns
 // (pool_round: rounds the pool has completed).
 cudaError_t launch_store_chain(const RoundArgs &a, const ChainDesc &ch, uint64_t pool_round, unsigned long long *E,
                                cudaStream_t s, int num_sms);
-// Fill n u32 words with v.
-cudaError_t launch_fill_u32(uint32_t *p, uint32_t n, uint32_t v, cudaStream_t s, int num_sms);
+// Fill four ranges of u32 words with v (the owner maps of a chain, or of a pool).
+struct FillRanges {
+  uint32_t *p[4];
+  uint32_t n[4];
+};
+cudaError_t launch_fill_ranges(const FillRanges &r, uint32_t v, cudaStream_t s, int num_sms);
+// A caller's list made canonical in place; flags, largest id and degree
+// fingerprint into words zeroed by the caller.
 cudaError_t launch_canonicalise(unsigned long long *E, uint32_t m, unsigned long long n_bound, uint32_t *flags,
-                                uint32_t *max_id, cudaStream_t s, int num_sms);
+                                uint32_t *max_id, unsigned long long *fp, cudaStream_t s, int num_sms);
 // Debug check of a list: kFlagLoop for an entry that is not canonical and
 // loop-free, kFlagRange for an id >= n (if n), and its degree fingerprint
 // added to *fp (zero it first).

@@ -2161,26 +2161,13 @@ __global__ void k_es_load(RoundArgs a, const EsJob *jobs, const uint32_t *job_of
   }
 }
 
-__global__ void k_fill_u32(uint32_t *p, uint32_t n, uint32_t v) {
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) p[i] = v;
+__global__ void k_fill_ranges(FillRanges r, uint32_t v) {
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < r.n[j]; i += gridDim.x * blockDim.x) r.p[j][i] = v;
 }
 
 // ---------------------------------------------------------------- create-time checks
-
-__global__ void k_canonicalise(unsigned long long *E, uint32_t m, unsigned long long n_bound, uint32_t *flags,
-                               uint32_t *max_id) {
-  uint32_t f = 0, mx = 0;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
-    const unsigned long long e = E[i];
-    const uint32_t x = (uint32_t)(e >> 32), y = (uint32_t)e;
-    if (x == y) f |= kFlagLoop;
-    if (n_bound && (x >= n_bound || y >= n_bound)) f |= kFlagRange;
-    mx = max(mx, max(x, y));
-    E[i] = pack_edge(x, y);
-  }
-  if (f) atomicOr(flags, f);
-  if (m) atomicMax(max_id, mx);
-}
 
 __global__ void k_fill_u64(unsigned long long *p, unsigned long long n, unsigned long long v) {
   for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < n;
@@ -2213,6 +2200,31 @@ __global__ void k_duplicates(const unsigned long long *E, uint32_t m, unsigned l
 // multiset of endpoints, i.e. of the degree sequence, which a switch keeps.
 __device__ __forceinline__ unsigned long long endpoint_term(uint32_t v) {
   return mix64(0x9E3779B97F4A7C15ull + v);
+}
+
+// The caller's list made canonical in place: flags for a loop or an id out of
+// range, the largest id, and the degree fingerprint.
+__global__ void k_canonicalise(unsigned long long *E, uint32_t m, unsigned long long n_bound, uint32_t *flags,
+                               uint32_t *max_id, unsigned long long *fp) {
+  uint32_t f = 0, mx = 0;
+  unsigned long long sum = 0;
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
+    const unsigned long long e = E[i];
+    const uint32_t x = (uint32_t)(e >> 32), y = (uint32_t)e;
+    if (x == y) f |= kFlagLoop;
+    if (n_bound && (x >= n_bound || y >= n_bound)) f |= kFlagRange;
+    mx = max(mx, max(x, y));
+    sum += endpoint_term(x) + endpoint_term(y);
+    E[i] = pack_edge(x, y);
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, off);
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if ((threadIdx.x & 31) == 0) {
+    if (sum) atomicAdd(fp, sum);
+    if (mx) atomicMax(max_id, mx);
+  }
+  if (f) atomicOr(flags, f);
 }
 
 // Debug check of a position-order list: every entry canonical and
@@ -2420,15 +2432,16 @@ cudaError_t launch_es_load(const RoundArgs &a, const EsJob *jobs, const uint32_t
   return cudaGetLastError();
 }
 
-cudaError_t launch_fill_u32(uint32_t *p, uint32_t n, uint32_t v, cudaStream_t s, int num_sms) {
-  if (n == 0) return cudaSuccess;
-  k_fill_u32<<<grid_for(n, 256, num_sms, 8), 256, 0, s>>>(p, n, v);
+cudaError_t launch_fill_ranges(const FillRanges &r, uint32_t v, cudaStream_t s, int num_sms) {
+  const uint32_t most = std::max(std::max(r.n[0], r.n[1]), std::max(r.n[2], r.n[3]));
+  if (most == 0) return cudaSuccess;
+  k_fill_ranges<<<grid_for(most, 256, num_sms, 8), 256, 0, s>>>(r, v);
   return cudaGetLastError();
 }
 
 cudaError_t launch_canonicalise(unsigned long long *E, uint32_t m, unsigned long long n_bound, uint32_t *flags,
-                                uint32_t *max_id, cudaStream_t s, int num_sms) {
-  k_canonicalise<<<grid_for(m, 256, num_sms, 8), 256, 0, s>>>(E, m, n_bound, flags, max_id);
+                                uint32_t *max_id, unsigned long long *fp, cudaStream_t s, int num_sms) {
+  k_canonicalise<<<grid_for(m, 256, num_sms, 8), 256, 0, s>>>(E, m, n_bound, flags, max_id, fp);
   return cudaGetLastError();
 }
 
