@@ -1040,8 +1040,9 @@ int pool_es_run(gesmc_pool_t p, uint64_t switches, uint32_t only) {
     for (uint64_t iter = 0; ok; ++iter) {
       const uint32_t groups[4] = {group[0], iter ? 0u : group[1], iter ? 0u : group[2], iter ? 0u : group[3]};
       if (group[0]) ok &= cudaMemsetAsync(nstop, 0, sizeof(uint32_t), s) == cudaSuccess;
-      ok &= launch_es_run(djobs, groups, n, samples, dists, a.st, a.chain_accepted, err, nstop, s, p->gstream, p->ev_in,
-                          p->ev_out, &run_launches) == cudaSuccess;
+      // (a job that went on alone does so for the rest of the call)
+      ok &= launch_es_run(djobs, groups, n, samples, dists, a.st, a.chain_accepted, err, nstop, iter > 0 || off > 0, s,
+                          p->gstream, p->ev_in, p->ev_out, &run_launches) == cudaSuccess;
       p->launches += run_launches;
       if (!ok || group[0] == 0) break;  // only the largest windows stop
       uint32_t stopped = 0, e = 0;

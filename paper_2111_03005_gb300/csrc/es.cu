@@ -15,7 +15,8 @@
 // earlier legal switch inserts it.
 //
 // Supersteps of ES-MC hold about sqrt(m) switches (the birthday bound), so
-// one CTA runs all supersteps of one chain, a switch per thread.  The list E
+// one CTA (for the largest chains a cluster of eight) runs all supersteps of
+// one chain, a switch per thread.  The list E
 // (position order) and the edge set H (open addressing over canonical ids,
 // tombstones on erase) live in HBM; a list entry also holds its edge's slot in
 // H, so that erasing it takes no search, and the search for a target ends at
@@ -232,7 +233,7 @@ __device__ __forceinline__ bool window_any(bool x) {
 // H <- empty, for every job (blockIdx.y = job).
 __global__ void k_es_clear(EsJob *jobs, uint32_t job_off, bool only_stopped) {
   const EsJob &jb = jobs[job_off + blockIdx.y];
-  if (jb.m < 2 || (only_stopped && !jb.stopped)) return;  // no list, no set; or a set that needs no rebuild
+  if (jb.m < 2 || (only_stopped && jb.stopped != 1)) return;  // no list, no set; or a set that needs no rebuild
   const unsigned long long cap = 1ull << jb.hlog2;
   const unsigned long long nth = (unsigned long long)gridDim.x * blockDim.x;
   unsigned long long *const H = jb.H;
@@ -244,7 +245,7 @@ __global__ void k_es_clear(EsJob *jobs, uint32_t job_off, bool only_stopped) {
 // H <- the entries of E, each entry's slot into the list.
 __global__ void k_es_fill(const EsJob *jobs, uint32_t job_off, uint32_t *err, bool only_stopped) {
   const EsJob jb = jobs[job_off + blockIdx.y];
-  if (jb.m < 2 || (only_stopped && !jb.stopped)) return;
+  if (jb.m < 2 || (only_stopped && jb.stopped != 1)) return;
   const uint32_t mask = (uint32_t)((1ull << jb.hlog2) - 1);
   for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < jb.m; s += gridDim.x * blockDim.x) {
     const unsigned long long e = rec_edge(jb.E[s]);
@@ -340,10 +341,10 @@ __global__ void __launch_bounds__(C) k_es_sample(EsJob *jobs, uint32_t job_off, 
 // that one SM moves to and from L2 (about 11 a switch, and one every two
 // cycles or so at random addresses).  With sampling and first-touch tables in
 // every window, key tables for every superstep and separate searches to find,
-// erase and insert, 2^19 switches of a chain of 1e6 edges took 21.4 ms, now 7.2
-// (26 -> 8.9 us a superstep); 512 chains of 65 to 118,000 edges with 2^14
-// switches each 22.0 ms, now 8.9 (most are single warps: 2270 -> 430
-// instructions a superstep).
+// erase and insert, 2^19 switches of a chain of 1e6 edges took 21.4 ms, then 7.2
+// (26 -> 8.9 us a superstep; on a cluster 5.1, see below); 512 chains of 65 to
+// 118,000 edges with 2^14 switches each 22.0 ms, now 8.9 (most are single warps:
+// 2270 -> 430 instructions a superstep).
 template <int B, bool kStopToRebuild>
 __device__ __forceinline__ void es_run_body(EsJob *jobs, uint32_t job_off, uint32_t nsw, const uint2 *samples,
                                             const uint16_t *dists, StatsDev *stats, unsigned long long *chain_acc,
@@ -367,6 +368,7 @@ __device__ __forceinline__ void es_run_body(EsJob *jobs, uint32_t job_off, uint3
   const uint16_t *const dist = dists + (size_t)job.row * nsw;
   const uint32_t mask = (uint32_t)((1ull << job.hlog2) - 1);
   uint32_t s = job.done;
+  if (kStopToRebuild && !job.alone) return;
   if (s >= nsw) {
     if (kStopToRebuild && x == 0) job.stopped = 0;
     return;
@@ -657,6 +659,346 @@ __device__ __forceinline__ void es_run_body(EsJob *jobs, uint32_t job_off, uint3
   }
 }
 
+// ---------------------------------------------------------------- large chains
+// One chain on a cluster of kClusterCtas CTAs, for chains of at least
+// kEsBigChain edges (windows of 1024 switches, thread x of CTA r holding switch
+// r * T + x): one SM moves about one 32-byte sector to or from L2 every two
+// cycles, and a window's switches need some 9,000, so that one CTA took 8.9 us
+// a superstep (7.2 ms for 2^19 switches of a chain of 1.05e6 edges); so, 6.2 us
+// (5.1 ms).  What is left is one superstep's chain of dependent accesses to L2
+// (sources, set, insertion, the stores' way there) and three cluster barriers.
+//
+// The CTAs exchange almost nothing: every CTA finds the cut by itself, and the
+// list and the set are in L2.  A superstep is
+//   1. gather the sources, search the set for the targets; a present target is
+//      an event, told to every CTA (its id and its switch);
+//   2. insert the targets of the switches with none present, each where its
+//      search ended.  Two switches with the same target meet in the same slot;
+//      the later to get there ends the superstep before its own switch.  A
+//      switch whose source is a later switch's present target ends it before
+//      that one.  (A target's eraser that comes after the switch is no matter:
+//      the edge is there when the switch runs.)
+//   3. the switches before that end are independent of one another: those with
+//      a present target are illegal, the others legal; they rewire and erase,
+//      and the ones past the end take their insertions back as tombstones.
+// Any cut into runs without a shared position gives the sequential result; the
+// first switch always runs.
+constexpr int kClusterCtas = 8;
+constexpr uint32_t kEvents = 128;  // present targets of a superstep that are told apart
+// Present targets a superstep on average (a graph with large hubs) from which
+// on the chain is left to one CTA and its waves: the events cost every switch a
+// comparison, and past kEvents of them end the superstep (a power law of 1.7e6
+// edges with exponent 2.2, 1e5 switches: 3.7 ms here, 1.7 there).
+constexpr uint32_t kBusyEvents = 16;
+
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// The same where only the threads with `told` have written anything that the
+// other CTAs read next: the others need no fence (a release by every thread
+// waits for all its stores and atomics on L2).
+__device__ __forceinline__ void cluster_sync_told(bool told) {
+  if (told) asm volatile("fence.acq_rel.cluster;" ::: "memory");
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// The address in CTA `rank`'s shared memory of what is at `p` in this CTA's.
+__device__ __forceinline__ uint32_t peer_addr(const void *p, uint32_t rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ uint32_t peer_add(uint32_t *p, uint32_t rank, uint32_t v) {
+  uint32_t old;
+  asm volatile("atom.relaxed.cluster.shared::cluster.add.u32 %0, [%1], %2;"
+               : "=r"(old)
+               : "r"(peer_addr(p, rank)), "r"(v)
+               : "memory");
+  return old;
+}
+// min / max / add into the same word of every CTA of the cluster.
+__device__ __forceinline__ void all_min(uint32_t *p, uint32_t v) {
+#pragma unroll 1
+  for (uint32_t r = 0; r < kClusterCtas; ++r)
+    asm volatile("red.relaxed.cluster.shared::cluster.min.u32 [%0], %1;" ::"r"(peer_addr(p, r)), "r"(v) : "memory");
+}
+__device__ __forceinline__ void all_max(uint32_t *p, uint32_t v) {
+#pragma unroll 1
+  for (uint32_t r = 0; r < kClusterCtas; ++r)
+    asm volatile("red.relaxed.cluster.shared::cluster.max.u32 [%0], %1;" ::"r"(peer_addr(p, r)), "r"(v) : "memory");
+}
+__device__ __forceinline__ void all_add(uint32_t *p, uint32_t v) {
+#pragma unroll 1
+  for (uint32_t r = 0; r < kClusterCtas; ++r)
+    asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], %1;" ::"r"(peer_addr(p, r)), "r"(v) : "memory");
+}
+__device__ __forceinline__ void all_store(unsigned long long *p, unsigned long long v) {
+#pragma unroll 1
+  for (uint32_t r = 0; r < kClusterCtas; ++r)
+    asm volatile("st.relaxed.cluster.shared::cluster.u64 [%0], %1;" ::"r"(peer_addr(p, r)), "l"(v) : "memory");
+}
+
+// Search for a key from slot s on: whether it is in the set, else the first
+// slot that could take it and what that held.
+struct SetSearch {
+  uint32_t s, at;
+  unsigned long long was;
+  bool present, done;
+};
+// One aligned group of four slots, a sector of L2 (the sets have 2^h >= 4 slots
+// and start on 256 bytes).
+struct Four {
+  unsigned long long v[4];
+};
+__device__ __forceinline__ Four load_four(const unsigned long long *p) {
+  Four f;
+  asm volatile("ld.global.cg.v2.u64 {%0, %1}, [%2];" : "=l"(f.v[0]), "=l"(f.v[1]) : "l"(p) : "memory");
+  asm volatile("ld.global.cg.v2.u64 {%0, %1}, [%2];" : "=l"(f.v[2]), "=l"(f.v[3]) : "l"(p + 2) : "memory");
+  return f;
+}
+// The search over the group that holds slot q.s, from there on.
+__device__ __forceinline__ void search_step(SetSearch &q, unsigned long long key, const Four &f, uint32_t mask) {
+  const uint32_t from = q.s & 3u;
+#pragma unroll
+  for (uint32_t v = 0; v < 4; ++v) {
+    if (v < from || q.done) continue;
+    const unsigned long long cur = f.v[v];
+    if (cur == key) {
+      q.present = q.done = true;
+      continue;
+    }
+    if ((cur == kEmptyKey || cur == kTombKey) && q.at == kNil) {
+      q.at = (q.s & ~3u) + v;
+      q.was = cur;
+    }
+    if (cur == kEmptyKey) q.done = true;
+  }
+  q.s = ((q.s & ~3u) + 4) & mask;
+}
+
+// Insert a key from slot s on, where a search ended; stops at the key itself,
+// which another switch of the superstep has put there (*twice), or, for the
+// superstep's first switch, takes the next free slot (the other switch will
+// take its own back).  Returns the slot, or kNil if the table is full or the key
+// was there.
+__device__ __forceinline__ uint32_t insert_once(unsigned long long *H, uint32_t mask, unsigned long long key, uint32_t s,
+                                                unsigned long long was, uint32_t *tomb, bool first, bool *twice, bool *full) {
+  for (uint32_t n = 0; n <= mask; ++n) {
+    if (was == kEmptyKey || was == kTombKey) {
+      const unsigned long long got = atomicCAS(&H[s], was, key);
+      if (got == was) {
+        *tomb = was == kTombKey ? 1u : 0u;
+        return s;
+      }
+      was = got;  // taken meanwhile: look at what is there now
+      continue;
+    }
+    if (was == key) {
+      *twice = true;
+      if (!first) return kNil;
+    }
+    s = (s + 1) & mask;
+    was = __ldcg(&H[s]);
+  }
+  *full = true;
+  return kNil;
+}
+
+template <int T>
+__global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(T)
+    k_es_run_cluster(EsJob *jobs, uint32_t job_off, uint32_t nsw, const uint2 *samples, const uint16_t *dists, StatsDev *stats,
+                 unsigned long long *chain_acc, uint32_t *err, uint32_t *nstop) {
+  constexpr uint32_t B = T * kClusterCtas;  // the window
+  constexpr int kDist = kClusterCtas;       // distances a thread looks at for the cut
+  // per parity of the superstep: events (told so far, in CTA 0: asked for), the
+  // end they force, this CTA's tombstones, the cut
+  __shared__ uint32_t s_events[2], s_asked[2], s_end[2], s_mine[2], s_cut[2], s_tombs;
+  __shared__ unsigned long long s_key[2][kEvents], s_who[2][kEvents];
+  EsJob &job = jobs[job_off + blockIdx.x / kClusterCtas];
+  const uint32_t rank = cluster_rank(), tid = threadIdx.x, x = rank * T + tid;
+  uint4 *const E = job.E;
+  unsigned long long *const H = job.H;
+  const uint2 *const samp = samples + (size_t)job.row * nsw;
+  const uint16_t *const dist = dists + (size_t)job.row * nsw;
+  const uint32_t mask = (uint32_t)((1ull << job.hlog2) - 1), limit = mask >> 3;
+  uint32_t s = job.done, acc = 0, rej_loop = 0, rej_exists = 0, tomb_total = 0;
+  if (job.alone || s >= nsw) {  // (the same in every CTA of the cluster)
+    if (x == 0 && !job.alone) job.stopped = 0;
+    return;
+  }
+  if (tid < 2) {
+    s_events[tid] = s_asked[tid] = s_mine[tid] = 0;
+    s_end[tid] = s_cut[tid] = B;
+  }
+  if (tid == 0) s_tombs = job.tombs;
+  uint2 cur;
+  uint32_t d[kDist];
+  // the window from s on: the thread's own switch, and its share of the
+  // distances (the same in every CTA: the cut needs all of them)
+  auto load_window = [&](uint32_t from) {
+    cur = from + x < nsw ? __ldg(&samp[from + x]) : make_uint2(0, 0);
+#pragma unroll
+    for (int v = 0; v < kDist; ++v) {
+      const uint32_t k = from + tid + v * T;
+      d[v] = k < nsw ? __ldg(&dist[k]) : 0xFFFFu;
+    }
+  };
+  auto find_cut = [&](uint32_t *cut) {
+    uint32_t c = B;
+#pragma unroll
+    for (int v = kDist - 1; v >= 0; --v)
+      if (d[v] <= tid + v * T) c = tid + v * T;
+    c = __reduce_min_sync(0xffffffffu, c);
+    if ((tid & 31u) == 0 && c < B) atomicMin(cut, c);
+  };
+  load_window(s);
+  __syncthreads();
+  find_cut(&s_cut[0]);
+  cluster_sync();  // (every CTA's shared memory is set up)
+  uint32_t stop = 0, steps = 0, met = 0;
+  for (uint32_t par = 0;; par ^= 1u) {
+    const uint32_t n = min(min(B, nsw - s), s_cut[par]);
+    const uint32_t i = cur.x, j = cur.y & 0x7FFFFFFFu, g = cur.y >> 31;
+    uint4 r1 = make_uint4(0, 0, 0, 0), r2 = r1;
+    if (x < n) {
+      r1 = __ldcg(&E[i]);
+      r2 = __ldcg(&E[j]);
+    }
+    load_window(s + n);
+    if (tid == 0) s_cut[par ^ 1] = B;
+    const unsigned long long e1 = rec_edge(r1), e2 = rec_edge(r2);
+    unsigned long long e3 = 0, e4 = 0;
+    const uint32_t code = x < n ? tau_g(g, e1, e2, e3, e4) : kCodeLazy;
+    SetSearch q3 = {0, kNil, kNoKey, false, true}, q4 = q3;
+    bool told = false;
+    if (code == 0) {
+      q3.s = hash32(e3) & mask;
+      q4.s = hash32(e4) & mask;
+      q3.done = q4.done = false;
+      for (uint32_t v = 0; v <= mask && !(q3.done && q4.done); ++v) {
+        Four c3, c4;
+        if (!q3.done) c3 = load_four(&H[q3.s & ~3u]);
+        if (!q4.done) c4 = load_four(&H[q4.s & ~3u]);
+        if (!q3.done) search_step(q3, e3, c3, mask);
+        if (!q4.done) search_step(q4, e4, c4, mask);
+      }
+      // present targets: told to every CTA; without room for them the
+      // superstep ends before this switch
+      for (int w = 0; w < 2; ++w) {
+        if (!(w ? q4.present : q3.present)) continue;
+        told = true;
+        const uint32_t at = peer_add(&s_asked[par], 0, 1u);
+        if (at < kEvents) {
+          all_store(&s_key[par][at], w ? e4 : e3);
+          all_store(&s_who[par][at], x);
+          all_max(&s_events[par], at + 1);
+        } else {
+          all_min(&s_end[par], x ? x : 1u);
+        }
+      }
+    }
+    cluster_sync_told(told);
+    // erasers of present targets, and the insertions
+    told = false;
+    const bool live = code == 0, clear = live && !q3.present && !q4.present;
+    const uint32_t events = s_events[par];
+    if (live) {
+      for (uint32_t v = 0; v < events; ++v) {
+        const uint32_t who = (uint32_t)s_who[par][v];
+        const unsigned long long key = s_key[par][v];
+        if (x < who && (key == e1 || key == e2)) {
+          all_min(&s_end[par], who);
+          told = true;
+        }
+      }
+    }
+    uint32_t p3 = kNil, p4 = kNil, t3 = 0, t4 = 0;
+    if (clear) {
+      bool twice = false, full = false;
+      p3 = insert_once(H, mask, e3, q3.at, q3.was, &t3, x == 0, &twice, &full);
+      p4 = insert_once(H, mask, e4, q4.at, q4.was, &t4, x == 0, &twice, &full);
+      if (twice) all_min(&s_end[par], x ? x : 1u);
+      told |= twice;
+      if (full) atomicOr(err, kErrTableFull);
+    }
+    cluster_sync_told(told);
+    const uint32_t end = min(n, s_end[par]);
+    uint32_t tombs = 0;
+    if (clear && x < end) {
+      H[r1.z] = kTombKey;
+      H[r2.z] = kTombKey;
+      E[i] = make_rec(e3, p3 & mask);  // (no slot, a full table, was reported: stay in bounds)
+      E[j] = make_rec(e4, p4 & mask);
+      tombs = 2u - t3 - t4;
+      ++acc;
+    } else if (clear) {  // past the end: its insertions become tombstones
+      if (p3 != kNil) {
+        H[p3] = kTombKey;
+        tombs += 1u - t3;
+      }
+      if (p4 != kNil) {
+        H[p4] = kTombKey;
+        tombs += 1u - t4;
+      }
+    }
+    if (x < end && !clear) {
+      if (code == kCodeLoop) ++rej_loop;
+      else ++rej_exists;  // a shared node (the targets re-create the sources) or a present target
+    }
+    if (end < n) load_window(s + end);
+    find_cut(&s_cut[par ^ 1]);
+    tombs = __reduce_add_sync(0xffffffffu, tombs);
+    if ((tid & 31u) == 0 && tombs) {
+      tomb_total += tombs;
+      atomicAdd(&s_mine[par], tombs);
+    }
+    if (tid == 0) {
+      // the superstep before this one's tombstones to every CTA, and its words
+      // for the next one
+      const uint32_t mine = s_mine[par ^ 1];
+      if (mine) all_add(&s_tombs, mine);
+      s_mine[par ^ 1] = s_events[par ^ 1] = s_asked[par ^ 1] = 0;
+      s_end[par ^ 1] = B;
+    }
+    s += end;
+    ++steps;
+    met += events;
+    cluster_sync();
+    if (s >= nsw) break;
+    if (s_tombs > limit) {  // a rebuild on the whole GPU is cheap: keep the probe chains short
+      stop = 1;             // (the same in every CTA)
+      break;
+    }
+    if (steps >= 4 && met > kBusyEvents * steps) {
+      stop = 2;
+      break;
+    }
+  }
+  if (tomb_total) atomicAdd(&job.tombs, tomb_total);
+  if (x == 0) {  // progress of the job (the host launches it again while stopped)
+    job.done = s;
+    job.stopped = stop;
+    if (stop == 2) job.alone = 1;
+    if (stop) atomicAdd(nstop, 1u);
+  }
+  // counts of this job
+  const unsigned a32 = __reduce_add_sync(0xffffffffu, acc);
+  const unsigned l32 = __reduce_add_sync(0xffffffffu, rej_loop);
+  const unsigned r32 = __reduce_add_sync(0xffffffffu, rej_exists);
+  if ((tid & 31) == 0) {
+    if (a32) {
+      atomicAdd(&stats->accepted, (unsigned long long)a32);
+      atomicAdd(&chain_acc[job.chain], (unsigned long long)a32);
+    }
+    if (l32) atomicAdd(&stats->rej_loop, (unsigned long long)l32);
+    if (r32) atomicAdd(&stats->rej_exists, (unsigned long long)r32);
+  }
+}
+
 // Windows of 32, 128 and 256 switches (the set rebuilt in place).
 template <int B, int MIN_BLOCKS>
 __global__ void __launch_bounds__(B, MIN_BLOCKS) k_es_run(EsJob *jobs, uint32_t job_off, uint32_t nsw,
@@ -666,8 +1008,8 @@ __global__ void __launch_bounds__(B, MIN_BLOCKS) k_es_run(EsJob *jobs, uint32_t 
   es_run_body<B, false>(jobs, job_off, nsw, samples, dists, stats, chain_acc, err, nullptr);
 }
 
-// Windows of 1024 switches (chains of at least 2^19 edges: the set rebuilt
-// on the whole GPU between launches).
+// Windows of 1024 switches on one CTA (chains of at least 2^19 edges that the
+// cluster left: the set rebuilt on the whole GPU between launches).
 __global__ void __launch_bounds__(1024, 1) k_es_run_big(EsJob *jobs, uint32_t job_off, uint32_t nsw,
                                                         const uint2 *samples, const uint16_t *dists, StatsDev *stats,
                                                         unsigned long long *chain_acc, uint32_t *err,
@@ -719,8 +1061,8 @@ cudaError_t launch_es_sample(EsJob *jobs, const uint32_t (&group)[4], unsigned l
 
 cudaError_t launch_es_run(EsJob *jobs, const uint32_t (&group)[4], uint32_t nsw, const uint2 *samples,
                           const uint16_t *dists, StatsDev *stats, unsigned long long *chain_acc, uint32_t *err,
-                          uint32_t *nstop, cudaStream_t s, cudaStream_t s2, cudaEvent_t fork, cudaEvent_t join,
-                          uint32_t *launches) {
+                          uint32_t *nstop, bool alone, cudaStream_t s, cudaStream_t s2, cudaEvent_t fork,
+                          cudaEvent_t join, uint32_t *launches) {
   // group[w] jobs with windows of 1024, 256, 128 and 32 switches, in that
   // order; the two small-window groups run on s2 (after s, and joined back
   // into s) when there is one, beside the others
@@ -734,16 +1076,22 @@ cudaError_t launch_es_run(EsJob *jobs, const uint32_t (&group)[4], uint32_t nsw,
   auto run = [&](int w, cudaStream_t st) {
     for (uint32_t off = beg[w]; off < beg[w + 1]; off += 65535u, ++n) {
       const uint32_t nj = beg[w + 1] - off < 65535u ? beg[w + 1] - off : 65535u;
-      if (w == 0)
-        k_es_run_big<<<nj, 1024, EsShape<1024>::kBytes, st>>>(jobs, off, nsw, samples, dists, stats, chain_acc, err,
-                                                              nstop);
-      else if (w == 1)
+      if (w == 0) {
+        k_es_run_cluster<1024 / kClusterCtas><<<nj * kClusterCtas, 1024 / kClusterCtas, 0, st>>>(
+            jobs, off, nsw, samples, dists, stats, chain_acc, err, nstop);
+        if (alone) {
+          k_es_run_big<<<nj, 1024, EsShape<1024>::kBytes, st>>>(jobs, off, nsw, samples, dists, stats, chain_acc, err,
+                                                                nstop);
+          ++n;
+        }
+      } else if (w == 1) {
         k_es_run<256, 6><<<nj, 256, EsShape<256>::kBytes, st>>>(jobs, off, nsw, samples, dists, stats, chain_acc, err);
-      else if (w == 2)
+      } else if (w == 2) {
         k_es_run<128, 12><<<nj, 128, EsShape<128>::kBytes, st>>>(jobs, off, nsw, samples, dists, stats, chain_acc,
                                                                  err);
-      else
+      } else {
         k_es_run<32, 32><<<nj, 32, EsShape<32>::kBytes, st>>>(jobs, off, nsw, samples, dists, stats, chain_acc, err);
+      }
     }
   };
   run(3, ss);

@@ -330,8 +330,8 @@ struct EsJob {
   uint32_t row;      // place of the job's samples among the batch's
   uint32_t done;     // switches of the batch that have run
   uint32_t tombs;    // tombstones in the set
-  uint32_t stopped;  // the kernel stopped this job for a rebuild of its set on the whole GPU
-  uint32_t pad;
+  uint32_t stopped;  // the kernel stopped this job: 1 for a rebuild of its set on the whole GPU, 2 for the other kernel
+  uint32_t alone;    // run on one CTA (largest window)
 };
 
 // Shared-memory opt-in of the ParES kernels, once per device.
@@ -352,12 +352,13 @@ cudaError_t launch_es_sample(EsJob *jobs, const uint32_t (&group)[4], unsigned l
 // with 128 and group[3] with 32 (these two on s2, forked from and joined back
 // into s through the two events, if given).  *launches receives the number of
 // launches.
-// Jobs of the largest window stop when their set needs a rebuild (counted
-// in *nstop); the caller rebuilds those sets and launches again.
+// Jobs of the largest window run on a cluster of CTAs; they stop when their
+// set needs a rebuild, or to go on alone on one CTA (counted in *nstop); the
+// caller rebuilds those sets and launches again (alone: some job may).
 cudaError_t launch_es_run(EsJob *jobs, const uint32_t (&group)[4], uint32_t nsw, const uint2 *samples,
                           const uint16_t *dists, StatsDev *stats, unsigned long long *chain_acc, uint32_t *err,
-                          uint32_t *nstop, cudaStream_t s, cudaStream_t s2, cudaEvent_t fork, cudaEvent_t join,
-                          uint32_t *launches);
+                          uint32_t *nstop, bool alone, cudaStream_t s, cudaStream_t s2, cudaEvent_t fork,
+                          cudaEvent_t join, uint32_t *launches);
 // Lists of the chains with a job (job_of[chain] != kNoChain) out of their
 // slots into the jobs' position-order lists, and back (slots in position
 // order, nothing pending).

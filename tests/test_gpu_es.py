@@ -193,3 +193,19 @@ def test_calls_longer_than_a_batch_of_samples(m, switches):
     n = max(8, int(3 * m ** 0.5) + 8)
     edges = inputs.random_simple_graph(n, m, seed=m + 3)
     es_compare(edges, n, seed=m, calls=[switches])
+
+
+@pytest.mark.slow
+@pytest.mark.parametrize("kind", ["sparse", "hubs", "dense"])
+def test_large_chains_on_a_cluster(kind):
+    # chains of at least 2^19 edges: sparse (supersteps nearly without
+    # dependencies), with hubs (two switches with the same target) and dense
+    # (most targets present, many of them erased in the same superstep)
+    if kind == "sparse":
+        edges, n = inputs.gnp(1 << 17, 9.0 / ((1 << 17) - 1), seed=3), 1 << 17
+    elif kind == "hubs":
+        edges, n = inputs.pld_graph(400_000, 2.05, 1, 8000, seed=5), 400_000
+    else:
+        edges, n = inputs.gnp(1200, 0.8, seed=4), 1200
+    assert len(edges) >= 1 << 19
+    es_compare(edges, n, seed=13, calls=[1, 5000, 150_000])
