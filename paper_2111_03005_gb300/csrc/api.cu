@@ -295,6 +295,7 @@ struct gesmc_pool_ctx {
   int broken = 0;
   RoundArgs args;
   uint64_t args_version = 1;  // bumped whenever args change (invalidates the graph)
+  bool waves_known = false;   // some round has run
   uint32_t wave_kernels = 0;  // whole-GPU wave kernel pairs per round (grows with the wide waves seen)
   // captured rounds (a CUDA graph of kGraphRounds rounds), replayed on gstream
   bool use_graphs = true;
@@ -332,6 +333,10 @@ struct gesmc_pool_ctx {
 // pools whose arguments stay.
 constexpr uint32_t kGraphRounds = 4;
 constexpr uint64_t kGraphAfterRounds = 16;
+// Fewer switches hardly ever have a wide wave (more than 2048 of them), and in
+// fewer rounds the wait would cost more than it gives.
+constexpr uint64_t kLearnRounds = 4;
+constexpr uint32_t kLearnSwitches = 1u << 15;
 
 struct gesmc_ctx {
   gesmc_pool_t pool = nullptr;
@@ -706,11 +711,22 @@ int pool_add_device(gesmc_pool_t p, unsigned long long *E, uint64_t m, uint64_t 
   return GESMC_OK;
 }
 
+// Waves after the first that many switches entered in the last round: run as
+// many on the whole GPU from now on.
+void learn_waves(gesmc_pool_t p, const Counters &ctl) {
+  p->waves_known = true;
+  const uint32_t want = std::min<uint32_t>(ctl.wide, kMaxWaveKernels);
+  if (want > p->wave_kernels) {
+    p->wave_kernels = want;
+    refresh_args(p);
+  }
+}
+
 int pool_run(gesmc_pool_t p, uint64_t rounds) {
   if (p->broken) return p->broken;
   DeviceGuard g(p->device);
   cudaStream_t s = p->stream;
-  const RoundArgs a = p->args;
+  RoundArgs a = p->args;
   // (the device's error word is zero: a call that sets it breaks the pool)
   const size_t per_round = kNumStages + 1;
   const bool stage_events = p->profiling && !p->resident;  // resident rounds have no separate stages
@@ -780,7 +796,8 @@ int pool_run(gesmc_pool_t p, uint64_t rounds) {
       const uint32_t r = (uint32_t)std::min<uint64_t>(per_launch, rounds - done);
       const bool final = done + r == rounds;
       nvtxRangePushA("gesmc resident rounds");
-      bool ok = cudaMemsetAsync(scratch, 0, 4ull * (r + kWaveHist), s) == cudaSuccess;
+      // (where permutations come first, their kernel zeroes the words)
+      bool ok = presort || cudaMemsetAsync(scratch, 0, 4ull * (r + kWaveHist), s) == cudaSuccess;
       uint16_t *pbuf = presort ? reinterpret_cast<uint16_t *>(a.prec) : nullptr;
       uint32_t *ebuf = presort ? reinterpret_cast<uint32_t *>(pbuf + (uint64_t)r * njobs * pstride) : nullptr;
       ok = ok && launch_round_resident(a, at<uint32_t>(p->base, p->lay.es_job_of), p->res_count, p->res_max_m, r,
@@ -872,12 +889,29 @@ int pool_run(gesmc_pool_t p, uint64_t rounds) {
         after = true;
       }
     };
-    const uint64_t lead = p->warm_rounds < kGraphAfterRounds ? std::min(rounds, kGraphAfterRounds - p->warm_rounds) : 0;
+    // A pool that has not run yet does not know which of its rounds' waves are
+    // wide, and its first call would run them all on one CTA: ask after one
+    // round (a power law of 7.8e5 edges, 20 rounds: 2.90 -> 2.45 ms).
+    uint64_t done = 0;  // rounds launched so far
+    if (ok && side && !p->waves_known && rounds >= kLearnRounds && a.switch_hw >= kLearnSwitches) {
+      direct(0, 1);
+      done = 1;
+      Counters ctl;
+      ok = ok && cudaMemcpyAsync(&ctl, a.ctl, sizeof(Counters), cudaMemcpyDeviceToHost, gs) == cudaSuccess &&
+           cudaStreamSynchronize(gs) == cudaSuccess;
+      if (ok) {
+        learn_waves(p, ctl);
+        a = p->args;
+        p->warm_version = p->args_version;
+      }
+      after = false;
+    }
+    const uint64_t first = done, left = rounds - done;
+    const uint64_t lead = p->warm_rounds < kGraphAfterRounds ? std::min(left, kGraphAfterRounds - p->warm_rounds) : 0;
     const bool have = p->gexec && p->graph_version == p->args_version;
-    uint64_t done = rounds;  // rounds launched directly before the graph's
-    if (side && rounds - lead >= (have ? kGraphRounds : kGraphAfterRounds)) {
-      done = lead;
-      direct(0, done);
+    if (side && left - lead >= (have ? kGraphRounds : kGraphAfterRounds)) {
+      done = first + lead;
+      direct(first, done);
       if (ok && !have) {
         if (p->gexec) cudaGraphExecDestroy(p->gexec);
         p->gexec = nullptr;
@@ -906,7 +940,7 @@ int pool_run(gesmc_pool_t p, uint64_t rounds) {
       after = false;  // a graph launch ended: nothing to overlap with
       direct(done, rounds);
     } else {
-      direct(0, rounds);
+      direct(first, rounds);
     }
     if (side && ok)
       ok = cudaEventRecord(p->ev_out, gs) == cudaSuccess && cudaStreamWaitEvent(s, p->ev_out, 0) == cudaSuccess;
@@ -943,12 +977,7 @@ int pool_run(gesmc_pool_t p, uint64_t rounds) {
   p->switches_run += rounds * sw;
   const int rc = map_device_errors(ctl.err);
   if (rc != GESMC_OK) p->broken = rc;
-  // waves after the first that many switches entered: run as many on the whole GPU from now on
-  const uint32_t want = std::min<uint32_t>(ctl.wide, kMaxWaveKernels);
-  if (rc == GESMC_OK && want > p->wave_kernels) {
-    p->wave_kernels = want;
-    refresh_args(p);
-  }
+  if (rc == GESMC_OK) learn_waves(p, ctl);
   return rc;
 }
 

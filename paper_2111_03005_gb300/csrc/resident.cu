@@ -71,6 +71,7 @@ struct ResidentJob {
   uint16_t *pbuf;
   uint32_t *ebuf;
   uint32_t pstride, njobs, job_base;
+  uint32_t first;  // the first class's launch
 };
 
 // Byte offsets of a chain's pieces of shared memory (all grow with m).
@@ -380,7 +381,11 @@ __global__ void __launch_bounds__(T, 1024 / T) k_round_resident(RoundArgs a, Res
   const uint32_t c = job.jobs[blockIdx.x];
   const ChainDesc &ch = a.chains[c];
   const uint32_t m = ch.m, L = ch.L;
-  dep_launch();
+  // after the permutations' launch, the first class's kernel waits for it before
+  // the rounds and only then lets the next class start, so that no class
+  // starts before them
+  const bool after_perms = kPre && job.first;
+  if (!after_perms) dep_launch();
   if (m < 2 || m > kResidentMaxEdges) {  // the host sends only chains that qualify
     dep_wait();
     return;
@@ -432,6 +437,10 @@ __global__ void __launch_bounds__(T, 1024 / T) k_round_resident(RoundArgs a, Res
   uint32_t acc = 0, rloop = 0, rexist = 0, rlazy = 0;  // this thread's tallies
   const bool exact = ch.exact_ell && ch.lazy_threshold;
   uint32_t err = 0;
+  if (after_perms) {
+    dep_wait();
+    dep_launch();
+  }
   constexpr uint32_t KS = ResPer<T>::kSwitches, KP = ResPer<T>::kPermVec;
   // a permutation sorted beforehand is loaded a round ahead, into registers
   const uint32_t nvec = (m + 7) / 8;
@@ -764,6 +773,8 @@ __global__ void __launch_bounds__(T, 1024 / T) k_resident_perm(RoundArgs a, Resi
   __shared__ uint32_t s_warp[32];
   __shared__ uint32_t s_ell;
   dep_launch();
+  if (blockIdx.x == 0 && blockIdx.y == 0 && job.first)  // (the host zeroes them where no permutations come first)
+    for (uint32_t w = threadIdx.x; w < job.rounds + kWaveHist; w += T) job.last_pending[w] = 0;
   const ChainDesc ch = a.chains[job.jobs[blockIdx.x]];
   const uint32_t m = ch.m;
   if (m < 2 || m > kResidentMaxEdges) {
@@ -796,6 +807,7 @@ __host__ __device__ inline uint32_t perm_smem_bytes(uint32_t m) {
 // The launch's rounds into the statistics (each round's wave count is the
 // largest over its chains, as in the general path) and the pool round on.
 __global__ void k_resident_fold(RoundArgs a, ResidentJob job) {
+  dep_wait();
   __shared__ unsigned long long hist[kWaveHist];
   __shared__ unsigned long long total, most;
   const uint32_t tid = threadIdx.x;
@@ -831,9 +843,9 @@ __global__ void k_resident_fold(RoundArgs a, ResidentJob job) {
 // threads).
 constexpr uint32_t kClassMaxEdges[kResidentClasses] = {kResidentMaxEdges, 4096, 2048, 1024};
 
-// One class's kernel.  `beside`: it need not wait for the launch before it,
-// another class's, and starts as soon as that one's CTAs are all on the GPU
-// (programmatic dependent launch).  Every kernel launched so waits for the one
+// One class's kernel.  `beside`: it need not wait to start for the launch
+// before it, another class's, and does as soon as that one's CTAs are all on the
+// GPU (programmatic dependent launch).  Every kernel launched so waits for the one
 // before it just before it ends, so what follows the last class follows all.
 // 50 rounds of 1024 chains of 100 to 9,600 edges: 6.2 ms with one class after
 // another, 4.4 ms beside each other (the largest class has one CTA an SM and
@@ -917,7 +929,8 @@ cudaError_t launch_round_resident(const RoundArgs &a, const uint32_t *jobs, cons
       if (!count[c]) continue;
       j.jobs = jobs + off;
       j.job_base = off;
-      const bool beside = off > 0;
+      const bool beside = off > 0 || (pbuf && !perms);
+      j.first = off == 0 ? 1u : 0u;
       off += count[c];
       cudaError_t e = cudaSuccess;
       switch (c) {
@@ -931,9 +944,8 @@ cudaError_t launch_round_resident(const RoundArgs &a, const uint32_t *jobs, cons
     }
   }
   j.jobs = jobs;
-  k_resident_fold<<<1, 256, 0, s>>>(a, j);
   ++*launches;
-  return cudaGetLastError();
+  return launch_beside(k_resident_fold, dim3(1), 256, 0, s, j.njobs > 0, a, j);
 }
 
 }  // namespace gesmc

@@ -36,7 +36,8 @@ cudaError_t prepare_resident();
 // run `rounds` rounds from the pool's current round, one CTA each (one
 // launch per class), then a one-CTA kernel folds the rounds' wave counts
 // into the statistics and advances the pool round.  round_waves (rounds
-// words) and last_pending (kWaveHist words) must be zero; `final` says
+// words) and last_pending (kWaveHist words, right before them) must be zero
+// unless pbuf is given; `final` says
 // whether the call's last round is in this launch (its per-wave undecided
 // counts become the statistics' last-round counts).  pbuf (optional): room
 // for rounds x jobs permutations of pstride u16 each (pstride >= the largest
