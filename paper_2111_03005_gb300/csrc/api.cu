@@ -163,7 +163,7 @@ Layout pool_layout(const Capacity &c, uint64_t M, uint64_t C) {
   l.list0 = take(4 * c.switches);
   l.list1 = take(4 * c.switches);
   l.ptup = take(16 * c.tuples);
-  l.otup = take(std::max<uint64_t>(16 * c.ovf, 4096));  // at least a few hundred samples of ParES
+  l.otup = take(std::max<uint64_t>(16 * c.ovf, 65536));  // at least a few thousand samples of ParES
   l.tcount = take(4 * c.tcounts);
   l.ocount = take(4 * c.parts);
   l.ooff = take(4 * (c.parts + 1));
@@ -1005,6 +1005,7 @@ int pool_es_run(gesmc_pool_t p, uint64_t switches, uint32_t only) {
     jb.seed = hc.d.seed;
     jb.k0 = hc.es_next;
     jb.chain = c;
+    jb.n = (uint32_t)std::min<uint64_t>(hc.n, 0xFFFFFFFFull);
     if (jb.m >= 2) {
       // the list (position order, 16 bytes per edge) in the chain's tuple
       // storage (at least 32 bytes per edge), the edge set in its permutation records (at least
@@ -1018,25 +1019,27 @@ int pool_es_run(gesmc_pool_t p, uint64_t switches, uint32_t only) {
       while ((16ull << hlog2) <= hbytes && hlog2 < 31) ++hlog2;  // largest 2^h with 8 * 2^h <= room
       if ((1ull << hlog2) < 2ull * jb.m) return GESMC_E_INTERNAL;
       jb.E = reinterpret_cast<uint4 *>(base);
-      jb.H = reinterpret_cast<unsigned long long *>(hbase);
+      // (a small chain has its set in shared memory)
+      jb.H = es_group(jb.m, hc.n) >= 4 ? nullptr : reinterpret_cast<unsigned long long *>(hbase);
       jb.hlog2 = hlog2;
     }
     jobs.push_back(jb);
   }
   if (jobs.empty()) return GESMC_OK;
-  // chains by window size, largest windows first (each group keeps chain
-  // order); chains with m < 2 have no list to move (their switches are only
+  // chains by group, largest windows first (each group keeps chain order); chains with m < 2 have no list to move (their switches are only
   // counted)
+  auto group_of = [p](const EsJob &x) { return es_group(x.m, p->chains[x.chain].n); };
   std::stable_sort(jobs.begin(), jobs.end(),
-                   [](const EsJob &x, const EsJob &y) { return es_window(x.m) > es_window(y.m); });
-  uint32_t group[4] = {0, 0, 0, 0}, rows = 0;
+                   [&](const EsJob &x, const EsJob &y) { return group_of(x) < group_of(y); });
+  uint32_t group[kEsGroups] = {}, smem_of[kEsGroups] = {}, rows = 0;
   for (uint32_t t = 0; t < jobs.size(); ++t) {
     if (jobs[t].m >= 2) {
       job_of[jobs[t].chain] = t;
       jobs[t].row = rows++;
     }
-    const uint32_t w = es_window(jobs[t].m);
-    ++group[w == 1024u ? 0 : w == 256u ? 1 : w == 128u ? 2 : 3];
+    const uint32_t w = group_of(jobs[t]);
+    ++group[w];
+    if (w >= 4) smem_of[w] = std::max(smem_of[w], es_smem_bytes(jobs[t].m, jobs[t].n));
   }
   EsJob *djobs = at<EsJob>(p->base, p->lay.es_jobs);
   uint32_t *djob_of = at<uint32_t>(p->base, p->lay.es_job_of);
@@ -1067,10 +1070,11 @@ int pool_es_run(gesmc_pool_t p, uint64_t switches, uint32_t only) {
     // job is done (each launch advances every stopped job by a superstep at
     // least)
     for (uint64_t iter = 0; ok; ++iter) {
-      const uint32_t groups[4] = {group[0], iter ? 0u : group[1], iter ? 0u : group[2], iter ? 0u : group[3]};
+      uint32_t groups[kEsGroups] = {group[0]};
+      for (uint32_t w = 1; w < kEsGroups && iter == 0; ++w) groups[w] = group[w];
       if (group[0]) ok &= cudaMemsetAsync(nstop, 0, sizeof(uint32_t), s) == cudaSuccess;
       // (a job that went on alone does so for the rest of the call)
-      ok &= launch_es_run(djobs, groups, n, samples, dists, a.st, a.chain_accepted, err, nstop, iter > 0 || off > 0, s,
+      ok &= launch_es_run(djobs, groups, smem_of, n, samples, dists, a.st, a.chain_accepted, err, nstop, iter > 0 || off > 0, s,
                           p->gstream, p->ev_in, p->ev_out, &run_launches) == cudaSuccess;
       p->launches += run_launches;
       if (!ok || group[0] == 0) break;  // only the largest windows stop

@@ -80,6 +80,24 @@ __device__ __forceinline__ uint32_t tau_g(uint32_t g, unsigned long long e1, uns
   return 0;
 }
 
+// ---------------------------------------------------------------- 16-bit node ids
+// Canonical 32-bit id of the edge {a, b}: smaller node in the high half.
+__device__ __forceinline__ uint32_t pack16(uint32_t a, uint32_t b) {
+  return a < b ? (a << 16) | b : (b << 16) | a;
+}
+
+// tau of Def. 1 on packed edges (the same rules as tau_g): targets e3, e4
+// and the outright-reject code (1: a loop, 2: sources sharing a node).
+__device__ __forceinline__ uint32_t tau16(uint32_t g, uint32_t e1, uint32_t e2, uint32_t &e3, uint32_t &e4) {
+  const uint32_t u = e1 >> 16, v = e1 & 0xFFFFu, x = e2 >> 16, y = e2 & 0xFFFFu;
+  const uint32_t a3 = u, b3 = g ? y : x, a4 = v, b4 = g ? x : y;
+  e3 = pack16(a3, b3);
+  e4 = pack16(a4, b4);
+  if (a3 == b3 || a4 == b4) return 1u;
+  if (u == x || u == y || v == x || v == y) return 2u;
+  return 0;
+}
+
 // ---------------------------------------------------------------- dependent launches
 // Programmatic dependent launch: let the next kernel of the stream start
 // (once every CTA of this one has called this or exited), and wait for the

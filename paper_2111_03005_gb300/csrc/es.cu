@@ -233,7 +233,7 @@ __device__ __forceinline__ bool window_any(bool x) {
 // H <- empty, for every job (blockIdx.y = job).
 __global__ void k_es_clear(EsJob *jobs, uint32_t job_off, bool only_stopped) {
   const EsJob &jb = jobs[job_off + blockIdx.y];
-  if (jb.m < 2 || (only_stopped && jb.stopped != 1)) return;  // no list, no set; or a set that needs no rebuild
+  if (!jb.H || (only_stopped && jb.stopped != 1)) return;  // no list, no set; or a set that needs no rebuild
   const unsigned long long cap = 1ull << jb.hlog2;
   const unsigned long long nth = (unsigned long long)gridDim.x * blockDim.x;
   unsigned long long *const H = jb.H;
@@ -245,7 +245,7 @@ __global__ void k_es_clear(EsJob *jobs, uint32_t job_off, bool only_stopped) {
 // H <- the entries of E, each entry's slot into the list.
 __global__ void k_es_fill(const EsJob *jobs, uint32_t job_off, uint32_t *err, bool only_stopped) {
   const EsJob jb = jobs[job_off + blockIdx.y];
-  if (jb.m < 2 || (only_stopped && jb.stopped != 1)) return;
+  if (!jb.H || (only_stopped && jb.stopped != 1)) return;
   const uint32_t mask = (uint32_t)((1ull << jb.hlog2) - 1);
   for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < jb.m; s += gridDim.x * blockDim.x) {
     const unsigned long long e = rec_edge(jb.E[s]);
@@ -659,6 +659,371 @@ __device__ __forceinline__ void es_run_body(EsJob *jobs, uint32_t job_off, uint3
   }
 }
 
+// ---------------------------------------------------------------- small chains
+// Chains of few edges or nodes, one warp each with the list and the set in
+// shared memory (16-bit node ids: a word per edge).
+// Their supersteps hold a handful of switches (five in a chain of 65 edges), so
+// a pool's time is that of its smallest chains' dependent accesses: with list
+// and set in L1 and L2 a superstep took 2.6 us, with the bits 0.35 (a chain of
+// 1,000 edges: 6.0 and 0.6; with a hash table in shared memory 2.8: its loops
+// are what takes the instructions).  As on the cluster
+// below, a superstep ends before a switch that depends on an earlier one (the
+// same target, found where both insert it, or a present target that an earlier
+// switch erases, found by its slot), so it needs no tables and waves.
+// Chains whose pairs of nodes fit as bits have the set as a bit matrix (no search,
+// no tombstones), others of at most kEsSmallestEdges edges as a hash table.  The
+// bit matrices run in three launches, by the shared memory they need (nine,
+// three and one CTA an SM).
+constexpr uint32_t kEsSmallestEdges = 2048;
+constexpr uint32_t kEsBitMax = 220 << 10, kEsBitBytes[3] = {24 << 10, 72 << 10, kEsBitMax};
+// Bytes of the bits of all pairs below n nodes and of a list of m edges.
+__host__ __device__ inline unsigned long long bits_bytes(uint32_t m, unsigned long long n) {
+  return 4 * ((n * (n - 1) / 2 + 31) / 32 + m);
+}
+constexpr uint32_t kEmpty32 = 0xFFFFFFFFu, kTomb32 = 0xFFFFFFFEu;  // no edges (not canonical)
+
+__host__ __device__ inline uint32_t small_log2(uint32_t m) {  // at least four slots per edge
+  uint32_t h = 10;
+  while ((1u << h) < 4 * m) ++h;
+  return h;
+}
+
+// Samples of a warp's chain, 32 a register: the window at s from the first two by
+// shuffles, the third on its way (loaded where they are used, they would cost
+// an access to L2 or memory a superstep).
+struct SampleRing {
+  uint2 c[3];
+  uint32_t d[3], base;
+  __device__ __forceinline__ void load(int v, uint32_t from, uint32_t nsw, const uint2 *samp, const uint16_t *dist) {
+    c[v] = make_uint2(0, 0);
+    d[v] = 0xFFFFu;
+    const uint32_t k = from + threadIdx.x;
+    if (k < nsw) {
+      c[v] = __ldg(&samp[k]);
+      d[v] = __ldg(&dist[k]);
+    }
+  }
+  __device__ __forceinline__ void start(uint32_t nsw, const uint2 *samp, const uint16_t *dist) {
+    base = 0;
+#pragma unroll
+    for (int v = 0; v < 3; ++v) load(v, 32 * v, nsw, samp, dist);
+  }
+  // The lane's switch of the window at s (at most 32 past the last one) and its distance.
+  __device__ __forceinline__ uint2 window(uint32_t s, uint32_t nsw, const uint2 *samp, const uint16_t *dist,
+                                          uint32_t &dd) {
+    if (s - base >= 32) {
+      c[0] = c[1];
+      d[0] = d[1];
+      c[1] = c[2];
+      d[1] = d[2];
+      base += 32;
+      load(2, base + 64, nsw, samp, dist);
+    }
+    const uint32_t at = s - base + threadIdx.x;
+    const uint32_t x0 = __shfl_sync(0xffffffffu, c[0].x, at), y0 = __shfl_sync(0xffffffffu, c[0].y, at);
+    const uint32_t x1 = __shfl_sync(0xffffffffu, c[1].x, at), y1 = __shfl_sync(0xffffffffu, c[1].y, at);
+    const uint32_t e0 = __shfl_sync(0xffffffffu, d[0], at), e1 = __shfl_sync(0xffffffffu, d[1], at);
+    dd = at < 32 ? e0 : e1;
+    return at < 32 ? make_uint2(x0, y0) : make_uint2(x1, y1);
+  }
+};
+
+// The list of a small chain into shared memory (a word per edge), and back.
+__device__ __forceinline__ void load_small(uint32_t *E, const uint4 *list, uint32_t m) {
+#pragma unroll 8
+  for (uint32_t t = threadIdx.x; t < m; t += 32) {
+    const uint2 r = *reinterpret_cast<const uint2 *>(&list[t]);
+    E[t] = (r.y << 16) | (r.x & 0xFFFFu);
+  }
+}
+__device__ __forceinline__ void store_small(uint4 *list, const uint32_t *E, uint32_t m) {
+  for (uint32_t t = threadIdx.x; t < m; t += 32) list[t] = make_uint4(E[t] & 0xFFFFu, E[t] >> 16, 0u, 0u);
+}
+
+// A warp's counts of its chain's switches.
+__device__ __forceinline__ void count_small(const EsJob &job, uint32_t acc, uint32_t rej_loop, uint32_t rej_exists,
+                                            StatsDev *stats, unsigned long long *chain_acc) {
+  const unsigned a32 = __reduce_add_sync(0xffffffffu, acc);
+  const unsigned l32 = __reduce_add_sync(0xffffffffu, rej_loop);
+  const unsigned r32 = __reduce_add_sync(0xffffffffu, rej_exists);
+  if (threadIdx.x == 0) {
+    if (a32) {
+      atomicAdd(&stats->accepted, (unsigned long long)a32);
+      atomicAdd(&chain_acc[job.chain], (unsigned long long)a32);
+    }
+    if (l32) atomicAdd(&stats->rej_loop, (unsigned long long)l32);
+    if (r32) atomicAdd(&stats->rej_exists, (unsigned long long)r32);
+  }
+}
+
+// The set as a bit matrix: the bit of {u, v}, u < v, at v (v - 1) / 2 + u.
+__global__ void __launch_bounds__(32) k_es_run_bits(EsJob *jobs, uint32_t job_off, uint32_t nsw, const uint2 *samples,
+                                                    const uint16_t *dists, StatsDev *stats,
+                                                    unsigned long long *chain_acc, uint32_t *err) {
+  extern __shared__ uint32_t small_dyn[];
+  dep_launch();
+  const EsJob &job = jobs[job_off + blockIdx.x];
+  const uint32_t x = threadIdx.x, m = job.m;
+  if (m >= 2 && bits_bytes(m, job.n) <= kEsBitMax) {  // the host sends only chains that qualify
+    const uint32_t words = (job.n * (job.n - 1) / 2 + 31) / 32;
+    uint32_t *const M = small_dyn, *const E = M + words;
+    const uint2 *const samp = samples + (size_t)job.row * nsw;
+    const uint16_t *const dist = dists + (size_t)job.row * nsw;
+    SampleRing ring;
+    ring.start(nsw, samp, dist);
+    load_small(E, job.E, m);
+    for (uint32_t t = x; t < words; t += 32) M[t] = 0;
+    __syncwarp();
+    auto pair = [](uint32_t e) {  // (0 for the 0 of a lane without a switch)
+      const uint32_t v = e & 0xFFFFu;
+      return v * (v - 1) / 2 + (e >> 16);
+    };
+    for (uint32_t t = x; t < m; t += 32) {
+      const uint32_t b = pair(E[t]);
+      atomicOr(&M[b >> 5], 1u << (b & 31u));
+    }
+    __syncwarp();
+    uint32_t acc = 0, rej_loop = 0, rej_exists = 0;
+    for (uint32_t s = 0; s < nsw;) {
+      uint32_t d;
+      const uint2 cur = ring.window(s, nsw, samp, dist, d);
+      uint32_t n = min(32u, nsw - s);
+      const unsigned hit = __ballot_sync(0xffffffffu, d <= x);
+      if (hit) n = min(n, (uint32_t)__ffs(hit) - 1);
+      const uint32_t i = cur.x, j = cur.y & 0x7FFFFFFFu, g = cur.y >> 31;
+      uint32_t e1 = 0, e2 = 0, e3 = 0, e4 = 0, code = kCodeLazy;
+      if (x < n) {
+        e1 = E[i];
+        e2 = E[j];
+        code = tau16(g, e1, e2, e3, e4);
+      }
+      const bool live = code == 0;
+      const uint32_t i3 = pair(e3), i4 = pair(e4), w3 = i3 >> 5, w4 = i4 >> 5;
+      const uint32_t b3 = 1u << (i3 & 31u), b4 = 1u << (i4 & 31u);
+      bool p3 = false, p4 = false;  // present
+      if (live) {
+        p3 = (M[w3] & b3) != 0;
+        p4 = (M[w4] & b4) != 0;
+      }
+      // the superstep ends before the first switch with a present target that
+      // an earlier one erases
+      uint32_t end = n;
+      for (unsigned who = __ballot_sync(0xffffffffu, p3 || p4); who; who &= who - 1) {
+        const int w = __ffs(who) - 1;
+        const uint32_t k3 = __shfl_sync(0xffffffffu, p3 ? e3 : 0u, w), k4 = __shfl_sync(0xffffffffu, p4 ? e4 : 0u, w);
+        const bool erases = live && (int)x < w && (e1 == k3 || e2 == k3 || e1 == k4 || e2 == k4);
+        if (__any_sync(0xffffffffu, erases)) {
+          end = min(end, (uint32_t)w);
+          break;
+        }
+      }
+      const bool clear = live && !p3 && !p4 && x < end;
+      __syncwarp();
+      bool o3 = false, o4 = false;  // this lane set the bit
+      if (clear) {
+        o3 = !(atomicOr(&M[w3], b3) & b3);
+        o4 = !(atomicOr(&M[w4], b4) & b4);
+      }
+      // a bit that another lane has set: the superstep ends before this switch
+      const unsigned two = __ballot_sync(0xffffffffu, clear && !(o3 && o4));
+      if (two) {
+        end = min(end, max(1u, (uint32_t)__ffs(two) - 1));
+        if (clear && x >= end) {  // what it set is taken back
+          if (o3) atomicAnd(&M[w3], ~b3);
+          if (o4) atomicAnd(&M[w4], ~b4);
+        }
+        __syncwarp();
+        if (clear && x == 0) {  // (the first switch always runs: another's bit may have been its own)
+          atomicOr(&M[w3], b3);
+          atomicOr(&M[w4], b4);
+        }
+      }
+      if (x < end) {
+        if (clear) {
+          const uint32_t i1 = pair(e1), i2 = pair(e2);
+          atomicAnd(&M[i1 >> 5], ~(1u << (i1 & 31u)));
+          atomicAnd(&M[i2 >> 5], ~(1u << (i2 & 31u)));
+          E[i] = e3;
+          E[j] = e4;
+          ++acc;
+        } else if (code == kCodeLoop) {
+          ++rej_loop;
+        } else {
+          ++rej_exists;
+        }
+      }
+      s += end;
+      __syncwarp();
+    }
+    store_small(job.E, E, m);
+    count_small(job, acc, rej_loop, rej_exists, stats, chain_acc);
+  }
+  dep_wait();
+}
+
+// Insert a key from slot s on, which held `was` when its search ended; as
+// insert_once.
+__device__ __forceinline__ uint32_t insert_small(uint32_t *H, uint32_t mask, uint32_t key, uint32_t s, uint32_t was,
+                                                 uint32_t *tomb, bool first, bool *twice, bool *full) {
+  for (uint32_t n = 0; n <= mask; ++n) {
+    if (was >= kTomb32) {
+      const uint32_t got = atomicCAS(&H[s], was, key);
+      if (got == was) {
+        *tomb = was == kTomb32 ? 1u : 0u;
+        return s;
+      }
+      was = got;
+      continue;
+    }
+    if (was == key) {
+      *twice = true;
+      if (!first) return kNil;
+    }
+    s = (s + 1) & mask;
+    was = H[s];
+  }
+  *full = true;
+  return kNil;
+}
+
+__global__ void __launch_bounds__(32) k_es_run_small(EsJob *jobs, uint32_t job_off, uint32_t nsw, const uint2 *samples,
+                                                     const uint16_t *dists, StatsDev *stats,
+                                                     unsigned long long *chain_acc, uint32_t *err) {
+  extern __shared__ uint32_t small_dyn[];
+  dep_launch();
+  EsJob &job = jobs[job_off + blockIdx.x];
+  const uint32_t x = threadIdx.x, m = job.m, hlog2 = small_log2(m), mask = (1u << hlog2) - 1;
+  if (m < 2 || m > kEsSmallestEdges) {  // the host sends only chains that qualify
+    dep_wait();
+    return;
+  }
+  uint32_t *const H = small_dyn, *const E = H + mask + 1;
+  uint16_t *const slot = reinterpret_cast<uint16_t *>(E + m);  // of the edge at each position
+  uint4 *const list = job.E;
+  const uint2 *const samp = samples + (size_t)job.row * nsw;
+  const uint16_t *const dist = dists + (size_t)job.row * nsw;
+  SampleRing ring;
+  ring.start(nsw, samp, dist);
+  bool full = false;
+  load_small(E, list, m);
+  auto build = [&] {
+    for (uint32_t t = x; t <= mask / 4; t += 32) reinterpret_cast<uint4 *>(H)[t] = make_uint4(~0u, ~0u, ~0u, ~0u);
+    __syncwarp();
+    for (uint32_t t = x; t < m; t += 32) {
+      uint32_t tomb;
+      bool twice = false;
+      const uint32_t s = (E[t] * 0x9E3779B1u) >> (32 - hlog2);
+      slot[t] = (uint16_t)insert_small(H, mask, E[t], s, H[s], &tomb, false, &twice, &full);
+    }
+    __syncwarp();
+  };
+  build();
+  uint32_t acc = 0, rej_loop = 0, rej_exists = 0, tombs = 0;
+  for (uint32_t s = 0; s < nsw;) {
+    uint32_t d;
+    const uint2 cur = ring.window(s, nsw, samp, dist, d);
+    uint32_t n = min(32u, nsw - s);
+    const unsigned hit = __ballot_sync(0xffffffffu, d <= x);
+    if (hit) n = min(n, (uint32_t)__ffs(hit) - 1);
+    const uint32_t i = cur.x, j = cur.y & 0x7FFFFFFFu, g = cur.y >> 31;
+    uint32_t e3 = 0, e4 = 0, s1 = kNil, s2 = kNil, code = kCodeLazy;
+    if (x < n) {
+      const uint32_t e1 = E[i], e2 = E[j];
+      s1 = slot[i] & mask;  // (a full table, which would have been reported: stay in bounds)
+      s2 = slot[j] & mask;
+      code = tau16(g, e1, e2, e3, e4);
+    }
+    const bool live = code == 0;
+    // present targets' slots, and where the others can go
+    uint32_t q3 = kNil, q4 = kNil, a3 = kNil, a4 = kNil, was3 = 0, was4 = 0;
+    if (live) {
+      uint32_t t = (e3 * 0x9E3779B1u) >> (32 - hlog2);
+      for (uint32_t v = 0; v <= mask; ++v, t = (t + 1) & mask) {
+        const uint32_t c = H[t];
+        if (c == e3) {
+          q3 = t;
+          break;
+        }
+        if (c >= kTomb32 && a3 == kNil) {
+          a3 = t;
+          was3 = c;
+        }
+        if (c == kEmpty32) break;
+      }
+      t = (e4 * 0x9E3779B1u) >> (32 - hlog2);
+      for (uint32_t v = 0; v <= mask; ++v, t = (t + 1) & mask) {
+        const uint32_t c = H[t];
+        if (c == e4) {
+          q4 = t;
+          break;
+        }
+        if (c >= kTomb32 && a4 == kNil) {
+          a4 = t;
+          was4 = c;
+        }
+        if (c == kEmpty32) break;
+      }
+    }
+    // the superstep ends before the first switch with a present target that an
+    // earlier one erases
+    uint32_t end = n;
+    for (unsigned who = __ballot_sync(0xffffffffu, q3 != kNil || q4 != kNil); who; who &= who - 1) {
+      const int w = __ffs(who) - 1;
+      const uint32_t t3 = __shfl_sync(0xffffffffu, q3, w), t4 = __shfl_sync(0xffffffffu, q4, w);
+      const bool erases = live && (int)x < w && ((s1 == t3 || s2 == t3) || (s1 == t4 || s2 == t4));
+      if (__any_sync(0xffffffffu, erases)) {
+        end = min(end, (uint32_t)w);
+        break;  // (the first such switch)
+      }
+    }
+    const bool clear = live && q3 == kNil && q4 == kNil && x < end;
+    uint32_t p3 = kNil, p4 = kNil, t3 = 0, t4 = 0;
+    bool twice = false;
+    __syncwarp();
+    if (clear) {
+      p3 = insert_small(H, mask, e3, a3, was3, &t3, x == 0, &twice, &full);
+      p4 = insert_small(H, mask, e4, a4, was4, &t4, x == 0, &twice, &full);
+    }
+    const unsigned two = __ballot_sync(0xffffffffu, twice);
+    if (two) end = min(end, max(1u, (uint32_t)__ffs(two) - 1));
+    uint32_t dead = 0;
+    if (clear && x < end) {
+      H[s1] = kTomb32;
+      H[s2] = kTomb32;
+      E[i] = e3;
+      E[j] = e4;
+      slot[i] = (uint16_t)p3;
+      slot[j] = (uint16_t)p4;
+      dead = 2u - t3 - t4;
+      ++acc;
+    } else if (clear) {  // past the end: its insertions become tombstones
+      if (p3 != kNil) {
+        H[p3] = kTomb32;
+        dead += 1u - t3;
+      }
+      if (p4 != kNil) {
+        H[p4] = kTomb32;
+        dead += 1u - t4;
+      }
+    }
+    if (x < end && !clear) {
+      if (code == kCodeLoop) ++rej_loop;
+      else ++rej_exists;
+    }
+    s += end;
+    tombs += __reduce_add_sync(0xffffffffu, dead);
+    __syncwarp();
+    if (tombs > (mask >> 3)) {
+      build();
+      tombs = 0;
+    }
+  }
+  store_small(list, E, m);
+  if (__any_sync(0xffffffffu, full) && x == 0) atomicOr(err, kErrTableFull);
+  count_small(job, acc, rej_loop, rej_exists, stats, chain_acc);
+  dep_wait();
+}
+
 // ---------------------------------------------------------------- large chains
 // One chain on a cluster of kClusterCtas CTAs, for chains of at least
 // kEsBigChain edges (windows of 1024 switches, thread x of CTA r holding switch
@@ -1005,7 +1370,9 @@ __global__ void __launch_bounds__(B, MIN_BLOCKS) k_es_run(EsJob *jobs, uint32_t 
                                                           const uint2 *samples, const uint16_t *dists,
                                                           StatsDev *stats, unsigned long long *chain_acc,
                                                           uint32_t *err) {
+  dep_launch();
   es_run_body<B, false>(jobs, job_off, nsw, samples, dists, stats, chain_acc, err, nullptr);
+  dep_wait();
 }
 
 // Windows of 1024 switches on one CTA (chains of at least 2^19 edges that the
@@ -1019,11 +1386,29 @@ __global__ void __launch_bounds__(1024, 1) k_es_run_big(EsJob *jobs, uint32_t jo
 
 }  // namespace
 
-uint32_t es_window(uint32_t m) {
-  return m >= kEsBigChain ? 1024u : m >= kEsMidChain ? 256u : m >= kEsSmallChain ? 128u : 32u;
+uint32_t es_group(uint32_t m, uint64_t n) {
+  if (m >= kEsBigChain) return 0;
+  if (m >= kEsMidChain) return 1;
+  if (m >= kEsSmallChain) return 2;
+  if (m < 2) return 3;
+  for (uint32_t v = 0; v < 3; ++v)
+    if (n <= 65536 && bits_bytes(m, n) <= kEsBitBytes[v]) return 7 - v;
+  return m <= kEsSmallestEdges && n <= 65536 ? 4 : 3;
+}
+
+uint32_t es_smem_bytes(uint32_t m, uint32_t n) {
+  const uint32_t g = es_group(m, n);
+  if (g < 4) return 0;
+  return g == 4 ? (4u << small_log2(m)) + 4 * m + 2 * m + 2 : (uint32_t)bits_bytes(m, n);
 }
 
 cudaError_t prepare_es_kernels() {
+  cudaError_t f = cudaFuncSetAttribute(k_es_run_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)es_smem_bytes(kEsSmallestEdges, 65536));
+  if (f == cudaSuccess)
+    f = cudaFuncSetAttribute(k_es_run_bits, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kEsBitBytes[2]);
+  if (f != cudaSuccess) return f;
   cudaError_t e = cudaFuncSetAttribute(k_es_run_big, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)EsShape<1024>::kBytes);
   if (e != cudaSuccess) return e;
@@ -1043,10 +1428,10 @@ cudaError_t launch_es_set(EsJob *jobs, uint32_t njobs, uint32_t *err, cudaStream
   return cudaGetLastError();
 }
 
-cudaError_t launch_es_sample(EsJob *jobs, const uint32_t (&group)[4], unsigned long long off, uint32_t n,
+cudaError_t launch_es_sample(EsJob *jobs, const uint32_t (&group)[kEsGroups], unsigned long long off, uint32_t n,
                              uint2 *samples, uint16_t *dists, cudaStream_t s, uint32_t *launches) {
   uint32_t beg = 0;
-  for (int w = 0; w < 4; ++w) {
+  for (int w = 0; w < (int)kEsGroups; ++w) {
     for (uint32_t o = beg; o < beg + group[w]; o += 65535u, ++*launches) {
       const uint32_t nj = beg + group[w] - o < 65535u ? beg + group[w] - o : 65535u;
       if (w == 0) k_es_sample<1024, 1024><<<dim3((n + 1023) / 1024, nj), 1024, 0, s>>>(jobs, o, off, n, samples, dists);
@@ -1059,23 +1444,42 @@ cudaError_t launch_es_sample(EsJob *jobs, const uint32_t (&group)[4], unsigned l
   return cudaGetLastError();
 }
 
-cudaError_t launch_es_run(EsJob *jobs, const uint32_t (&group)[4], uint32_t nsw, const uint2 *samples,
+cudaError_t launch_es_run(EsJob *jobs, const uint32_t (&group)[kEsGroups], const uint32_t (&smem_of)[kEsGroups], uint32_t nsw, const uint2 *samples,
                           const uint16_t *dists, StatsDev *stats, unsigned long long *chain_acc, uint32_t *err,
                           uint32_t *nstop, bool alone, cudaStream_t s, cudaStream_t s2, cudaEvent_t fork,
                           cudaEvent_t join, uint32_t *launches) {
-  // group[w] jobs with windows of 1024, 256, 128 and 32 switches, in that
-  // order; the two small-window groups run on s2 (after s, and joined back
-  // into s) when there is one, beside the others
-  uint32_t beg[5] = {0, 0, 0, 0, 0};
-  for (int w = 0; w < 4; ++w) beg[w + 1] = beg[w] + group[w];
+  // group[w] jobs with windows of 1024, 256, 128 and 32 switches, then the
+  // small chains in shared memory, in that order; all but the two largest
+  // groups run on s2 (after s, and joined back into s) when there is one,
+  // beside the others
+  uint32_t beg[kEsGroups + 1] = {};
+  for (uint32_t w = 0; w < kEsGroups; ++w) beg[w + 1] = beg[w] + group[w];
   uint32_t n = 0;
-  const bool side = s2 && fork && join && beg[2] > 0 && beg[4] > beg[2];
+  const bool side = s2 && fork && join && beg[2] > 0 && beg[kEsGroups] > beg[2];
   cudaStream_t ss = side ? s2 : s;
   if (side && (cudaEventRecord(fork, s) != cudaSuccess || cudaStreamWaitEvent(s2, fork, 0) != cudaSuccess))
     return cudaGetLastError();
+  // The groups of the side stream need not wait for one another: each starts
+  // when the CTAs of the one before are all on the GPU (programmatic dependent
+  // launch), and every one of these kernels waits for the one before it just
+  // before it ends, so that the last one's end is the end of all.
+  uint32_t beside = 0;
+  auto go = [&](auto fn, uint32_t ctas, uint32_t threads, size_t smem, uint32_t off) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = ss;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = beside++ ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, fn, jobs, off, nsw, samples, dists, stats, chain_acc, err);
+  };
   auto run = [&](int w, cudaStream_t st) {
     for (uint32_t off = beg[w]; off < beg[w + 1]; off += 65535u, ++n) {
-      const uint32_t nj = beg[w + 1] - off < 65535u ? beg[w + 1] - off : 65535u;
+      const uint32_t nj = beg[w + 1] - off < 65535u ? beg[w + 1] - off : 65535u, smem = smem_of[w];
       if (w == 0) {
         k_es_run_cluster<1024 / kClusterCtas><<<nj * kClusterCtas, 1024 / kClusterCtas, 0, st>>>(
             jobs, off, nsw, samples, dists, stats, chain_acc, err, nstop);
@@ -1087,15 +1491,18 @@ cudaError_t launch_es_run(EsJob *jobs, const uint32_t (&group)[4], uint32_t nsw,
       } else if (w == 1) {
         k_es_run<256, 6><<<nj, 256, EsShape<256>::kBytes, st>>>(jobs, off, nsw, samples, dists, stats, chain_acc, err);
       } else if (w == 2) {
-        k_es_run<128, 12><<<nj, 128, EsShape<128>::kBytes, st>>>(jobs, off, nsw, samples, dists, stats, chain_acc,
-                                                                 err);
+        go(k_es_run<128, 12>, nj, 128, EsShape<128>::kBytes, off);
+      } else if (w == 3) {
+        go(k_es_run<32, 32>, nj, 32, EsShape<32>::kBytes, off);
+      } else if (w == 4) {
+        go(k_es_run_small, nj, 32, smem, off);
       } else {
-        k_es_run<32, 32><<<nj, 32, EsShape<32>::kBytes, st>>>(jobs, off, nsw, samples, dists, stats, chain_acc, err);
+        go(k_es_run_bits, nj, 32, smem, off);
       }
     }
   };
-  run(3, ss);
-  run(2, ss);
+  // the groups that take longest first
+  for (const int w : {3, 2, 4, 7, 6, 5}) run(w, ss);
   run(0, s);
   run(1, s);
   if (side && (cudaEventRecord(join, s2) != cudaSuccess || cudaStreamWaitEvent(s, join, 0) != cudaSuccess))

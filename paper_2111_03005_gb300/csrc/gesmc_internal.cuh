@@ -332,30 +332,34 @@ struct EsJob {
   uint32_t tombs;    // tombstones in the set
   uint32_t stopped;  // the kernel stopped this job: 1 for a rebuild of its set on the whole GPU, 2 for the other kernel
   uint32_t alone;    // run on one CTA (largest window)
+  uint32_t n;        // node ids are below n (small chains)
 };
 
 // Shared-memory opt-in of the ParES kernels, once per device.
 cudaError_t prepare_es_kernels();
-// Switches per window of the ParES kernel for a chain of m edges (1024,
-// 256, 128 or 32, by chain size).
-uint32_t es_window(uint32_t m);
+// Jobs run in groups by their chains: windows of 1024, 256, 128 and 32
+// switches, by the number of edges m, and four groups of chains with few edges
+// or nodes that run in shared memory (windows of 32; H null).
+constexpr uint32_t kEsGroups = 8;
+uint32_t es_group(uint32_t m, uint64_t n);
+uint32_t es_smem_bytes(uint32_t m, uint32_t n);  // of a job of the last four groups
 // Edge sets of all jobs (or only of the stopped ones) rebuilt from their lists.
 cudaError_t launch_es_set(EsJob *jobs, uint32_t njobs, uint32_t *err, cudaStream_t s, int num_sms,
                           bool only_stopped);
 // A batch: the switches off .. off + n - 1 of the call, for every job with
 // m >= 2, sampled into row job.row (n entries each) of samples and dists.
 // group as for launch_es_run.
-cudaError_t launch_es_sample(EsJob *jobs, const uint32_t (&group)[4], unsigned long long off, uint32_t n,
+cudaError_t launch_es_sample(EsJob *jobs, const uint32_t (&group)[kEsGroups], unsigned long long off, uint32_t n,
                              uint2 *samples, uint16_t *dists, cudaStream_t s, uint32_t *launches);
-// All jobs' switches of the batch, one CTA per job: the first group[0] jobs
-// with windows of 1024, the next group[1] with windows of 256, then group[2]
-// with 128 and group[3] with 32 (these two on s2, forked from and joined back
-// into s through the two events, if given).  *launches receives the number of
-// launches.
+// All jobs' switches of the batch: the first group[0] jobs are of group 0, the
+// next group[1] of group 1, and so on (smem_of: the most shared memory that a
+// job of the group needs; from group 2 on on s2, forked from and
+// joined back into s through the two events, if given).  *launches receives the
+// number of launches.
 // Jobs of the largest window run on a cluster of CTAs; they stop when their
 // set needs a rebuild, or to go on alone on one CTA (counted in *nstop); the
 // caller rebuilds those sets and launches again (alone: some job may).
-cudaError_t launch_es_run(EsJob *jobs, const uint32_t (&group)[4], uint32_t nsw, const uint2 *samples,
+cudaError_t launch_es_run(EsJob *jobs, const uint32_t (&group)[kEsGroups], const uint32_t (&smem_of)[kEsGroups], uint32_t nsw, const uint2 *samples,
                           const uint16_t *dists, StatsDev *stats, unsigned long long *chain_acc, uint32_t *err,
                           uint32_t *nstop, bool alone, cudaStream_t s, cudaStream_t s2, cudaEvent_t fork,
                           cudaEvent_t join, uint32_t *launches);

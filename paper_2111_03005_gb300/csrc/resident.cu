@@ -125,23 +125,6 @@ __device__ __forceinline__ uint32_t bit_of(uint32_t e, uint32_t bits_log2) {
 
 __device__ __forceinline__ bool bit_set(const uint32_t *map, uint32_t b) { return (map[b >> 5] >> (b & 31)) & 1u; }
 
-// Canonical 32-bit id of the edge {a, b}: smaller node in the high half.
-__device__ __forceinline__ uint32_t pack16(uint32_t a, uint32_t b) {
-  return a < b ? (a << 16) | b : (b << 16) | a;
-}
-
-// tau of Def. 1 on packed edges (the same rules as tau_g): targets e3, e4
-// and the outright-reject code (a loop, or sources sharing a node).
-__device__ __forceinline__ uint32_t tau16(uint32_t g, uint32_t e1, uint32_t e2, uint32_t &e3, uint32_t &e4) {
-  const uint32_t u = e1 >> 16, v = e1 & 0xFFFFu, x = e2 >> 16, y = e2 & 0xFFFFu;
-  const uint32_t a3 = u, b3 = g ? y : x, a4 = v, b4 = g ? x : y;
-  e3 = pack16(a3, b3);
-  e4 = pack16(a4, b4);
-  if (a3 == b3 || a4 == b4) return kCodeLoop;
-  if (u == x || u == y || v == x || v == y) return kCodeShared;
-  return 0;
-}
-
 __device__ __forceinline__ uint32_t home_slot(uint32_t e, uint32_t slog2) { return (e * 0x9E3779B1u) >> (32 - slog2); }
 
 // Slot of id e in the table (linear probing from its home slot), which e

@@ -185,11 +185,11 @@ def test_pool_mixes_window_sizes_with_rebuilds():
         assert np.array_equal(outs[t], x), t
 
 
-@pytest.mark.parametrize("m, switches", [(2, 1500), (5, 3000), (40, 5000), (300, 4000), (5000, 40_000),
+@pytest.mark.parametrize("m, switches", [(2, 8000), (5, 9000), (40, 20_000), (300, 30_000), (5000, 40_000),
                                          (9000, 60_000), (70_000, 400_000)])
 def test_calls_longer_than_a_batch_of_samples(m, switches):
     # a call samples its switches in batches of about three per edge (at least
-    # a few hundred): batches end inside windows of every size but the largest
+    # a few thousand): batches end inside windows of every size but the largest
     n = max(8, int(3 * m ** 0.5) + 8)
     edges = inputs.random_simple_graph(n, m, seed=m + 3)
     es_compare(edges, n, seed=m, calls=[switches])
@@ -209,3 +209,35 @@ def test_large_chains_on_a_cluster(kind):
         edges, n = inputs.gnp(1200, 0.8, seed=4), 1200
     assert len(edges) >= 1 << 19
     es_compare(edges, n, seed=13, calls=[1, 5000, 150_000])
+
+
+@pytest.mark.parametrize("m", [2, 3, 64, 65, 511, 1025, 2047, 2048, 2049, 8191, 8192])
+@pytest.mark.parametrize("kind", ["sparse", "dense", "630 nodes", "1100 nodes", "1750 nodes", "wide ids"])
+def test_small_chains_in_shared_memory(m, kind):
+    # a chain of few nodes has its list and its set (a bit matrix, three sizes) in
+    # shared memory, one of at most 2048 edges its list and a hash table; ids of
+    # more than 16 bits, or more edges, take the general kernels
+    if kind.endswith("nodes"):
+        n = int(kind.split()[0])
+    elif kind == "dense":
+        n = next(v for v in range(3, 10_000) if v * (v - 1) // 2 >= m + m // 3 + 1)
+    else:
+        n = 4 * m + 8 if kind == "sparse" else 70_000
+    edges = inputs.random_simple_graph(n, m, seed=m)
+    es_compare(edges, n, seed=m + 2, calls=[1, 40, 3000])
+
+
+def test_pool_of_small_chains_of_every_group():
+    sizes = [(5, 6), (40, 60), (1000, 8000), (1700, 2048), (4000, 2048), (4000, 2049), (3000, 9000), (70_000, 300)]
+    graphs = [(inputs.random_simple_graph(n, m, seed=20 + t), n) for t, (n, m) in enumerate(sizes)]
+    with gesmc.Pool(max_edges=sum(len(e) for e, _ in graphs), max_chains=len(graphs)) as pool:
+        ids = [pool.add(e, n=n, seed=70 + t) for t, (e, n) in enumerate(graphs)]
+        pool.es_run(700)
+        pool.run(2)
+        pool.es_run(2500)
+        outs = [pool.edges(c) for c in ids]
+    for t, (e, n) in enumerate(graphs):
+        x, _ = oracle.es_run(e, seed=70 + t, switches=700)
+        x, _ = oracle.run(x, seed=70 + t, rounds=2)
+        x, _ = oracle.es_run(x, seed=70 + t, switches=2500, start_switch=700)
+        assert np.array_equal(outs[t], x), t
