@@ -1222,10 +1222,13 @@ __device__ __forceinline__ void group_decide(const RoundArgs &a, const GroupSmem
 }
 
 // Persistent CTAs over the partitions.  Fast path: a thread keeps the hash
-// and the value of its (at most kR) tuples in registers, reads the ids of
-// those that go into the table again, and clears the slots it claimed.
-// Partitions with more tuples than that, or more distinct marked ids than
-// slots, take the sub-pass path, all tuples into the table: the ids whose hash
+// and the value of its R tuples (a quarter more in a partition of more than
+// R T, if the table has room for so many ids) in registers, reads the ids of those that go into the table again, and
+// clears the slots it claimed.  R T is the mean a partition may reach by its
+// layout with every source in it, as in a graph so large that the filter lets
+// nearly all through; half of those have more (G(2^27), 1.07e9 edges: 362 ms a
+// round with them on the sub-pass path, 138 so).  Partitions with more tuples
+// than that, or more distinct marked ids than slots, take the sub-pass path, all tuples into the table: the ids whose hash
 // bits 16.. select them, split further until each sub-pass fits.
 //
 // What bounds it: the barriers and shared-memory latency of one partition
@@ -1243,6 +1246,77 @@ __device__ __forceinline__ void prefetch_partition(const RoundArgs &a, uint32_t 
   const ChainDesc &cd = a.chains[c];
   const uint32_t n = min(a.tcount[cd.tcount_base + (part - cd.part_base) * cd.tstride], cd.capt);
   if (n) bulk_prefetch_l2(a.ptup + cd.tuple_base + (size_t)(part - cd.part_base) * cd.capt, n * (uint32_t)sizeof(uint4));
+}
+
+// A partition's tuples, R to a thread.  Returns true, with *overflow set and
+// the slots claimed here cleared again, if the table was too small for them.
+template <int T, int R>
+__device__ __forceinline__ bool group_fast(const RoundArgs &a, const GroupSmem &g, uint32_t S, const uint4 *prim,
+                                           uint32_t nprim, uint32_t obeg, uint32_t ntup, uint32_t *overflow) {
+  const int tid = threadIdx.x;
+  uint32_t h[R], v[R], todo = 0;  // todo: this thread's tuples that go into the table
+#pragma unroll
+  for (int j = 0; j < R; ++j) {
+    const uint32_t t = tid + j * T;
+    v[j] = kTupleSource;
+    if (t < ntup) {
+      const uint2 zw = __ldcs(reinterpret_cast<const uint2 *>(t < nprim ? &prim[t] : &a.stup[obeg + (t - nprim)]) + 1);
+      v[j] = zw.x;
+      h[j] = zw.y;
+      if (!(zw.x & kTupleSource)) {
+        const uint32_t bit = h[j] >> (32 - kGroupBitsLog2), m = 1u << (bit & 31);
+        if (atomicOr(&g.seen[bit >> 5], m) & m) atomicOr(&g.marked[bit >> 5], m);
+      }
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < R; ++j)
+    if (tid + j * T < ntup && (v[j] & kTupleSource)) {
+      const uint32_t bit = h[j] >> (32 - kGroupBitsLog2), m = 1u << (bit & 31);
+      if (g.seen[bit >> 5] & m) {
+        atomicOr(&g.marked[bit >> 5], m);
+        todo |= 1u << j;
+      }
+    }
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < R; ++j)
+    if (!(v[j] & kTupleSource)) {
+      const uint32_t bit = h[j] >> (32 - kGroupBitsLog2);
+      if ((g.marked[bit >> 5] >> (bit & 31)) & 1u) todo |= 1u << j;
+    }
+  // h of a tuple that goes into the table becomes its slot
+#pragma unroll
+  for (int j = 0; j < R; ++j)
+    if ((todo >> j) & 1u) {
+      const uint32_t t = tid + j * T;
+      const uint2 id = *reinterpret_cast<const uint2 *>(t < nprim ? &prim[t] : &a.stup[obeg + (t - nprim)]);
+      h[j] = group_insert(g, S, ((unsigned long long)id.y << 32) | id.x, h[j], v[j]);
+      if (h[j] == S) {
+        *overflow = 1;
+        todo &= ~(1u << j);
+      }
+    }
+  __syncthreads();
+  const bool full = *overflow != 0;
+  for (uint32_t w = tid; w < 2 * kGroupWords / 4; w += T)  // both bitmaps
+    reinterpret_cast<uint4 *>(g.seen)[w] = make_uint4(0, 0, 0, 0);
+  if (!full) {
+#pragma unroll
+    for (int j = 0; j < R; ++j)
+      if (((todo >> j) & 1u) && (h[j] & kClaimed)) group_alloc(a, g, h[j] & ~kClaimed);
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < R; ++j)
+      if (((todo >> j) & 1u) && !(v[j] & kTupleSource)) group_decide(a, g, h[j] & ~kClaimed, v[j]);
+  }
+  __syncthreads();
+  // (the next partition's first table access comes two barriers later)
+#pragma unroll
+  for (int j = 0; j < R; ++j)
+    if (((todo >> j) & 1u) && (h[j] & kClaimed)) group_reset_slot(g, h[j] & ~kClaimed);
+  return full;
 }
 
 template <int T, int R>
@@ -1270,69 +1344,11 @@ __device__ __forceinline__ void group_body(const RoundArgs &a) {
     const uint32_t nprim = min(a.tcount[cd.tcount_base + (part - pbase) * cd.tstride], capt);
     const uint32_t obeg = ovf ? overflow_offset(a, part) : 0, oend = ovf ? overflow_offset(a, part + 1) : 0;
     const uint32_t ntup = nprim + (oend - obeg);
-    if (ntup <= (uint32_t)(R * T)) {
-      uint32_t h[R], v[R], todo = 0;  // todo: this thread's tuples that go into the table
-#pragma unroll
-      for (int j = 0; j < R; ++j) {
-        const uint32_t t = tid + j * T;
-        v[j] = kTupleSource;
-        if (t < ntup) {
-          const uint2 zw = __ldcs(reinterpret_cast<const uint2 *>(t < nprim ? &prim[t] : &a.stup[obeg + (t - nprim)]) + 1);
-          v[j] = zw.x;
-          h[j] = zw.y;
-          if (!(zw.x & kTupleSource)) {
-            const uint32_t bit = h[j] >> (32 - kGroupBitsLog2), m = 1u << (bit & 31);
-            if (atomicOr(&g.seen[bit >> 5], m) & m) atomicOr(&g.marked[bit >> 5], m);
-          }
-        }
-      }
-      __syncthreads();
-#pragma unroll
-      for (int j = 0; j < R; ++j)
-        if (tid + j * T < ntup && (v[j] & kTupleSource)) {
-          const uint32_t bit = h[j] >> (32 - kGroupBitsLog2), m = 1u << (bit & 31);
-          if (g.seen[bit >> 5] & m) {
-            atomicOr(&g.marked[bit >> 5], m);
-            todo |= 1u << j;
-          }
-        }
-      __syncthreads();
-#pragma unroll
-      for (int j = 0; j < R; ++j)
-        if (!(v[j] & kTupleSource)) {
-          const uint32_t bit = h[j] >> (32 - kGroupBitsLog2);
-          if ((g.marked[bit >> 5] >> (bit & 31)) & 1u) todo |= 1u << j;
-        }
-      // h of a tuple that goes into the table becomes its slot
-#pragma unroll
-      for (int j = 0; j < R; ++j)
-        if ((todo >> j) & 1u) {
-          const uint32_t t = tid + j * T;
-          const uint2 id = *reinterpret_cast<const uint2 *>(t < nprim ? &prim[t] : &a.stup[obeg + (t - nprim)]);
-          h[j] = group_insert(g, S, ((unsigned long long)id.y << 32) | id.x, h[j], v[j]);
-          if (h[j] == S) {
-            overflow = 1;
-            todo &= ~(1u << j);
-          }
-        }
-      __syncthreads();
-      const bool full = overflow != 0;
-      for (uint32_t w = tid; w < 2 * kGroupWords / 4; w += T)  // both bitmaps
-        reinterpret_cast<uint4 *>(g.seen)[w] = make_uint4(0, 0, 0, 0);
-      if (!full) {
-#pragma unroll
-        for (int j = 0; j < R; ++j)
-          if (((todo >> j) & 1u) && (h[j] & kClaimed)) group_alloc(a, g, h[j] & ~kClaimed);
-        __syncthreads();
-#pragma unroll
-        for (int j = 0; j < R; ++j)
-          if (((todo >> j) & 1u) && !(v[j] & kTupleSource)) group_decide(a, g, h[j] & ~kClaimed, v[j]);
-      }
-      __syncthreads();
-      // (the next partition's first table access comes two barriers later)
-#pragma unroll
-      for (int j = 0; j < R; ++j)
-        if (((todo >> j) & 1u) && (h[j] & kClaimed)) group_reset_slot(g, h[j] & ~kClaimed);
+    constexpr int kWide = R + R / 4;
+    if (ntup <= (uint32_t)((S >= R * T ? kWide : R) * T)) {
+      const bool full = ntup <= (uint32_t)(R * T)
+                            ? group_fast<T, R>(a, g, S, prim, nprim, obeg, ntup, &overflow)
+                            : group_fast<T, kWide>(a, g, S, prim, nprim, obeg, ntup, &overflow);
       if (!full) continue;
       if (tid == 0) overflow = 0;
       __syncthreads();

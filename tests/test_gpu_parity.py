@@ -397,3 +397,13 @@ def test_grouping_with_few_and_many_marked_ids(n, m, tuple_log2, group_log2):
     # ids outnumber the slots of a small table; sparse ones: few are marked
     edges = inputs.random_simple_graph(n, m, seed=m + n)
     run_and_compare(edges, n, seed=31, rounds=2, tuple_log2=tuple_log2, group_log2=group_log2)
+
+
+@pytest.mark.parametrize("group_log2", [10, 11, 12])
+@pytest.mark.parametrize("n,m", [(67, 2100), (70, 2200), (75, 2620), (79, 3000)])
+def test_grouping_of_partitions_around_the_register_path(n, m, group_log2):
+    # nearly complete graphs in two partitions: every source passes the filter,
+    # so a partition gets about m tuples, around 2048 (four to a thread) and
+    # 2560 (five; above, the sub-pass path)
+    edges = inputs.random_simple_graph(n, m, seed=m)
+    run_and_compare(edges, n, seed=37, rounds=6, tuple_log2=12, group_log2=group_log2)
