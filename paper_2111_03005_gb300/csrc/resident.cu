@@ -345,7 +345,7 @@ __device__ __forceinline__ uint32_t sort_round(const ChainDesc &ch, unsigned lon
 }
 
 // The rounds of one chain on one CTA.  What bounds it: issued instructions
-// (about 48 thousand warp instructions a round of 5,000 edges, two a cycle)
+// (about 44 thousand warp instructions a round of 5,000 edges, two a cycle)
 // and, between them, the chains of dependent shared-memory operations of each
 // step; nothing goes to memory.  A table of all targets and a failing search
 // of it for every edge of E took 18 us a round of G(1000, 0.01) with its
@@ -424,6 +424,7 @@ __global__ void __launch_bounds__(T, 1024 / T) k_round_resident(RoundArgs a, Res
     dep_wait();
     dep_launch();
   }
+  bool dense = false;  // (the same in all threads) the bitmaps are left out
   constexpr uint32_t KS = ResPer<T>::kSwitches, KP = ResPer<T>::kPermVec;
   // a permutation sorted beforehand is loaded a round ahead, into registers
   const uint32_t nvec = (m + 7) / 8;
@@ -456,7 +457,8 @@ __global__ void __launch_bounds__(T, 1024 / T) k_round_resident(RoundArgs a, Res
 
     // 2. switches: outright rejects, the others' targets into the bitmap
     // (the sort's keys are dead)
-    for (uint32_t w = tid; w < words / 2; w += T) reinterpret_cast<uint4 *>(seen)[w] = make_uint4(0, 0, 0, 0);
+    if (!dense)
+      for (uint32_t w = tid; w < words / 2; w += T) reinterpret_cast<uint4 *>(seen)[w] = make_uint4(0, 0, 0, 0);
     if (tid == 0) s_cand = s_hit = 0;
     __syncthreads();
     uint32_t lazies = 0;  // the thread's switches that laziness skips
@@ -489,84 +491,90 @@ __global__ void __launch_bounds__(T, 1024 / T) k_round_resident(RoundArgs a, Res
         continue;
       }
       live |= 1u << u;
+      if (dense) {
+        status[k] = (uint16_t)kUndecided;
+        continue;
+      }
       const uint32_t b3 = bit_of(e3, bits_log2), b4 = bit_of(e4, bits_log2);
       if ((atomicOr(&seen[b3 >> 5], 1u << (b3 & 31)) >> (b3 & 31)) & 1u) atomicOr(&marked[b3 >> 5], 1u << (b3 & 31));
       if ((atomicOr(&seen[b4 >> 5], 1u << (b4 & 31)) >> (b4 & 31)) & 1u) atomicOr(&marked[b4 >> 5], 1u << (b4 & 31));
     }
     __syncthreads();
-    // edges of E on a target's bit (few; one counter atomic for a thread's)
-    uint32_t mine = 0;
-#pragma unroll
-    for (uint32_t u = 0; u < KS; ++u) {
-      if (tid + u * T >= L) continue;
-      const uint32_t b1 = bit_of(e1[u], bits_log2), b2 = bit_of(e2[u], bits_log2);
-      mine |= bit_set(seen, b1) ? 1u << (2 * u) : 0u;
-      mine |= bit_set(seen, b2) ? 2u << (2 * u) : 0u;
-    }
-    if (mine) {
-      uint32_t at = atomicAdd(&s_hit, (uint32_t)__popc(mine));
+    uint32_t ncand = L, nhit = 0;
+    if (!dense) {
+      // edges of E on a target's bit (few; one counter atomic for a thread's)
+      uint32_t mine = 0;
 #pragma unroll
       for (uint32_t u = 0; u < KS; ++u) {
-        const uint32_t k = tid + u * T, b1 = bit_of(e1[u], bits_log2), b2 = bit_of(e2[u], bits_log2);
-        if ((mine >> (2 * u)) & 1u) {
-          atomicOr(&marked[b1 >> 5], 1u << (b1 & 31));
-          hits[at++] = (uint16_t)(2 * k);
-        }
-        if ((mine >> (2 * u)) & 2u) {
-          atomicOr(&marked[b2 >> 5], 1u << (b2 & 31));
-          hits[at++] = (uint16_t)(2 * k + 1);
+        if (tid + u * T >= L) continue;
+        const uint32_t b1 = bit_of(e1[u], bits_log2), b2 = bit_of(e2[u], bits_log2);
+        mine |= bit_set(seen, b1) ? 1u << (2 * u) : 0u;
+        mine |= bit_set(seen, b2) ? 2u << (2 * u) : 0u;
+      }
+      if (mine) {
+        uint32_t at = atomicAdd(&s_hit, (uint32_t)__popc(mine));
+#pragma unroll
+        for (uint32_t u = 0; u < KS; ++u) {
+          const uint32_t k = tid + u * T, b1 = bit_of(e1[u], bits_log2), b2 = bit_of(e2[u], bits_log2);
+          if ((mine >> (2 * u)) & 1u) {
+            atomicOr(&marked[b1 >> 5], 1u << (b1 & 31));
+            hits[at++] = (uint16_t)(2 * k);
+          }
+          if ((mine >> (2 * u)) & 2u) {
+            atomicOr(&marked[b2 >> 5], 1u << (b2 & 31));
+            hits[at++] = (uint16_t)(2 * k + 1);
+          }
         }
       }
-    }
-    if ((m & 1u) && tid == T - 1) {  // the unpaired slot
-      const uint32_t b = bit_of(E[perm[m - 1]], bits_log2);
-      if (bit_set(seen, b)) {
-        atomicOr(&marked[b >> 5], 1u << (b & 31));
-        hits[atomicAdd(&s_hit, 1u)] = (uint16_t)(m - 1);
+      if ((m & 1u) && tid == T - 1) {  // the unpaired slot
+        const uint32_t b = bit_of(E[perm[m - 1]], bits_log2);
+        if (bit_set(seen, b)) {
+          atomicOr(&marked[b >> 5], 1u << (b & 31));
+          hits[atomicAdd(&s_hit, 1u)] = (uint16_t)(m - 1);
+        }
       }
-    }
-    __syncthreads();
-    // free targets: legal in the first wave; the others are candidates, with
-    // which of their targets are marked in tslot
-    mine = 0;
+      __syncthreads();
+      // free targets: legal in the first wave; the others are candidates, with
+      // which of their targets are marked in tslot
+      mine = 0;
 #pragma unroll
-    for (uint32_t u = 0; u < KS; ++u) {
-      if (!((live >> u) & 1u)) continue;
-      const uint32_t k = tid + u * T;
-      uint32_t e3, e4;
-      tau16((ij[u] & 0xFFFFu) < (ij[u] >> 16) ? 1u : 0u, e1[u], e2[u], e3, e4);
-      const uint32_t f = (bit_set(marked, bit_of(e3, bits_log2)) ? 1u : 0u) |
-                         (bit_set(marked, bit_of(e4, bits_log2)) ? 2u : 0u);
-      status[k] = (uint16_t)(f ? kUndecided : (1u << 2) | kLegal);
-      tslot[k] = f;
-      mine |= f ? 1u << u : 0u;
-    }
-    if (mine) {
-      uint32_t at = atomicAdd(&s_cand, (uint32_t)__popc(mine));
+      for (uint32_t u = 0; u < KS; ++u) {
+        if (!((live >> u) & 1u)) continue;
+        const uint32_t k = tid + u * T;
+        uint32_t e3, e4;
+        tau16((ij[u] & 0xFFFFu) < (ij[u] >> 16) ? 1u : 0u, e1[u], e2[u], e3, e4);
+        const uint32_t f = (bit_set(marked, bit_of(e3, bits_log2)) ? 1u : 0u) |
+                           (bit_set(marked, bit_of(e4, bits_log2)) ? 2u : 0u);
+        status[k] = (uint16_t)(f ? kUndecided : (1u << 2) | kLegal);
+        tslot[k] = f;
+        mine |= f ? 1u << u : 0u;
+      }
+      if (mine) {
+        uint32_t at = atomicAdd(&s_cand, (uint32_t)__popc(mine));
 #pragma unroll
-      for (uint32_t u = 0; u < KS; ++u)
-        if ((mine >> u) & 1u) cand[at++] = (uint16_t)(tid + u * T);
+        for (uint32_t u = 0; u < KS; ++u)
+          if ((mine >> u) & 1u) cand[at++] = (uint16_t)(tid + u * T);
+      }
+      __syncthreads();
+      ncand = s_cand;
+      nhit = s_hit;
     }
-    __syncthreads();
-    const uint32_t ncand = s_cand, nhit = s_hit;
 
     // 3. the candidates' marked targets into the table, over the bitmaps; a
-    // table that does not fit there takes the lists' bytes too, and the
-    // candidates are then found by their status (and every edge of E looked
-    // up)
+    // table that does not fit there takes the lists' bytes too, and every
+    // thread then goes through its own switches (and every edge of E is looked
+    // up).  Where most switches are candidates (a dense graph: most targets are
+    // edges), the call's next rounds enter all of them at once: the bitmaps are
+    // a sixth of such a round (20 rounds of K_140 less a hundredth, 9,641 edges:
+    // 929 us with them, 779 without; a quarter of free switches pays for them).
     uint32_t wave = 1;
     if (ncand) {
       uint32_t slog2 = 5;  // room for twice the marked targets (at most two a candidate)
       while (slog2 < lay.slog2 && (1u << slog2) < 4 * ncand) ++slog2;
-      const bool listed = slog2 <= lay.list_slog2;
+      const bool listed = !dense && slog2 <= lay.list_slog2;
       if (!listed) slog2 = lay.slog2;
       const uint32_t S = 1u << slog2, ntake = listed ? ncand : L;
       uint32_t *const tpq = tkey + S;
-      if (!listed) {
-        for (uint32_t k = tid; k < L; k += T)
-          if (status[k] != kUndecided) tslot[k] = 0;
-        __syncthreads();  // the lists have been read
-      }
       for (uint32_t s = tid; s < S / 2; s += T) reinterpret_cast<uint4 *>(tkey)[s] = make_uint4(~0u, ~0u, ~0u, ~0u);
       for (uint32_t w = tid; w < S / 32; w += T) multi[w] = 0;
       if (tid < 3) s_wave[tid] = 0;
@@ -574,38 +582,66 @@ __global__ void __launch_bounds__(T, 1024 / T) k_round_resident(RoundArgs a, Res
       // every candidate enters its marked targets, registers there as an
       // inserter (smallest q per id) and keeps their slots
       bool full = false;
-      for (uint32_t c = tid; c < ntake; c += T) {
-        const uint32_t k = listed ? cand[c] : c, f = tslot[k];
-        uint32_t s3 = kFree, s4 = kFree;
-        if (f) {
-          const uint32_t pij = reinterpret_cast<const uint32_t *>(perm)[k], i = pij & 0xFFFFu, j = pij >> 16;
-          uint32_t e3, e4;
-          tau16(i < j ? 1u : 0u, E[i], E[j], e3, e4);
-          if (f & 1u) s3 = tab_insert(tkey, slog2, e3);
-          if (f & 2u) s4 = tab_insert(tkey, slog2, e4);
-          if (s3 == S || s4 == S) {
-            full = true;
-            s3 = s4 = kFree;
-          }
-          // a slot whose q was already set has a second inserter
-          if (s3 != kFree && (tab_qmin(tpq, s3, k) & 0xFFFFu) != kQ16None) atomicOr(&multi[s3 >> 5], 1u << (s3 & 31));
-          if (s4 != kFree && (tab_qmin(tpq, s4, k) & 0xFFFFu) != kQ16None) atomicOr(&multi[s4 >> 5], 1u << (s4 & 31));
+      auto enter = [&](uint32_t k, uint32_t f, uint32_t i, uint32_t j, uint32_t x1, uint32_t x2) {
+        uint32_t e3, e4, s3 = kFree, s4 = kFree;
+        tau16(i < j ? 1u : 0u, x1, x2, e3, e4);
+        if (f & 1u) s3 = tab_insert(tkey, slog2, e3);
+        if (f & 2u) s4 = tab_insert(tkey, slog2, e4);
+        if (s3 == S || s4 == S) {
+          full = true;
+          s3 = s4 = kFree;
         }
+        // a slot whose q was already set has a second inserter
+        if (s3 != kFree && (tab_qmin(tpq, s3, k) & 0xFFFFu) != kQ16None) atomicOr(&multi[s3 >> 5], 1u << (s3 & 31));
+        if (s4 != kFree && (tab_qmin(tpq, s4, k) & 0xFFFFu) != kQ16None) atomicOr(&multi[s4 >> 5], 1u << (s4 & 31));
         tslot[k] = s3 | (s4 << 16);
+      };
+      if (listed) {
+        for (uint32_t c = tid; c < ncand; c += T) {
+          const uint32_t k = cand[c], pij = reinterpret_cast<const uint32_t *>(perm)[k], i = pij & 0xFFFFu, j = pij >> 16;
+          enter(k, tslot[k], i, j, E[i], E[j]);
+        }
+      } else if constexpr (!kPre) {  // (the sort leaves no registers to unroll this)
+#pragma unroll 1
+        for (uint32_t k = tid; k < L; k += T) {
+          const uint32_t f = status[k] != kUndecided ? 0u : dense ? 3u : tslot[k];
+          const uint32_t pij = reinterpret_cast<const uint32_t *>(perm)[k], i = pij & 0xFFFFu, j = pij >> 16;
+          if (f) enter(k, f, i, j, E[i], E[j]);
+          else tslot[k] = kFree | (kFree << 16);
+        }
+      } else {
+#pragma unroll
+        for (uint32_t u = 0; u < KS; ++u) {
+          const uint32_t k = tid + u * T;
+          if (k >= L) continue;
+          const uint32_t f = !((live >> u) & 1u) ? 0u : dense ? 3u : tslot[k];
+          if (f) enter(k, f, ij[u] & 0xFFFFu, ij[u] >> 16, e1[u], e2[u]);
+          else tslot[k] = kFree | (kFree << 16);
+        }
       }
       if (__syncthreads_or(full)) {
         err = kErrTableFull;
         break;
       }
       // erasers of the edges that are targets
-      const uint32_t nsrc = listed ? nhit : m;
-      for (uint32_t x = tid; x < nsrc; x += T) {
-        const uint32_t s = listed ? hits[x] : x;
-        const uint32_t slot = tab_find(tkey, slog2, E[perm[s]]);
-        if (slot < S) {
-          const uint32_t p = (s >> 1) < L ? (s >> 1) : kP16Keep;
-          atomicAnd(&tpq[slot], (p << 16) | 0xFFFFu);
+      auto erase = [&](uint32_t e, uint32_t p) {
+        const uint32_t slot = tab_find(tkey, slog2, e);
+        if (slot < S) atomicAnd(&tpq[slot], (p << 16) | 0xFFFFu);
+      };
+      if (listed || !kPre) {
+        for (uint32_t x = tid; x < (listed ? nhit : m); x += T) {
+          const uint32_t s = listed ? hits[x] : x;
+          erase(E[perm[s]], (s >> 1) < L ? (s >> 1) : kP16Keep);
         }
+      } else {
+#pragma unroll
+        for (uint32_t u = 0; u < KS; ++u) {
+          const uint32_t k = tid + u * T;
+          if (k >= L) continue;
+          erase(e1[u], k);
+          erase(e2[u], k);
+        }
+        if ((m & 1u) && tid == T - 1) erase(E[perm[m - 1]], kP16Keep);
       }
       __syncthreads();
 
@@ -696,6 +732,7 @@ __global__ void __launch_bounds__(T, 1024 / T) k_round_resident(RoundArgs a, Res
         requeue = I;
       }
       if (err) break;
+      dense = 4 * ncand > 3 * L;
     }
     if (tid == 0) atomicMax(&job.round_waves[t], wave);
 

@@ -266,6 +266,26 @@ def test_edges_of_the_size_classes(m, dense):
         assert st[k] == want_st[k], k
 
 
+def test_dense_chains_sorted_in_their_own_ctas():
+    # after a round with most switches as candidates the call's next rounds
+    # leave the bitmaps out; chains of every class and of a handful of edges,
+    # half of them lazy
+    sizes = [3, 8, 16, 17, 33, 700, 1501, 3000, 4097, 9000]
+    graphs = []
+    for t in range(50):
+        m = sizes[t % len(sizes)]
+        n = next(v for v in range(3, 70000) if v * (v - 1) // 2 >= m + m // 8 + 1)
+        graphs.append((inputs.random_simple_graph(n, m, seed=t), n, (1 << 62) * (t // 10 % 2)))
+    with gesmc.Pool(max_edges=sum(len(g[0]) for g in graphs), max_chains=50) as pool:
+        ids = [pool.add(e, n=n, seed=t, lazy_threshold=thr) for t, (e, n, thr) in enumerate(graphs)]
+        pool.set_round_launch(RESIDENT)
+        pool.run(5)
+        outs = [pool.edges(c) for c in ids]
+    for t, (e, n, thr) in enumerate(graphs):
+        want, _ = oracle.run(e, seed=t, rounds=5, lazy_threshold=thr)
+        assert np.array_equal(outs[t], want), t
+
+
 def test_keys_that_agree_in_the_bits_the_sort_compares():
     # seed 7, round 994747: the keys of two positions below 10240 agree in
     # their top 46 bits, the bucket's 14 and the 32 compared in it, so that
