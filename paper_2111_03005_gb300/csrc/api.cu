@@ -140,8 +140,8 @@ Layout pool_layout(const Capacity &c, uint64_t M, uint64_t C) {
   l.chains = take(sizeof(ChainDesc) * C);
   l.chain_acc = take(8 * C);
   l.chain_ell = take(4 * C);
-  l.es_jobs = take(sizeof(EsJob) * C);
   l.es_job_of = take(4 * C);
+  l.es_jobs = take(sizeof(EsJob) * C);  // (behind es_job_of: one copy brings both)
   l.owner_slot = take(4 * c.slots);
   l.owner_switch = take(4 * c.switches);
   l.owner_bucket = take(4 * c.buckets);
@@ -1045,11 +1045,15 @@ int pool_es_run(gesmc_pool_t p, uint64_t switches, uint32_t only) {
   uint32_t *djob_of = at<uint32_t>(p->base, p->lay.es_job_of);
   uint32_t *err = &a.ctl->err;
   const uint32_t nj = (uint32_t)jobs.size();
-  bool ok = cudaMemcpyAsync(djob_of, job_of.data(), 4ull * p->max_chains, cudaMemcpyHostToDevice, s) == cudaSuccess;
-  ok &= cudaMemcpyAsync(djobs, jobs.data(), sizeof(EsJob) * nj, cudaMemcpyHostToDevice, s) == cudaSuccess;
+  std::vector<unsigned char> both(p->lay.es_jobs - p->lay.es_job_of + sizeof(EsJob) * nj);
+  std::memcpy(both.data(), job_of.data(), 4ull * p->max_chains);
+  std::memcpy(both.data() + (p->lay.es_jobs - p->lay.es_job_of), jobs.data(), sizeof(EsJob) * nj);
+  bool ok = cudaMemcpyAsync(djob_of, both.data(), both.size(), cudaMemcpyHostToDevice, s) == cudaSuccess;
   ok &= launch_es_store(a, djobs, djob_of, s, p->num_sms) == cudaSuccess;
-  const uint64_t set_launches = 2ull * ((nj + 65534) / 65535);
-  ok &= launch_es_set(djobs, nj, err, s, p->num_sms, false) == cudaSuccess;
+  // (no sets to build if every chain has its own in shared memory)
+  const uint32_t nset = group[0] + group[1] + group[2] + group[3];
+  const uint64_t set_launches = 2ull * ((nset + 65534) / 65535);
+  ok &= launch_es_set(djobs, nset, err, s, p->num_sms, false) == cudaSuccess;
   p->launches += set_launches + 2;
   // The switches run in batches, sampled beforehand into the overflow-tuple
   // array (free between rounds): 8 bytes and a 16-bit distance per switch and
@@ -1084,7 +1088,7 @@ int pool_es_run(gesmc_pool_t p, uint64_t switches, uint32_t only) {
       ok &= cudaStreamSynchronize(s) == cudaSuccess;
       if (e != 0) off = switches;  // an error ends the call
       if (!ok || stopped == 0 || e != 0) break;
-      ok &= launch_es_set(djobs, nj, err, s, p->num_sms, true) == cudaSuccess;
+      ok &= launch_es_set(djobs, nset, err, s, p->num_sms, true) == cudaSuccess;
       p->launches += set_launches;
     }
   }
