@@ -201,7 +201,8 @@ def algorithmic_bytes(stage: str, m: int, L: int, nb: int, npart: int, accepted:
       permute:   read the list in slot order (2 x 12 B) and the status word (4 B),
                  write two 16-byte bucket records (their write frontiers stay in L2)
       sortpair:  read the two records (32 B); write the list in slot order (24 B),
-                 the reject word (4 B), the dependency-entry pair (8 B) and append
+                 the reject word (4 B), the dependency-entry pair (8 B; only targets
+                 with an entry still have it written, by the grouping) and append
                  the two target tuples to their hash partitions (32 B)
       sources:   read the two list edges (16 B) and the reject word (4 B); the
                  source tuples a target needs are rare in a sparse graph, and the

@@ -158,7 +158,10 @@ int gesmc_run(gesmc_t h, uint64_t global_switches, uint64_t seed);
  * 0), key = (seed, 0)) = (w0, w1, w2, w3): i = floor(w0 m / 2^64),
  * j = j' + [j' >= i] with j' = floor(w1 (m - 1) / 2^64), g = the top bit of
  * w2; switches are numbered on from the handle's last ES-MC switch.  Runs
- * in supersteps without source dependencies, one CTA per chain.  May be
+ * in supersteps without source dependencies, one CTA per chain (a cluster of
+ * eight for chains of 2^19 edges or more, a warp with the edge set in shared
+ * memory for small chains), the switches sampled beforehand in batches on the
+ * whole GPU.  May be
  * mixed with gesmc_run on the same handle.  A seed different from the
  * handle's current one re-seeds it as gesmc_run does.  With m < 2 every
  * switch is counted as skipped (stats.lazy).  Synchronises the stream. */
@@ -191,7 +194,8 @@ int gesmc_stage_times(gesmc_t h, double *ms, int n_stages, uint64_t *rounds);
 const char *gesmc_stage_name(int stage);
 
 /* How a round is launched.  ctas == 0 (the default): the round's kernels one
- * after another (about 14 of them, replayed from a captured CUDA graph), each
+ * after another (about 14 of them; a handle's first rounds are launched one by
+ * one, later ones are replayed from a captured CUDA graph of a few rounds), each
  * shaped for large graphs.  ctas >= 1: the whole round in one cooperative
  * launch of that many 512-thread CTAs (at most as many as the device holds
  * at once; *effective, if not NULL, receives the count used), the stages
@@ -204,9 +208,10 @@ const char *gesmc_stage_name(int stage);
  * (gesmc_set_profiling) always uses the separate kernels.
  *
  * ctas == GESMC_ROUND_RESIDENT: resident rounds, for small chains.  Each
- * chain runs on one 1024-thread CTA that keeps its list (one 32-bit word per
- * edge), the permutation, the switch statuses and a hash table of the round's
- * target edge ids in shared memory, and runs ALL rounds of a gesmc_run call
+ * chain runs on one CTA (128 to 1024 threads by its size) that keeps its list
+ * (one 32-bit word per edge), the permutation, the switch statuses, a bitmap of
+ * the round's targets and a hash table of the few that may have a dependency in
+ * shared memory, and runs ALL rounds of a gesmc_run call
  * in that one launch (plus a one-CTA launch that folds the rounds' wave
  * counts into the statistics); a round's steps (Philox keys, the counting
  * sort of the positions, the switches, their erasers and inserters,
@@ -214,8 +219,8 @@ const char *gesmc_stage_name(int stage);
  * barriers only.  When a pool holds few chains, the permutations of the
  * call's rounds are sorted beforehand by one more launch (one CTA per chain
  * and round, on the other SMs), and the chains' CTAs load them.  Calls with
- * more rounds than the pool's scratch space holds take several launches.  Chains qualify with m <= GESMC_RESIDENT_MAX_EDGES and
- * n <= GESMC_RESIDENT_MAX_NODES (n: the node bound given at creation, else
+ * more rounds than the pool's scratch space holds take several launches.
+ * Chains qualify with m <= GESMC_RESIDENT_MAX_EDGES and n <= GESMC_RESIDENT_MAX_NODES (n: the node bound given at creation, else
  * the largest id + 1); GESMC_E_TOO_LARGE if a chain does not (and, in a pool,
  * for a later gesmc_pool_add of such a chain).  The same lists, counters and
  * wave telemetry as the other launches.  This is the dedicated base case the

@@ -10,8 +10,8 @@ Two choices shape a round without changing its result:
   the grouping kernel's occupancy (20 bytes of shared memory per slot).
 
 A third choice, for small problems only, is how a round is launched:
-``round_ctas`` = 0 runs the round's kernels one after another (replayed from
-a captured CUDA graph); ``round_ctas`` >= 1 runs the whole round in one
+``round_ctas`` = 0 runs the round's kernels one after another (after the first
+rounds replayed from a captured CUDA graph); ``round_ctas`` >= 1 runs the whole round in one
 cooperative launch of that many CTAs (the block-count axis), which saves the
 launch latency between stages that dominates the rounds of small graphs;
 ``round_ctas`` = ROUND_RESIDENT (when every chain is small enough) runs all

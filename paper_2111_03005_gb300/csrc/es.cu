@@ -18,9 +18,10 @@
 // one CTA (for the largest chains a cluster of eight) runs all supersteps of
 // one chain, a switch per thread.  The list E
 // (position order) and the edge set H (open addressing over canonical ids,
-// tombstones on erase) live in HBM; a list entry also holds its edge's slot in
-// H, so that erasing it takes no search, and the search for a target ends at
-// the slot where it would be inserted.  Most supersteps have no dependency at
+// tombstones on erase) live in HBM (small chains have both in shared memory,
+// with a bit per pair of nodes for H where that fits); a list entry also holds
+// its edge's slot in H, so that erasing it takes no search, and the search for
+// a target ends at the slot where it would be inserted.  Most supersteps have no dependency at
 // all: the targets go into a shared-memory table of fingerprints, and if no
 // fingerprint is met twice, by two targets or by a source, a switch is legal
 // iff none of its targets is in H.  Else the superstep's erasers and
@@ -46,7 +47,8 @@ constexpr uint8_t kEsUndecided = 0, kEsLegal = 1, kEsIllegal = 2;
 // windows of 1024 switches, chains of at least 2^16 windows of 256 on CTAs of
 // 256 threads (six per SM), chains of at least 2^13 windows of 128, smaller
 // ones windows of 32 on one warp each (up to 32 per SM), whose barriers cost
-// next to nothing.
+// next to nothing; of these, a chain whose bit matrix or table fits in shared
+// memory keeps its list and set there.
 constexpr uint32_t kEsBigChain = 1u << 19;
 constexpr uint32_t kEsMidChain = 1u << 16;
 constexpr uint32_t kEsSmallChain = 1u << 13;
