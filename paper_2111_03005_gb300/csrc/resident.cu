@@ -285,6 +285,17 @@ __device__ __forceinline__ uint32_t sort_round(const ChainDesc &ch, unsigned lon
   for (uint32_t b = tid; b < nb / 4; b += T) reinterpret_cast<uint4 *>(cnt)[b] = make_uint4(0, 0, 0, 0);
   if (tid == 0) *s_ell = 0;
   __syncthreads();
+  if (exact) {
+    uint32_t n = 0;
+    const uint32_t nl = (L + 3) / 4;
+    for (uint32_t q = tid; q < nl; q += T) {
+      const U64x4 w0 = philox(q, round, 1, 0, ch.seed, 0);
+#pragma unroll
+      for (uint32_t u = 0; u < 4; ++u) n += (4 * q + u < L && w0.w[u] >= ch.lazy_threshold) ? 1u : 0u;
+    }
+    n = warp_sum(n);
+    if ((tid & 31u) == 0 && n) atomicAdd(s_ell, n);
+  }
   uint32_t key[4 * KB], bk[4 * KB];  // bk: bucket, and the place among its arrivals in the high half
 #pragma unroll
   for (uint32_t u = 0; u < KB; ++u) {
@@ -297,17 +308,6 @@ __device__ __forceinline__ uint32_t sort_round(const ChainDesc &ch, unsigned lon
       key[4 * u + v] = __funnelshift_l((uint32_t)w.w[v], hi, nb_log2);
       bk[4 * u + v] = 4 * q + v < m ? b | (atomicAdd(&cnt[b], 1u) << 16) : 0u;
     }
-  }
-  if (exact) {
-    uint32_t n = 0;
-    const uint32_t nl = (L + 3) / 4;
-    for (uint32_t q = tid; q < nl; q += T) {
-      const U64x4 w0 = philox(q, round, 1, 0, ch.seed, 0);
-#pragma unroll
-      for (uint32_t u = 0; u < 4; ++u) n += (4 * q + u < L && w0.w[u] >= ch.lazy_threshold) ? 1u : 0u;
-    }
-    n = warp_sum(n);
-    if ((tid & 31u) == 0 && n) atomicAdd(s_ell, n);
   }
   __syncthreads();
   const uint32_t ell = exact ? *s_ell : L;
@@ -343,6 +343,20 @@ __device__ __forceinline__ uint32_t sort_round(const ChainDesc &ch, unsigned lon
   }
   return ell;
 }
+
+// The same as a call of its own, for the CTA of 1024 threads: inlined, the twelve
+// keys of a thread and what the round keeps besides left it 324 bytes of
+// spills, which go to L2 (shared memory takes nearly all of L1).  20 rounds of
+// 200 chains of 8,011 edges: 1299 -> 1275 us, of 9,641 (dense) 2320 -> 2114.
+// The smaller CTAs, eight keys a thread, are 3 to 4% slower so.
+template <int T>
+__device__ __noinline__ uint32_t sort_apart(const ChainDesc &ch, unsigned long long round, uint32_t m, uint32_t L,
+                                            uint32_t nb_log2, uint32_t *skey, uint32_t *cnt, uint16_t *spos,
+                                            uint16_t *perm, uint32_t *s_warp, uint32_t *s_ell) {
+  return sort_round<T>(ch, round, m, L, nb_log2, skey, cnt, spos, perm, s_warp, s_ell);
+}
+template <int T>
+constexpr bool kSortApart = T == 1024;
 
 // The rounds of one chain on one CTA.  What bounds it: issued instructions
 // (about 44 thousand warp instructions a round of 5,000 edges, two a cycle)
@@ -452,7 +466,8 @@ __global__ void __launch_bounds__(T, 1024 / T) k_round_resident(RoundArgs a, Res
       }
       ell = exact ? __ldcg(&job.ebuf[(size_t)t * job.njobs + job.job_base + blockIdx.x]) : L;
     } else {
-      ell = sort_round<T>(ch, round, m, L, nb_log2, skey, cnt, scat, perm, s_warp, &s_ell);
+      ell = kSortApart<T> ? sort_apart<T>(ch, round, m, L, nb_log2, skey, cnt, scat, perm, s_warp, &s_ell)
+                          : sort_round<T>(ch, round, m, L, nb_log2, skey, cnt, scat, perm, s_warp, &s_ell);
     }
 
     // 2. switches: outright rejects, the others' targets into the bitmap
