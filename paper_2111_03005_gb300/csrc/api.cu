@@ -124,7 +124,7 @@ uint64_t filter_bits(uint64_t M) {
 
 // Offsets of the pieces of a pool's single device allocation.
 struct Layout {
-  size_t chains, chain_acc, chain_ell, es_jobs, es_job_of, tfilter, owner_slot, owner_switch, owner_bucket, owner_part, cpos, cedge, prec, pcount, poff, pblk,
+  size_t chains, chain_acc, chain_ell, es_jobs, es_job_of, res_jobs, tfilter, owner_slot, owner_switch, owner_bucket, owner_part, cpos, cedge, prec, pcount, poff, pblk,
       bnd, word, sw, status, list0, list1, ptup, otup, stup, tcount, ocount, ooff, oblk, ocursor, dep,
       E, ctl, st, scratch, total;
 };
@@ -142,6 +142,7 @@ Layout pool_layout(const Capacity &c, uint64_t M, uint64_t C) {
   l.chain_ell = take(4 * C);
   l.es_job_of = take(4 * C);
   l.es_jobs = take(sizeof(EsJob) * C);  // (behind es_job_of: one copy brings both)
+  l.res_jobs = take(4 * C);  // kept between calls, so in no other mode's words
   l.owner_slot = take(4 * c.slots);
   l.owner_switch = take(4 * c.switches);
   l.owner_bucket = take(4 * c.buckets);
@@ -317,7 +318,7 @@ struct gesmc_pool_ctx {
   bool fused_graph_refused = false;
   // resident rounds (GESMC_ROUND_RESIDENT): one CTA per chain, the list in
   // shared memory for all rounds of a call; the chain list for the kernel
-  // (in es_job_of) is rebuilt when the chains change (res_version)
+  // (in res_jobs) is rebuilt when the chains change (res_version)
   bool resident = false;
   uint64_t res_version = 0;
   uint32_t res_count[kResidentClasses] = {}, res_max_m[kResidentClasses] = {};  // chains and largest m per class
@@ -766,7 +767,7 @@ int pool_run(gesmc_pool_t p, uint64_t rounds) {
         jobs.insert(jobs.end(), by_class[k].begin(), by_class[k].end());
         p->res_count[k] = (uint32_t)by_class[k].size();
       }
-      if (!jobs.empty() && (cudaMemcpyAsync(at<uint32_t>(p->base, p->lay.es_job_of), jobs.data(), 4 * jobs.size(),
+      if (!jobs.empty() && (cudaMemcpyAsync(at<uint32_t>(p->base, p->lay.res_jobs), jobs.data(), 4 * jobs.size(),
                                             cudaMemcpyHostToDevice, s) != cudaSuccess ||
                             cudaStreamSynchronize(s) != cudaSuccess)) {
         cudaGetLastError();
@@ -800,7 +801,7 @@ int pool_run(gesmc_pool_t p, uint64_t rounds) {
       bool ok = presort || cudaMemsetAsync(scratch, 0, 4ull * (r + kWaveHist), s) == cudaSuccess;
       uint16_t *pbuf = presort ? reinterpret_cast<uint16_t *>(a.prec) : nullptr;
       uint32_t *ebuf = presort ? reinterpret_cast<uint32_t *>(pbuf + (uint64_t)r * njobs * pstride) : nullptr;
-      ok = ok && launch_round_resident(a, at<uint32_t>(p->base, p->lay.es_job_of), p->res_count, p->res_max_m, r,
+      ok = ok && launch_round_resident(a, at<uint32_t>(p->base, p->lay.res_jobs), p->res_count, p->res_max_m, r,
                                        scratch + kWaveHist, scratch, final, pbuf, ebuf, pstride, s,
                                        &launches) == cudaSuccess;
       nvtxRangePop();

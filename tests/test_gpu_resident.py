@@ -142,6 +142,32 @@ def test_resident_and_pares_on_one_chain():
         assert np.array_equal(c.edges(), want)
 
 
+def test_resident_and_pares_on_a_pool_of_every_class():
+    # the resident rounds' list of chains (by class, longest first) and ParES's
+    # (by group: nodes, bytes, edges) are two orders of the same chains; either
+    # is still right after the other has run.  Chains of every class, small ones
+    # first, a chain too short for a switch and a place left by a removed one
+    sizes = [(3000, 1000), (2, 1), (600, 2000), (40, 300), (300, 1024), (65536, 700), (4000, 9500), (1500, 3000),
+             (30000, 2048), (2400, 6000)]
+    graphs = [(inputs.random_simple_graph(n, m, seed=60 + t), n) for t, (n, m) in enumerate(sizes)]
+    gone = 3
+    with gesmc.Pool(max_edges=sum(len(e) for e, _ in graphs), max_chains=len(graphs) + 2) as pool:
+        ids = [pool.add(e, n=n, seed=30 + t) for t, (e, n) in enumerate(graphs)]
+        pool.remove(ids[gone])
+        pool.set_round_launch(RESIDENT)
+        pool.run(3).es_run(700).run(2).es_run(50).run(1)
+        outs = [None if t == gone else pool.edges(c) for t, c in enumerate(ids)]
+    for t, (e, n) in enumerate(graphs):
+        if t == gone:
+            continue
+        want, _ = oracle.run(e, seed=30 + t, rounds=3)
+        want, _ = oracle.es_run(want, seed=30 + t, switches=700)
+        want, _ = oracle.run(want, seed=30 + t, rounds=2, start_round=3)
+        want, _ = oracle.es_run(want, seed=30 + t, switches=50, start_switch=700)
+        want, _ = oracle.run(want, seed=30 + t, rounds=1, start_round=5)
+        assert np.array_equal(outs[t], want), (t, sizes[t])
+
+
 def test_resident_pool_matches_the_multi_kernel_pool():
     graphs = inputs.ensemble_graphs(64, seed=41, n_lo=20, n_hi=3000)
     graphs = [(e, n) for e, n in graphs if len(e) <= gesmc.RESIDENT_MAX_EDGES]
