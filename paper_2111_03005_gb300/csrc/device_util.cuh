@@ -131,6 +131,12 @@ __device__ __forceinline__ void mbar_arrive_expect(unsigned long long *bar, uint
                : "memory");
 }
 
+// A bulk copy accesses memory through another proxy than loads and stores do.
+// Where a kernel copies what its own threads have written, or over what they have
+// read, with no kernel's end in between, the writers run this before the barrier
+// that orders them and the thread that starts the copy after it.
+__device__ __forceinline__ void proxy_fence() { asm volatile("fence.proxy.async;" ::: "memory"); }
+
 __device__ __forceinline__ void bulk_copy_g2s(void *dst, const void *src, uint32_t bytes, unsigned long long *bar) {
   asm volatile(
       "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_addr(dst)),

@@ -793,6 +793,9 @@ __device__ __forceinline__ bool sort_bucket(const RoundArgs &a, uint32_t b, cons
   if (c == kNoChain) return true;
   const uint32_t cnt = min(a.pcount[b], kCap);
   if (tid == 0 && cnt) {
+    // the one-launch round: the records were appended by this launch's threads,
+    // and the CTA's bucket before this one was read where the copy goes
+    if constexpr (kMeet) proxy_fence();
     mbar_arrive_expect(sm.bar, cnt * (uint32_t)sizeof(uint4));
     bulk_copy_g2s(srec, a.prec + ((size_t)b << kLog2), cnt * (uint32_t)sizeof(uint4), sm.bar);
   }
@@ -1890,6 +1893,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_round_fused(RoundArgs a) {
       if (!grid_sync(ctl, target)) return;
     }
     permute_body(a);
+    proxy_fence();  // the buckets' records are copied by the TMA engine
     if (!grid_sync(ctl, target)) return;
     if (!a.fused_local_offsets) {
       if (blockIdx.x == 0) {  // bucket offsets: full offsets in poff, zero block offsets

@@ -87,6 +87,21 @@ def test_sources_are_free_of_x86_only_code():
                 assert "immintrin" not in src and "__builtin_ia32" not in src and "march=native" not in src
 
 
+def test_bulk_copies_of_what_the_same_kernel_wrote_are_fenced():
+    # the one-launch round's sort copies, through the async proxy, records that
+    # the same launch stored: a proxy fence by the writers before the grid
+    # barrier, and by the thread that starts the copy after it (no outcome
+    # shows a missing one reliably, so this reads the source)
+    src = re.sub(r"//[^\n]*", "", open(os.path.join(ROOT, "paper_2111_03005_gb300/csrc/round.cu")).read())
+    fused = src[src.index("k_round_fused(RoundArgs a) {"):]
+    stage = fused[fused.index("permute_body(a);"):]
+    assert "proxy_fence();" in stage[:stage.index("grid_sync(")]
+    sort = src[src.index("bool sort_bucket("):]
+    start = sort[:sort.index("bulk_copy_g2s(")]
+    assert re.search(r"if \(tid == 0 && cnt\) \{\s+if constexpr \(kMeet\) proxy_fence\(\);", start)
+    assert src.count("bulk_copy_g2s(") == 1  # the only copy there is
+
+
 def test_noalloc_binding_refuses_a_stream_of_another_device():
     # the allocation-free call runs on the edge list's device; a torch stream
     # that belongs to another device is refused before anything is launched
