@@ -1182,8 +1182,9 @@ __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(T)
   constexpr uint32_t B = T * kClusterCtas;  // the window
   constexpr int kDist = kClusterCtas;       // distances a thread looks at for the cut
   // per parity of the superstep: events (told so far, in CTA 0: asked for), the
-  // end they force, this CTA's tombstones, the cut
-  __shared__ uint32_t s_events[2], s_asked[2], s_end[2], s_mine[2], s_cut[2], s_tombs;
+  // end they force, this CTA's tombstones; and the cuts of three supersteps, the
+  // running one's, the next one's, and the one after that's, which is set up
+  __shared__ uint32_t s_events[2], s_asked[2], s_end[2], s_mine[2], s_cut[3], s_tombs;
   __shared__ unsigned long long s_key[2][kEvents], s_who[2][kEvents];
   EsJob &job = jobs[job_off + blockIdx.x / kClusterCtas];
   const uint32_t rank = cluster_rank(), tid = threadIdx.x, x = rank * T + tid;
@@ -1199,8 +1200,9 @@ __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(T)
   }
   if (tid < 2) {
     s_events[tid] = s_asked[tid] = s_mine[tid] = 0;
-    s_end[tid] = s_cut[tid] = B;
+    s_end[tid] = B;
   }
+  if (tid < 3) s_cut[tid] = B;
   if (tid == 0) s_tombs = job.tombs;
   uint2 cur;
   uint32_t d[kDist];
@@ -1227,8 +1229,9 @@ __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(T)
   find_cut(&s_cut[0]);
   cluster_sync();  // (every CTA's shared memory is set up)
   uint32_t stop = 0, steps = 0, met = 0;
+  uint32_t cut = 0, next_cut = 1, last_cut = 2;
   for (uint32_t par = 0;; par ^= 1u) {
-    const uint32_t n = min(min(B, nsw - s), s_cut[par]);
+    const uint32_t n = min(min(B, nsw - s), s_cut[cut]);
     const uint32_t i = cur.x, j = cur.y & 0x7FFFFFFFu, g = cur.y >> 31;
     uint4 r1 = make_uint4(0, 0, 0, 0), r2 = r1;
     if (x < n) {
@@ -1236,7 +1239,6 @@ __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(T)
       r2 = __ldcg(&E[j]);
     }
     load_window(s + n);
-    if (tid == 0) s_cut[par ^ 1] = B;
     const unsigned long long e1 = rec_edge(r1), e2 = rec_edge(r2);
     unsigned long long e3 = 0, e4 = 0;
     const uint32_t code = x < n ? tau_g(g, e1, e2, e3, e4) : kCodeLazy;
@@ -1317,7 +1319,7 @@ __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(T)
       else ++rej_exists;  // a shared node (the targets re-create the sources) or a present target
     }
     if (end < n) load_window(s + end);
-    find_cut(&s_cut[par ^ 1]);
+    find_cut(&s_cut[next_cut]);
     tombs = __reduce_add_sync(0xffffffffu, tombs);
     if ((tid & 31u) == 0 && tombs) {
       tomb_total += tombs;
@@ -1325,12 +1327,18 @@ __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(T)
     }
     if (tid == 0) {
       // the superstep before this one's tombstones to every CTA, and its words
-      // for the next one
+      // for the next one (here, since the barriers above order nothing but what
+      // was told)
       const uint32_t mine = s_mine[par ^ 1];
       if (mine) all_add(&s_tombs, mine);
       s_mine[par ^ 1] = s_events[par ^ 1] = s_asked[par ^ 1] = 0;
       s_end[par ^ 1] = B;
+      s_cut[last_cut] = B;
     }
+    const uint32_t freed = cut;
+    cut = next_cut;
+    next_cut = last_cut;
+    last_cut = freed;
     s += end;
     ++steps;
     met += events;

@@ -102,6 +102,20 @@ def test_bulk_copies_of_what_the_same_kernel_wrote_are_fenced():
     assert src.count("bulk_copy_g2s(") == 1  # the only copy there is
 
 
+def test_words_of_the_cluster_are_reset_before_its_full_barrier():
+    # two of the three barriers of a superstep on a cluster order only what a
+    # thread told the others: a word that the next superstep counts in is reset
+    # between the last of these and the barrier that orders everything
+    src = re.sub(r"//[^\n]*", "", open(os.path.join(ROOT, "paper_2111_03005_gb300/csrc/es.cu")).read())
+    body = src[src.index("k_es_run_cluster(EsJob *jobs"):]
+    loop = body[body.index("for (uint32_t par = 0;;"):]
+    loop = loop[:loop.index("if (s >= nsw) break;")]
+    last_told, full = loop.rindex("cluster_sync_told("), loop.rindex("cluster_sync();")
+    for word in ("s_cut", "s_end", "s_mine", "s_events", "s_asked"):
+        resets = [m.start() for m in re.finditer(word + r"\[[^]]*\] = ", loop)]
+        assert resets and all(last_told < at < full for at in resets), word
+
+
 def test_noalloc_binding_refuses_a_stream_of_another_device():
     # the allocation-free call runs on the edge list's device; a torch stream
     # that belongs to another device is refused before anything is launched
