@@ -296,7 +296,7 @@ struct gesmc_pool_ctx {
   int broken = 0;
   RoundArgs args;
   uint64_t args_version = 1;  // bumped whenever args change (invalidates the graph)
-  bool waves_known = false;   // some round has run
+  uint64_t unseen_switches = 0;  // of chains that joined since the separate kernels last ran a round
   uint32_t wave_kernels = 0;  // whole-GPU wave kernel pairs per round (grows with the wide waves seen)
   // captured rounds (a CUDA graph of kGraphRounds rounds), replayed on gstream
   bool use_graphs = true;
@@ -334,10 +334,9 @@ struct gesmc_pool_ctx {
 // pools whose arguments stay.
 constexpr uint32_t kGraphRounds = 4;
 constexpr uint64_t kGraphAfterRounds = 16;
-// Fewer switches hardly ever have a wide wave (more than 2048 of them), and in
-// fewer rounds the wait would cost more than it gives.
-constexpr uint64_t kLearnRounds = 4;
-constexpr uint32_t kLearnSwitches = 1u << 15;
+// Fewer switches of new chains hardly ever have a wide wave (more than 2048 of
+// them), and in fewer rounds the wait would cost more than it gives.
+constexpr uint64_t kLearnRounds = 4, kLearnSwitches = 1u << 15;
 
 struct gesmc_ctx {
   gesmc_pool_t pool = nullptr;
@@ -704,6 +703,7 @@ int pool_add_device(gesmc_pool_t p, unsigned long long *E, uint64_t m, uint64_t 
     return GESMC_E_CUDA;
   }
   p->chains[c] = hc;
+  p->unseen_switches += hc.shape.L;
   ++p->live_chains;
   if (m >= 2) ++p->working_chains;
   p->live_edges += m;
@@ -712,10 +712,11 @@ int pool_add_device(gesmc_pool_t p, unsigned long long *E, uint64_t m, uint64_t 
   return GESMC_OK;
 }
 
-// Waves after the first that many switches entered in the last round: run as
-// many on the whole GPU from now on.
+// Waves after the first that many switches entered in the last round, which the
+// separate kernels ran (the other launches do not count them): run as many on
+// the whole GPU from now on.
 void learn_waves(gesmc_pool_t p, const Counters &ctl) {
-  p->waves_known = true;
+  p->unseen_switches = 0;
   const uint32_t want = std::min<uint32_t>(ctl.wide, kMaxWaveKernels);
   if (want > p->wave_kernels) {
     p->wave_kernels = want;
@@ -731,6 +732,7 @@ int pool_run(gesmc_pool_t p, uint64_t rounds) {
   // (the device's error word is zero: a call that sets it breaks the pool)
   const size_t per_round = kNumStages + 1;
   const bool stage_events = p->profiling && !p->resident;  // resident rounds have no separate stages
+  const bool fused = !p->resident && p->fused_ctas && !p->profiling, separate = !p->resident && !fused;
   if (stage_events) {
     const size_t need = per_round * (size_t)rounds;
     while (p->events.size() < need) {
@@ -812,7 +814,7 @@ int pool_run(gesmc_pool_t p, uint64_t rounds) {
       }
       done += r;
     }
-  } else if (p->fused_ctas && !p->profiling) {
+  } else if (fused) {
     if (cudaMemsetAsync(&a.ctl->clean, 0, sizeof(uint32_t), s) != cudaSuccess) return GESMC_E_CUDA;
     // one cooperative launch per round, replayed from a captured graph when
     // the driver captures it (else launched directly)
@@ -890,11 +892,11 @@ int pool_run(gesmc_pool_t p, uint64_t rounds) {
         after = true;
       }
     };
-    // A pool that has not run yet does not know which of its rounds' waves are
-    // wide, and its first call would run them all on one CTA: ask after one
-    // round (a power law of 7.8e5 edges, 20 rounds: 2.90 -> 2.45 ms).
+    // Which waves of its rounds are wide is not known of chains that have not run
+    // yet, and a call would run such waves on one CTA: ask after one round (a power
+    // law of 7.8e5 edges, 20 rounds: 2.90 -> 2.45 ms).
     uint64_t done = 0;  // rounds launched so far
-    if (ok && side && !p->waves_known && rounds >= kLearnRounds && a.switch_hw >= kLearnSwitches) {
+    if (ok && side && rounds >= kLearnRounds && p->unseen_switches >= kLearnSwitches) {
       direct(0, 1);
       done = 1;
       Counters ctl;
@@ -978,7 +980,7 @@ int pool_run(gesmc_pool_t p, uint64_t rounds) {
   p->switches_run += rounds * sw;
   const int rc = map_device_errors(ctl.err);
   if (rc != GESMC_OK) p->broken = rc;
-  if (rc == GESMC_OK) learn_waves(p, ctl);
+  if (rc == GESMC_OK && separate && rounds > 0) learn_waves(p, ctl);
   return rc;
 }
 

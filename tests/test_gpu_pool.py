@@ -177,3 +177,38 @@ def test_one_chain_pool_holds_any_smaller_chain(max_edges):
             expect_es, _ = oracle.es_run(expect, seed=40 + t, switches=500)
             assert np.array_equal(pool.edges(c), expect_es), m
             pool.remove(c)
+
+
+@pytest.mark.parametrize("before", ["kernels", "no rounds", "resident", "one launch"])
+def test_wide_waves_of_a_chain_that_joins_later_are_learnt_in_its_first_call(before):
+    # a pool whose small chain has run, in whichever launch, gets a chain with
+    # hubs whose second and third waves more than 2048 switches enter: from the
+    # second round of its first call on they run as pairs of kernels
+    small, n = inputs.workload_gnp_small(seed=4)
+    big = inputs.pld_graph(40000, 2.01, 1, 4000, seed=23)
+    _, _, entering = oracle.run_rounds(big, seed=4, rounds=1)
+    pairs = sum(int(x) > 2048 for x in entering[0][2:])
+    assert pairs == 2 and len(big) >= 1 << 16
+    with gesmc.Pool(max_edges=len(small) + len(big), max_chains=2) as pool:
+        a = pool.add(small, n=n, seed=3)
+        done = 0
+        if before in ("resident", "one launch"):
+            pool.set_round_launch(gesmc.ROUND_RESIDENT if before == "resident" else 8)
+            pool.run(2)
+            pool.set_round_launch(0)
+            done = 2
+        count = lambda: pool.stats()["kernel_launches"]
+        start = count()
+        if before == "kernels":
+            pool.run(1)
+            done = 1
+        else:
+            pool.run(0)
+        b = pool.add(big, n=40000, seed=4)
+        base = count() - start if before == "kernels" else 14
+        start = count()
+        pool.run(5)
+        assert count() - start >= 5 * base + 4 * 2 * pairs
+        got = pool.edges(a), pool.edges(b)
+    assert np.array_equal(got[0], oracle.run(small, seed=3, rounds=done + 5)[0])
+    assert np.array_equal(got[1], oracle.run(big, seed=4, rounds=5)[0])
