@@ -293,6 +293,7 @@ struct gesmc_pool_ctx {
   uint64_t live_edges = 0;
   uint64_t pool_round = 0;  // rounds completed (host copy of the device counter)
   uint64_t rounds = 0, switches_run = 0, launches = 0;
+  uint64_t es_skipped = 0;  // ES-MC switches of chains with fewer than two edges
   int broken = 0;
   RoundArgs args;
   uint64_t args_version = 1;  // bumped whenever args change (invalidates the graph)
@@ -997,11 +998,16 @@ int pool_es_run(gesmc_pool_t p, uint64_t switches, uint32_t only) {
   cudaStream_t s = p->stream;
   const RoundArgs &a = p->args;
   std::vector<EsJob> jobs;
+  std::vector<uint32_t> short_chains;  // fewer than two edges: their switches are only counted, however many
   std::vector<uint32_t> job_of(p->max_chains, kNoChain);
   char *tup = reinterpret_cast<char *>(a.ptup);
   for (uint32_t c = 0; c < p->max_chains; ++c) {
     const HostChain &hc = p->chains[c];
     if (!hc.live || (only != kNoChain && c != only)) continue;
+    if (hc.shape.m < 2) {
+      short_chains.push_back(c);
+      continue;
+    }
     EsJob jb;
     std::memset(&jb, 0, sizeof(jb));
     jb.m = hc.d.m;
@@ -1009,37 +1015,45 @@ int pool_es_run(gesmc_pool_t p, uint64_t switches, uint32_t only) {
     jb.k0 = hc.es_next;
     jb.chain = c;
     jb.n = (uint32_t)std::min<uint64_t>(hc.n, 0xFFFFFFFFull);
-    if (jb.m >= 2) {
-      // the list (position order, 16 bytes per edge) in the chain's tuple
-      // storage (at least 32 bytes per edge), the edge set in its permutation records (at least
-      // 32 bytes per edge: 2^h >= 2m slots)
-      char *base = tup + 16ull * hc.d.tuple_base;
-      const uint64_t bytes = 16ull * hc.d.capt << hc.d.P;
-      if (16ull * jb.m > bytes) return GESMC_E_INTERNAL;
-      char *hbase = reinterpret_cast<char *>(a.prec) + (16ull << p->cap.bucket_log2) * hc.d.bucket_base;
-      const uint64_t hbytes = (16ull << p->cap.bucket_log2) * hc.shape.nb;
-      uint32_t hlog2 = 0;
-      while ((16ull << hlog2) <= hbytes && hlog2 < 31) ++hlog2;  // largest 2^h with 8 * 2^h <= room
-      if ((1ull << hlog2) < 2ull * jb.m) return GESMC_E_INTERNAL;
-      jb.E = reinterpret_cast<uint4 *>(base);
-      // (a small chain has its set in shared memory)
-      jb.H = es_group(jb.m, hc.n) >= 4 ? nullptr : reinterpret_cast<unsigned long long *>(hbase);
-      jb.hlog2 = hlog2;
-    }
+    // the list (position order, 16 bytes per edge) in the chain's tuple storage
+    // (at least 32 bytes per edge), the edge set in its permutation records (at
+    // least 32 bytes per edge: 2^h >= 2m slots)
+    char *base = tup + 16ull * hc.d.tuple_base;
+    const uint64_t bytes = 16ull * hc.d.capt << hc.d.P;
+    if (16ull * jb.m > bytes) return GESMC_E_INTERNAL;
+    char *hbase = reinterpret_cast<char *>(a.prec) + (16ull << p->cap.bucket_log2) * hc.d.bucket_base;
+    const uint64_t hbytes = (16ull << p->cap.bucket_log2) * hc.shape.nb;
+    uint32_t hlog2 = 0;
+    while ((16ull << hlog2) <= hbytes && hlog2 < 31) ++hlog2;  // largest 2^h with 8 * 2^h <= room
+    if ((1ull << hlog2) < 2ull * jb.m) return GESMC_E_INTERNAL;
+    jb.E = reinterpret_cast<uint4 *>(base);
+    // (a small chain has its set in shared memory)
+    jb.H = es_group(jb.m, hc.n) >= 4 ? nullptr : reinterpret_cast<unsigned long long *>(hbase);
+    jb.hlog2 = hlog2;
     jobs.push_back(jb);
   }
-  if (jobs.empty()) return GESMC_OK;
-  // chains by group, largest windows first (each group keeps chain order); chains with m < 2 have no list to move (their switches are only
-  // counted)
+  auto count_short = [&] {
+    for (const uint32_t c : short_chains) p->chains[c].es_next += switches;
+    p->es_skipped += switches * short_chains.size();
+    p->switches_run += switches * short_chains.size();
+  };
+  if (jobs.empty()) {
+    if (cudaStreamSynchronize(s) != cudaSuccess) {
+      cudaGetLastError();
+      p->broken = GESMC_E_CUDA;
+      return GESMC_E_CUDA;
+    }
+    count_short();
+    return GESMC_OK;
+  }
+  // chains by group, largest windows first (each group keeps chain order)
   auto group_of = [p](const EsJob &x) { return es_group(x.m, p->chains[x.chain].n); };
   std::stable_sort(jobs.begin(), jobs.end(),
                    [&](const EsJob &x, const EsJob &y) { return group_of(x) < group_of(y); });
-  uint32_t group[kEsGroups] = {}, smem_of[kEsGroups] = {}, rows = 0;
+  uint32_t group[kEsGroups] = {}, smem_of[kEsGroups] = {};
   for (uint32_t t = 0; t < jobs.size(); ++t) {
-    if (jobs[t].m >= 2) {
-      job_of[jobs[t].chain] = t;
-      jobs[t].row = rows++;
-    }
+    job_of[jobs[t].chain] = t;
+    jobs[t].row = t;
     const uint32_t w = group_of(jobs[t]);
     ++group[w];
     if (w >= 4) smem_of[w] = std::max(smem_of[w], es_smem_bytes(jobs[t].m, jobs[t].n));
@@ -1064,11 +1078,11 @@ int pool_es_run(gesmc_pool_t p, uint64_t switches, uint32_t only) {
   // of each chain, and three for every edge of the largest.
   uint2 *samples = reinterpret_cast<uint2 *>(a.otup);
   const uint64_t room = p->lay.tcount - p->lay.otup;
-  const uint64_t batch = std::min<uint64_t>(1u << 30, rows ? room / (10ull * rows) : switches);
+  const uint64_t batch = std::min<uint64_t>(1u << 30, room / (10ull * nj));
   uint32_t *nstop = &a.ctl->es_stopped;
   for (uint64_t off = 0; ok && off < switches; off += batch) {
     const uint32_t n = (uint32_t)std::min<uint64_t>(batch, switches - off);
-    uint16_t *dists = reinterpret_cast<uint16_t *>(samples + (uint64_t)rows * n);
+    uint16_t *dists = reinterpret_cast<uint16_t *>(samples + (uint64_t)nj * n);
     uint32_t run_launches = 0;
     ok &= launch_es_sample(djobs, group, off, n, samples, dists, s, &run_launches) == cudaSuccess;
     p->launches += run_launches;
@@ -1106,6 +1120,7 @@ int pool_es_run(gesmc_pool_t p, uint64_t switches, uint32_t only) {
   }
   for (uint32_t t = 0; t < nj; ++t) p->chains[jobs[t].chain].es_next += switches;
   p->switches_run += switches * nj;
+  count_short();
   const int rc = map_device_errors(host_err);
   if (rc != GESMC_OK) p->broken = rc;
   return rc;
@@ -1391,7 +1406,7 @@ int gesmc_pool_stats(gesmc_pool_t p, gesmc_stats_t *out) {
   std::memset(out, 0, sizeof(*out));
   out->rounds = p->rounds;
   out->switches = p->switches_run;
-  out->lazy = st.lazy;
+  out->lazy = st.lazy + p->es_skipped;
   out->accepted = st.accepted;
   out->rejected_loop = st.rej_loop;
   out->rejected_exists = st.rej_exists;
@@ -1419,6 +1434,7 @@ int gesmc_pool_reset_stats(gesmc_pool_t p) {
   }
   p->rounds = 0;
   p->switches_run = 0;
+  p->es_skipped = 0;
   p->launches = 0;
   for (double &x : p->stage_ms) x = 0.0;
   p->stage_rounds = 0;

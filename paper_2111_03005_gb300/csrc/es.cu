@@ -275,7 +275,6 @@ __global__ void __launch_bounds__(C) k_es_sample(EsJob *jobs, uint32_t job_off, 
   __shared__ __align__(4) uint16_t head[1 << kLog2];
   EsJob &jb = jobs[job_off + blockIdx.y];
   const uint32_t x = threadIdx.x, beg = blockIdx.x * C;
-  if (jb.m < 2) return;
   if (blockIdx.x == 0 && x == 0) {  // the batch starts
     jb.done = 0;
     jb.stopped = 0;
@@ -360,10 +359,6 @@ __device__ __forceinline__ void es_run_body(EsJob *jobs, uint32_t job_off, uint3
   const uint32_t x = threadIdx.x;
   const uint32_t m = job.m;
   uint32_t acc = 0, rej_loop = 0, rej_exists = 0;
-  if (m < 2) {  // no pair of positions: every requested switch is skipped
-    if (x == 0) atomicAdd(&stats->lazy, (unsigned long long)nsw);
-    return;
-  }
   uint4 *const E = job.E;
   unsigned long long *const H = job.H;
   const uint2 *const samp = samples + (size_t)job.row * nsw;
@@ -1400,7 +1395,6 @@ uint32_t es_group(uint32_t m, uint64_t n) {
   if (m >= kEsBigChain) return 0;
   if (m >= kEsMidChain) return 1;
   if (m >= kEsSmallChain) return 2;
-  if (m < 2) return 3;
   for (uint32_t v = 0; v < 3; ++v)
     if (n <= 65536 && bits_bytes(m, n) <= kEsBitBytes[v]) return 7 - v;
   return m <= kEsSmallestEdges && n <= 65536 ? 4 : 3;

@@ -317,7 +317,7 @@ cudaError_t launch_list_check(const unsigned long long *E, uint32_t m, unsigned 
 cudaError_t launch_duplicate_check(const unsigned long long *E, uint32_t m, unsigned long long *set,
                                    unsigned long long cap, uint32_t *flags, cudaStream_t s, int num_sms);
 
-// ParES (Algorithm 2) for one chain: its list in position order (in the
+// ParES (Algorithm 2) for one chain of two edges or more: its list in position order (in the
 // chain's tuple storage, {edge lo, edge hi, its slot in the edge set, 0} per
 // position) and its edge set (open addressing, 2^hlog2 slots, in the chain's
 // permutation records), neither of which a round uses between rounds; ES-MC
@@ -346,8 +346,7 @@ uint32_t es_smem_bytes(uint32_t m, uint32_t n);  // of a job of the last four gr
 // Edge sets of all jobs (or only of the stopped ones) rebuilt from their lists.
 cudaError_t launch_es_set(EsJob *jobs, uint32_t njobs, uint32_t *err, cudaStream_t s, int num_sms,
                           bool only_stopped);
-// A batch: the switches off .. off + n - 1 of the call, for every job with
-// m >= 2, sampled into row job.row (n entries each) of samples and dists.
+// A batch: the switches off .. off + n - 1 of the call, for every job, sampled into row job.row (n entries each) of samples and dists.
 // group as for launch_es_run.
 cudaError_t launch_es_sample(EsJob *jobs, const uint32_t (&group)[kEsGroups], unsigned long long off, uint32_t n,
                              uint2 *samples, uint16_t *dists, cudaStream_t s, uint32_t *launches);

@@ -70,6 +70,32 @@ def test_empty_and_single_edge():
         assert st["lazy"] == 15
 
 
+def test_any_number_of_switches_of_a_chain_without_a_pair_of_edges():
+    # they are only counted: no work per switch, alone or beside other chains
+    many = 1 << 60
+    with gesmc.Chain(np.array([1], np.uint64), n=4) as c:   # the edge {0, 1}
+        launches = c.stats()["kernel_launches"]
+        c.es_run(many, 3)
+        c.es_run(5, 3)
+        st = c.stats()
+        assert st["lazy"] == st["switches"] == many + 5 and st["kernel_launches"] == launches
+        assert np.array_equal(c.edges(), np.array([1], np.uint64))
+        c.reset_stats()
+        assert c.stats()["lazy"] == 0
+        c.run(2, 3)
+        assert c.verify() == gesmc.GESMC_OK
+    edges = inputs.random_simple_graph(50, 200, seed=6)
+    with gesmc.Pool(max_edges=300, max_chains=4) as pool:
+        one, chain, none = pool.add([1], n=4, seed=1), pool.add(edges, n=50, seed=2), pool.add([], n=4, seed=3)
+        pool.es_run(3000).es_run(40)
+        assert [pool.chain_info(c)["es_switches"] for c in (one, chain, none)] == [3040] * 3
+        st = pool.stats()
+        want, want_st = oracle.es_run(edges, seed=2, switches=3040)
+        assert st["lazy"] == 2 * 3040 and st["switches"] == 3 * 3040 and st["accepted"] == want_st["accepted"]
+        assert np.array_equal(pool.edges(chain), want)
+        assert np.array_equal(pool.edges(one), np.array([1], np.uint64))
+
+
 def test_mixed_with_global_switches_and_reseed():
     edges, n = inputs.workload_gnp_small(seed=2)
     expect = oracle.validate(edges, n)[1]
