@@ -142,7 +142,6 @@ Layout pool_layout(const Capacity &c, uint64_t M, uint64_t C) {
   l.chain_ell = take(4 * C);
   l.es_job_of = take(4 * C);
   l.es_jobs = take(sizeof(EsJob) * C);  // (behind es_job_of: one copy brings both)
-  l.res_jobs = take(4 * C);  // kept between calls, so in no other mode's words
   l.owner_slot = take(4 * c.slots);
   l.owner_switch = take(4 * c.switches);
   l.owner_bucket = take(4 * c.buckets);
@@ -176,6 +175,7 @@ Layout pool_layout(const Capacity &c, uint64_t M, uint64_t C) {
   l.ctl = take(sizeof(Counters));
   l.st = take(sizeof(StatsDev));
   l.scratch = take(64);
+  l.res_jobs = take(4 * C);  // kept between calls, so in no other mode's words
   l.total = o;
   return l;
 }
