@@ -1066,12 +1066,11 @@ int pool_es_run(gesmc_pool_t p, uint64_t switches, uint32_t only) {
   std::memcpy(both.data(), job_of.data(), 4ull * p->max_chains);
   std::memcpy(both.data() + (p->lay.es_jobs - p->lay.es_job_of), jobs.data(), sizeof(EsJob) * nj);
   bool ok = cudaMemcpyAsync(djob_of, both.data(), both.size(), cudaMemcpyHostToDevice, s) == cudaSuccess;
-  ok &= launch_es_store(a, djobs, djob_of, s, p->num_sms) == cudaSuccess;
   // (no sets to build if every chain has its own in shared memory)
   const uint32_t nset = group[0] + group[1] + group[2] + group[3];
-  const uint64_t set_launches = 2ull * ((nset + 65534) / 65535);
-  ok &= launch_es_set(djobs, nset, err, s, p->num_sms, false) == cudaSuccess;
-  p->launches += set_launches + 2;
+  ok &= launch_es_set(djobs, nset, err, s, p->num_sms, false, &p->launches) == cudaSuccess;
+  ok &= launch_es_store(a, djobs, djob_of, err, s, p->num_sms) == cudaSuccess;
+  p->launches += 2;
   // The switches run in batches, sampled beforehand into the overflow-tuple
   // array (free between rounds): 8 bytes and a 16-bit distance per switch and
   // chain.  It has 32 bytes for every edge, so a batch has at least 6 switches
@@ -1105,8 +1104,7 @@ int pool_es_run(gesmc_pool_t p, uint64_t switches, uint32_t only) {
       ok &= cudaStreamSynchronize(s) == cudaSuccess;
       if (e != 0) off = switches;  // an error ends the call
       if (!ok || stopped == 0 || e != 0) break;
-      ok &= launch_es_set(djobs, nset, err, s, p->num_sms, true) == cudaSuccess;
-      p->launches += set_launches;
+      ok &= launch_es_set(djobs, nset, err, s, p->num_sms, true, &p->launches) == cudaSuccess;
     }
   }
   ok &= launch_es_load(a, djobs, djob_of, s, p->num_sms) == cudaSuccess;

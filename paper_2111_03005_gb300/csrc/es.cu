@@ -34,12 +34,12 @@
 // the CTA for the smaller windows, on the whole GPU between launches for the
 // largest.
 #include "device_util.cuh"
+#include "es_set.cuh"
 #include "gesmc_internal.cuh"
 
 namespace gesmc {
 namespace {
 
-constexpr uint32_t kNil = 0xFFFFFFFFu;
 constexpr unsigned long long kNoKey = 0;  // {0, 0}: not an edge, empty or tombstone
 constexpr uint8_t kEsUndecided = 0, kEsLegal = 1, kEsIllegal = 2;
 // Window sizes by chain size (supersteps hold about 0.63 sqrt(m) switches:
@@ -53,29 +53,7 @@ constexpr uint32_t kEsBigChain = 1u << 19;
 constexpr uint32_t kEsMidChain = 1u << 16;
 constexpr uint32_t kEsSmallChain = 1u << 13;
 
-__device__ __forceinline__ uint32_t hash32(unsigned long long key) { return (uint32_t)mix64(key); }
-
-// ---------------------------------------------------------------- the edge set H
-// Open addressing with linear probing from h & mask (h = hash32(key)).
-// Insert a key that is not in the set into the first empty or tombstone
-// slot of its probe sequence from slot s on.  Returns the slot (with
-// *tomb = 1 if it held a tombstone), or kNil if the table is full.
-__device__ __forceinline__ uint32_t hset_insert(unsigned long long *H, uint32_t mask, unsigned long long key,
-                                                uint32_t s, uint32_t *tomb) {
-  for (uint32_t n = 0; n <= mask; ++n) {
-    const unsigned long long cur = __ldcg(&H[s]);
-    if (cur == kEmptyKey || cur == kTombKey) {
-      if (atomicCAS(&H[s], cur, key) == cur) {
-        *tomb = cur == kTombKey ? 1u : 0u;
-        return s;
-      }
-      continue;  // taken meanwhile: look at the same slot again
-    }
-    s = (s + 1) & mask;
-  }
-  return kNil;
-}
-
+// ---------------------------------------------------------------- the list and the edge set H
 // Loads of a chain's list and set by its CTA.  kL1: through the SM's L1, for
 // the small windows, whose chains' lists and sets fit there (one CTA writes
 // them while the kernel runs, and its barriers order its own accesses); else
@@ -244,10 +222,10 @@ __global__ void k_es_clear(EsJob *jobs, uint32_t job_off, bool only_stopped) {
   if (blockIdx.x == 0 && threadIdx.x == 0) jobs[job_off + blockIdx.y].tombs = 0;
 }
 
-// H <- the entries of E, each entry's slot into the list.
-__global__ void k_es_fill(const EsJob *jobs, uint32_t job_off, uint32_t *err, bool only_stopped) {
+// H <- the entries of E, each entry's slot into the list, for the stopped jobs.
+__global__ void k_es_fill(const EsJob *jobs, uint32_t job_off, uint32_t *err) {
   const EsJob jb = jobs[job_off + blockIdx.y];
-  if (!jb.H || (only_stopped && jb.stopped != 1)) return;
+  if (!jb.H || jb.stopped != 1) return;
   const uint32_t mask = (uint32_t)((1ull << jb.hlog2) - 1);
   for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < jb.m; s += gridDim.x * blockDim.x) {
     const unsigned long long e = rec_edge(jb.E[s]);
@@ -1420,14 +1398,15 @@ cudaError_t prepare_es_kernels() {
                               (int)EsShape<256>::kBytes);
 }
 
-cudaError_t launch_es_set(EsJob *jobs, uint32_t njobs, uint32_t *err, cudaStream_t s, int num_sms,
-                          bool only_stopped) {
+cudaError_t launch_es_set(EsJob *jobs, uint32_t njobs, uint32_t *err, cudaStream_t s, int num_sms, bool rebuild,
+                          uint64_t *launches) {
   for (uint32_t off = 0; off < njobs; off += 65535u) {
     const uint32_t nj = njobs - off < 65535u ? njobs - off : 65535u;
     const uint32_t gx = (uint32_t)((num_sms * 8 + nj - 1) / nj);
     const dim3 grid(gx < 1 ? 1 : gx, nj);
-    k_es_clear<<<grid, 256, 0, s>>>(jobs, off, only_stopped);
-    k_es_fill<<<grid, 256, 0, s>>>(jobs, off, err, only_stopped);
+    k_es_clear<<<grid, 256, 0, s>>>(jobs, off, rebuild);
+    if (rebuild) k_es_fill<<<grid, 256, 0, s>>>(jobs, off, err);
+    *launches += rebuild ? 2 : 1;
   }
   return cudaGetLastError();
 }

@@ -343,9 +343,10 @@ cudaError_t prepare_es_kernels();
 constexpr uint32_t kEsGroups = 8;
 uint32_t es_group(uint32_t m, uint64_t n);
 uint32_t es_smem_bytes(uint32_t m, uint32_t n);  // of a job of the last four groups
-// Edge sets of all jobs (or only of the stopped ones) rebuilt from their lists.
-cudaError_t launch_es_set(EsJob *jobs, uint32_t njobs, uint32_t *err, cudaStream_t s, int num_sms,
-                          bool only_stopped);
+// Edge sets of all jobs emptied (launch_es_store fills them), or, rebuild, those
+// of the stopped jobs filled again from their lists.  Adds to *launches.
+cudaError_t launch_es_set(EsJob *jobs, uint32_t njobs, uint32_t *err, cudaStream_t s, int num_sms, bool rebuild,
+                          uint64_t *launches);
 // A batch: the switches off .. off + n - 1 of the call, for every job, sampled into row job.row (n entries each) of samples and dists.
 // group as for launch_es_run.
 cudaError_t launch_es_sample(EsJob *jobs, const uint32_t (&group)[kEsGroups], unsigned long long off, uint32_t n,
@@ -363,10 +364,10 @@ cudaError_t launch_es_run(EsJob *jobs, const uint32_t (&group)[kEsGroups], const
                           uint32_t *nstop, bool alone, cudaStream_t s, cudaStream_t s2, cudaEvent_t fork,
                           cudaEvent_t join, uint32_t *launches);
 // Lists of the chains with a job (job_of[chain] != kNoChain) out of their
-// slots into the jobs' position-order lists, and back (slots in position
-// order, nothing pending).
-cudaError_t launch_es_store(const RoundArgs &a, const EsJob *jobs, const uint32_t *job_of, cudaStream_t s,
-                            int num_sms);
+// slots into the jobs' position-order lists and their (empty) edge sets, and
+// back (slots in position order, nothing pending).
+cudaError_t launch_es_store(const RoundArgs &a, const EsJob *jobs, const uint32_t *job_of, uint32_t *err,
+                            cudaStream_t s, int num_sms);
 cudaError_t launch_es_load(const RoundArgs &a, const EsJob *jobs, const uint32_t *job_of, cudaStream_t s,
                            int num_sms);
 

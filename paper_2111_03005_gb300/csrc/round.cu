@@ -38,6 +38,7 @@
 #include <algorithm>
 
 #include "device_util.cuh"
+#include "es_set.cuh"
 #include "gesmc_internal.cuh"
 
 namespace gesmc {
@@ -2142,9 +2143,12 @@ __global__ void __launch_bounds__(256) k_store_out(const uint4 *rec, uint32_t m,
 }
 
 // ParES: the lists of the chains with a job, by position, with the last
-// round's legal switches applied; and back into their slots (slot s holds
-// position s, nothing pending).
-__global__ void k_es_store(RoundArgs a, const EsJob *jobs, const uint32_t *job_of) {
+// round's legal switches applied, and their edge sets; and back into their slots
+// (slot s holds position s, nothing pending).  An edge goes into the set on the
+// way to the list, whose entry then has its slot at once: with a pass of its own
+// that read and wrote the list again, a call of one switch took 1126 us on 1.6e7
+// edges and 58 us on 9,000, now 1085 and 54.
+__global__ void k_es_store(RoundArgs a, const EsJob *jobs, const uint32_t *job_of, uint32_t *err) {
   const unsigned long long R = a.ctl->pool_round;
   const uint32_t npair = (a.slot_hw + 1) >> 1;
   for (uint32_t x = blockIdx.x * blockDim.x + threadIdx.x; x < npair; x += gridDim.x * blockDim.x) {
@@ -2152,9 +2156,17 @@ __global__ void k_es_store(RoundArgs a, const EsJob *jobs, const uint32_t *job_o
     const uint32_t c = a.owner_slot[s0];
     if (c == kNoChain || job_of[c] == kNoChain) continue;
     const ChainDesc ch = a.chains[c];
-    uint4 *E = jobs[job_of[c]].E;
-    auto put = [E](uint32_t pos, unsigned long long e) {
-      E[pos] = make_uint4((uint32_t)e, (uint32_t)(e >> 32), 0u, 0u);
+    const EsJob &jb = jobs[job_of[c]];
+    uint4 *const E = jb.E;
+    unsigned long long *const H = jb.H;
+    const uint32_t mask = (uint32_t)((1ull << jb.hlog2) - 1);
+    auto put = [=](uint32_t pos, unsigned long long e) {
+      uint32_t at = 0, tomb;
+      if (H && (at = hset_insert(H, mask, e, hash32(e) & mask, &tomb)) == kNil) {
+        atomicOr(err, kErrTableFull);
+        at = 0;
+      }
+      E[pos] = make_uint4((uint32_t)e, (uint32_t)(e >> 32), at, 0u);
     };
     const uint32_t ls = s0 - ch.slot_base;
     if (ls + 1 < ch.m) {
@@ -2438,10 +2450,10 @@ cudaError_t launch_store_chain(const RoundArgs &a, const ChainDesc &ch, uint64_t
   return cudaGetLastError();
 }
 
-cudaError_t launch_es_store(const RoundArgs &a, const EsJob *jobs, const uint32_t *job_of, cudaStream_t s,
-                            int num_sms) {
+cudaError_t launch_es_store(const RoundArgs &a, const EsJob *jobs, const uint32_t *job_of, uint32_t *err,
+                            cudaStream_t s, int num_sms) {
   if (a.slot_hw == 0) return cudaSuccess;
-  k_es_store<<<grid_for((a.slot_hw + 1) / 2, 256, num_sms, 8), 256, 0, s>>>(a, jobs, job_of);
+  k_es_store<<<grid_for((a.slot_hw + 1) / 2, 256, num_sms, 8), 256, 0, s>>>(a, jobs, job_of, err);
   return cudaGetLastError();
 }
 

@@ -96,6 +96,24 @@ def test_any_number_of_switches_of_a_chain_without_a_pair_of_edges():
         assert np.array_equal(pool.edges(one), np.array([1], np.uint64))
 
 
+@pytest.mark.parametrize("m, n, launches", [(9001, 5000, 5), (900, 400, 4), (900, 60_000, 4), (900, 70_000, 5)])
+def test_a_call_of_one_switch_passes_over_the_list_twice(m, n, launches):
+    # out of the slots, with the edge set on the way, and back; a set in memory
+    # is emptied first, one in shared memory needs no launch
+    edges = inputs.random_simple_graph(n, m, seed=m + n)
+    with gesmc.Chain(edges, n=n) as c:
+        before = c.stats()["kernel_launches"]
+        c.es_run(1, 9)
+        assert c.stats()["kernel_launches"] - before == launches
+        c.run(1, 9)
+        c.es_run(1, 9)
+        got = c.edges()
+    want, _ = oracle.es_run(edges, seed=9, switches=1)
+    want, _ = oracle.run(want, seed=9, rounds=1)
+    want, _ = oracle.es_run(want, seed=9, switches=1, start_switch=1)
+    assert np.array_equal(got, want)
+
+
 def test_mixed_with_global_switches_and_reseed():
     edges, n = inputs.workload_gnp_small(seed=2)
     expect = oracle.validate(edges, n)[1]
