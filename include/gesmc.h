@@ -183,7 +183,8 @@ int gesmc_reset_stats(gesmc_t h);
  * gesmc_reset_stats) of the first n_stages stages into ms and the number of
  * profiled rounds into *rounds.  Stage i is named by gesmc_stage_name(i);
  * GESMC_NUM_STAGES stages exist, in launch order, each one kernel except
- * "overflow" (three kernels that return at once when nothing overflowed)
+ * "clear" (a second kernel where some chain has GESMC_CHAIN_EXACT_ELL set),
+ * "scan_perm" (two), "overflow" (four kernels that return at once when nothing overflowed)
  * and "waves" (a pair of kernels per wave after the first that more than
  * 2048 undecided switches enter, run on the whole GPU; as many pairs as the
  * handle's rounds have needed such waves so far, at most 8, none while no

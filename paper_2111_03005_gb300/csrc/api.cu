@@ -308,7 +308,7 @@ struct gesmc_pool_ctx {
   uint32_t graph_launches = 0;
   uint64_t warm_version = 0, warm_rounds = 0;  // rounds launched with the current arguments
   // one-launch rounds (k_round_fused) with this many CTAs; 0: the kernels of
-  // a round one after another (replayed from the captured graph)
+  // a round one after another
   uint32_t fused_ctas = 0;
   uint32_t fused_max = 0;  // CTAs of the one-launch round the device holds at once
   // the one-launch round captured in a graph of its own (replayed per round),

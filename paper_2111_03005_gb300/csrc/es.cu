@@ -322,8 +322,9 @@ __global__ void __launch_bounds__(C) k_es_sample(EsJob *jobs, uint32_t job_off, 
 // every window, key tables for every superstep and separate searches to find,
 // erase and insert, 2^19 switches of a chain of 1e6 edges took 21.4 ms, then 7.2
 // (26 -> 8.9 us a superstep; on a cluster 5.1, see below); 512 chains of 65 to
-// 118,000 edges with 2^14 switches each 22.0 ms, now 8.9 (most are single warps:
-// 2270 -> 430 instructions a superstep).
+// 118,000 edges with 2^14 switches each 22.0 ms, then 8.9 (most were single warps:
+// 2270 -> 430 instructions a superstep), now 5.4: the chains of few nodes or edges
+// have left this kernel for shared memory, see below.
 template <int B, bool kStopToRebuild>
 __device__ __forceinline__ void es_run_body(EsJob *jobs, uint32_t job_off, uint32_t nsw, const uint2 *samples,
                                             const uint16_t *dists, StatsDev *stats, unsigned long long *chain_acc,

@@ -119,11 +119,12 @@ inline uint32_t bucket_log2(unsigned long long max_edges) {
 }
 
 // Tuple partitions: a chain's tuples go to 2^P partitions by the top P bits
-// of the hash of the edge id (about 2^tuple_log2 tuples each, room for
-// twice that); one CTA groups a partition by edge id, the few ids that may have
-// a dependency in a shared-memory table of 2^group_log2 slots of 20 bytes.
+// of the hash of the edge id: between half of and 2^tuple_log2 tuples each on
+// average, if every source had one, with room for that average and 64 more; one CTA
+// groups a partition by edge id, the few ids that may have a dependency in a
+// shared-memory table of 2^group_log2 slots of 20 bytes.
 constexpr int kDefaultTupleLog2 = 10;
-constexpr int kDefaultGroupLog2 = 11;  // as many slots as a partition of the fast path has tuples
+constexpr int kDefaultGroupLog2 = 11;  // the fast path takes partitions of up to 5/4 as many tuples
 constexpr int kMaxGroupLog2 = 13;
 constexpr int kGroupThreads = 512;
 constexpr int kGroupMin = 3;  // CTAs per SM

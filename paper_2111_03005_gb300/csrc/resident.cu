@@ -346,9 +346,10 @@ __device__ __forceinline__ uint32_t sort_round(const ChainDesc &ch, unsigned lon
 
 // The same as a call of its own, for the CTA of 1024 threads: inlined, the twelve
 // keys of a thread and what the round keeps besides left it 324 bytes of
-// spills, which go to L2 (shared memory takes nearly all of L1).  20 rounds of
-// 200 chains of 8,011 edges: 1299 -> 1275 us, of 9,641 (dense) 2320 -> 2114.
-// The smaller CTAs, eight keys a thread, are 3 to 4% slower so.
+// spills, which go to L2 (shared memory takes nearly all of L1); so, the kernel
+// has 252 and the call 116.  20 rounds of 200 chains of 8,011 edges: 1299 -> 1275
+// us, of 9,641 (dense) 2320 -> 2114.  The smaller CTAs, eight keys a thread and
+// 264 bytes of spills, are 3 to 4% slower so.
 template <int T>
 __device__ __noinline__ uint32_t sort_apart(const ChainDesc &ch, unsigned long long round, uint32_t m, uint32_t L,
                                             uint32_t nb_log2, uint32_t *skey, uint32_t *cnt, uint16_t *spos,
@@ -955,7 +956,7 @@ cudaError_t launch_round_resident(const RoundArgs &a, const uint32_t *jobs, cons
   j.round_waves = round_waves;
   j.last_pending = last_pending;
   j.final = final ? 1u : 0u;
-  // status words hold the wave in 14 bits; a round needs at most L + 1 <= 6145 waves
+  // status words hold the wave in 14 bits; a round needs at most L + 1 <= 5121 waves
   const uint32_t cap = a.max_waves ? a.max_waves : kDefaultWaveCap;
   j.wave_cap = cap < 16383u ? cap : 16383u;
   for (int perms = pbuf ? 1 : 0; perms >= 0; --perms) {

@@ -27,9 +27,9 @@
 //                    an undecided switch; edge ids with a dependency get an
 //                    entry {p, q} for the later waves
 //   k_wave1          per switch: legal, illegal or pending
-//   k_wave_register  waves 2, 3, ... over the pending switches on the whole
-//   k_wave_decide    GPU, one pair of kernels per wave
-//   k_tail           any remaining waves, on one CTA
+//   k_wave_register  waves that more than kSoloPending pending switches enter,
+//   k_wave_decide    on the whole GPU, one pair of kernels per wave
+//   k_tail           all other waves, on one CTA
 //
 // The waves are Jacobi steps: a switch decided in wave w only uses decisions
 // of waves < w (status words carry their wave), so the result and the wave
